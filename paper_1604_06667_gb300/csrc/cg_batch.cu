@@ -154,10 +154,6 @@ cg_status build_plan(cg_batch* b) {
     q.n = J.n_samples;
     q.off = samp_off.back();
     q.nside = g->nside;
-    q.lg = -1;
-    if ((g->nside & (g->nside - 1)) == 0)
-      for (q.lg = 0; (1LL << q.lg) < g->nside; ++q.lg) {
-      }
     q.key_base = key_base;
     q.ring_base = ring_base;
     q.ranges = t.ranges;
@@ -172,7 +168,7 @@ cg_status build_plan(cg_batch* b) {
     ring_base += 4 * ns + 1;
     samp_off.push_back(q.off + J.n_samples);
     key_blk.push_back(key_blk.back() + (J.n_samples + 255) / 256);
-    gth_blk.push_back(gth_blk.back() + (J.n_samples + 1 + 255) / 256);
+    gth_blk.push_back(gth_blk.back() + (J.n_samples + 255) / 256 + (4 * ns + 1 + 255) / 256);
     tile_off.push_back(tile_off.back() + t.n_tiles);
     if (tc) p->tc_jobs.push_back(j);
   }

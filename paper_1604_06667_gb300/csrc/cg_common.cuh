@@ -88,25 +88,6 @@ __device__ __forceinline__ int64_t ang2pix_ring_f64(int64_t ns, double lon_deg, 
   }
 }
 
-// Ring number (1 .. 4ns-1) of RING pixel p; integer arithmetic with an
-// FP32 square-root estimate corrected exactly.
-__device__ __forceinline__ int ring_of_pix(int64_t ns, int64_t p) {
-  const int64_t npix = 12 * ns * ns;
-  const int64_t ncap = 2 * ns * (ns - 1);
-  if (p < ncap) {
-    int64_t k = (int64_t)(0.5f * (1.0f + sqrtf(1.0f + 2.0f * (float)p)));
-    while (k > 1 && 2 * k * (k - 1) > p) --k;
-    while (2 * (k + 1) * k <= p) ++k;
-    return (int)k;
-  }
-  if (p < npix - ncap) return (int)(ns + (p - ncap) / (4 * ns));
-  const int64_t q = npix - 1 - p;
-  int64_t k = (int64_t)(0.5f * (1.0f + sqrtf(1.0f + 2.0f * (float)q)));
-  while (k > 1 && 2 * k * (k - 1) > q) --k;
-  while (2 * (k + 1) * k <= q) ++k;
-  return (int)(4 * ns - k);
-}
-
 // ---------------------------------------------------------------------------
 // double-float helpers
 // ---------------------------------------------------------------------------

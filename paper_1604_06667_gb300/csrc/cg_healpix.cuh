@@ -14,102 +14,129 @@
 namespace cg {
 namespace {
 
-struct RingGeo {
-  int64_t count, first;
-  double z, phase;
-};
+// The disc queries propose candidates; the support cut decides every pair
+// exactly afterwards, so an interval only has to contain the pixels that a
+// disc meets.  They run in FP32 (GB300 executes 1.6 FP64 operations per clock
+// and SM; the same queries in FP64 took 4.4 ms per pass over the 24,576 tiles
+// of an nside-256 HEALPix target grid): every angle below is good to ~5e-7
+// rad, and the discs are widened by kQueryMargin, which covers those errors
+// and widens the intervals by at most 4 % of a pixel of nside 8192.
+constexpr float kQueryMargin = 4e-6f;
+constexpr float kPiF = 3.14159265f;
 
-__device__ __forceinline__ RingGeo ring_geo(int64_t ns, int64_t i) {
-  RingGeo r;
-  const double dns = (double)ns;
-  if (i < ns) {
-    r.count = 4 * i;
-    r.first = 2 * i * (i - 1);
-    r.z = 1.0 - (double)(i * i) / (3.0 * dns * dns);
-    r.phase = 0.5;
-  } else if (i <= 3 * ns) {
-    r.count = 4 * ns;
-    r.first = 2 * ns * (ns - 1) + (i - ns) * 4 * ns;
-    r.z = 4.0 / 3.0 - 2.0 * (double)i / (3.0 * dns);
-    r.phase = (((i - ns) & 1) == 0) ? 0.5 : 0.0;
-  } else {
-    const int64_t k = 4 * ns - i;
-    r.count = 4 * k;
-    r.first = 12 * ns * ns - 2 * k * (k + 1);
-    r.z = -(1.0 - (double)(k * k) / (3.0 * dns * dns));
-    r.phase = 0.5;
-  }
-  return r;
-}
-
-__device__ __forceinline__ double ring_colat(int64_t ns, int64_t i) {
-  if (i <= 0) return 0.0;
-  if (i >= 4 * ns) return kPi;
-  return acos(ring_geo(ns, i).z);
-}
-
-// Continuous ring coordinate of a direction with cos(colatitude) = z.
-__device__ __forceinline__ double ring_coord(int64_t ns, double z) {
-  const double dns = (double)ns;
-  if (fabs(z) <= 2.0 / 3.0) return dns * (2.0 - 1.5 * z);
-  if (z > 0.0) return dns * sqrt(3.0 * (1.0 - z));
-  return 4.0 * dns - dns * sqrt(3.0 * (1.0 + z));
-}
-
-// Widest longitude half-width of the disc (centre colatitude tc, radius R)
-// over the colatitude band [ta, tb]: -1 if the disc misses the band, >= pi if
-// it covers every longitude there.  The half-width at colatitude t solves
-// cos R = cos tc cos t + sin tc sin t cos(dphi); its widest point over t is
-// at cos t = cos tc / cos R (or at a band edge).
-__device__ double disc_halfwidth(double tc, double R, double ta, double tb) {
-  if (tb < tc - R || ta > tc + R) return -1.0;
-  if (ta <= 0.0 && tc <= R) return 4.0 * kPi;
-  if (tb >= kPi && tc + R >= kPi) return 4.0 * kPi;
-  const double st = sin(tc), ct = cos(tc), cr = cos(R);
-  if (st <= 0.0) return 4.0 * kPi;
-  double lo = fmax(ta, tc - R), hi = fmin(tb, tc + R);
-  lo = fmax(lo, 1e-300);
-  hi = fmin(hi, kPi - 1e-16);
-  double ts = (fabs(ct / cr) <= 1.0) ? acos(ct / cr) : lo;
-  ts = fmin(fmax(ts, lo), hi);
-  double xmin = 1e300;
-  const double cand[3] = {lo, hi, ts};
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const double x = (cr - ct * cos(cand[q])) / (st * sin(cand[q]));
-    xmin = fmin(xmin, x);
-  }
-  if (xmin <= -1.0) return 4.0 * kPi;
-  if (xmin > 1.0) return -1.0;
-  return acos(xmin);
-}
-
-// A disc on the sphere: colatitude, longitude (radians) and radius.
+// A disc on the sphere: colatitude, longitude (radians), radius (< 0: none)
+// and the constants of its half-widths: sin(tc), and the colatitude where the
+// disc is widest (cos ts = cos tc / cos R; -1 if the disc holds a pole).
 struct Disc {
-  double tc, pc, R;
+  float tc, pc, R, st, ts;
 };
+
+__host__ __device__ __forceinline__ Disc make_disc_f(float x, float y, float z, float R) {
+  Disc d;
+  const float rho = sqrtf(x * x + y * y);
+  // colatitude from the nearer pole: accurate next to it, unlike acos(z)
+  const float tn = atan2f(rho, fabsf(z));
+  d.tc = z < 0.f ? kPiF - tn : tn;
+  d.pc = atan2f(y, x);
+  d.R = R + kQueryMargin;
+  d.st = sinf(tn);
+  // sin^2(ts / 2) = sin((tc + R) / 2) sin((tc - R) / 2) / cos R
+  d.ts = -1.f;
+  if (d.R < 1.5f && tn > d.R) {
+    const float q = sinf(0.5f * (tn + d.R)) * sinf(0.5f * (tn - d.R)) / cosf(d.R);
+    const float ts = 2.f * asinf(fminf(1.f, sqrtf(q)));
+    d.ts = z < 0.f ? kPiF - ts : ts;
+  }
+  return d;
+}
+
+// Half-width in longitude of the disc at its widest within the colatitude
+// band [ta, tb]: -1 if it misses the band, >= 4 if it may cover every
+// longitude there.  With u = t - tc, the haversine form
+//   sin^2(dphi / 2) = sin((R + u) / 2) sin((R - u) / 2) / (sin t sin tc)
+// has no cancellation; the half-width grows towards ts and falls beyond it,
+// so the band's colatitude nearest to ts is the widest.
+__host__ __device__ __forceinline__ float disc_halfwidth(const Disc& d, float ta, float tb) {
+  if (tb < d.tc - d.R || ta > d.tc + d.R) return -1.f;
+  if (ta <= 0.f && d.tc <= d.R) return 4.f;
+  if (tb >= kPiF && d.tc + d.R >= kPiF) return 4.f;
+  if (d.R >= 1.5f || !(d.st > 0.f)) return 4.f;
+  const float lo = fmaxf(fmaxf(ta, d.tc - d.R), 0.f);
+  const float hi = fminf(fminf(tb, d.tc + d.R), kPiF);
+  // a disc that holds a pole is widest at the end of the band nearest to it
+  float t = d.ts;
+  if (t < 0.f) t = (d.tc < 1.5707964f) ? lo : hi;
+  t = fminf(fmaxf(t, lo), hi);
+  const float u = t - d.tc;
+  const float num = fmaxf(sinf(0.5f * (d.R + u)), 0.f) * fmaxf(sinf(0.5f * (d.R - u)), 0.f);
+  const float den = sinf(t) * d.st;
+  if (!(num < den)) return 4.f;
+  return 2.f * asinf(sqrtf(num / den));
+}
+
+// Colatitude of ring i = 0 .. 4 ns: sin(theta / 2) = k / (ns sqrt 6) on the
+// caps' rings (z = 1 - k^2 / (3 ns^2)), acos(z) in the belt.
+__host__ __device__ __forceinline__ float ring_colat(int ns, int i) {
+  if (i <= 0) return 0.f;
+  if (i >= 4 * ns) return kPiF;
+  const float inv = 1.f / (float)ns;
+  if (i < ns) return 2.f * asinf((float)i * inv * 0.40824829f);
+  if (i > 3 * ns) return kPiF - 2.f * asinf((float)(4 * ns - i) * inv * 0.40824829f);
+  return acosf((float)(2 * ns - i) * inv * (2.f / 3.f));
+}
+
+// Continuous ring number of colatitude t (the inverse of ring_colat).
+__host__ __device__ __forceinline__ float ring_coord(int ns, float t) {
+  const float z = cosf(t);
+  if (fabsf(z) <= 2.f / 3.f) return (float)ns * (2.f - 1.5f * z);
+  if (z > 0.f) return (float)ns * 2.4494897f * sinf(0.5f * t);
+  return (float)ns * (4.f - 2.4494897f * sinf(0.5f * (kPiF - t)));
+}
+
+// The rings that a colatitude span [tlo, thi] meets, two on each side for the
+// pixels' extent and the rounding of the inverse.
+__host__ __device__ __forceinline__ void ring_span(int ns, float tlo, float thi, int& ilo, int& ihi) {
+  ilo = (int)floorf(ring_coord(ns, fmaxf(0.f, tlo))) - 2;
+  ihi = (int)ceilf(ring_coord(ns, fminf(kPiF, thi))) + 2;
+  ilo = ilo < 1 ? 1 : ilo;
+  ihi = ihi > 4 * ns - 1 ? 4 * ns - 1 : ihi;
+}
 
 // Pixel ranges of ring i met by the union of nd discs (the hull of their
 // pixel intervals on the ring, a superset); writes up to 2 into out.
-__device__ int ring_ranges(int64_t ns, int64_t i, const Disc* discs, int nd, Range* out) {
-  const RingGeo g = ring_geo(ns, i);
-  const double dphi = 2.0 * kPi / (double)g.count;
-  const double ta = ring_colat(ns, i - 1), tb = ring_colat(ns, i + 1);
+__host__ __device__ inline int ring_ranges(int ns, int i, const Disc* discs, int nd, Range* out) {
+  int count, first;
+  float phase = 0.5f;
+  if (i < ns) {
+    count = 4 * i;
+    first = 2 * i * (i - 1);
+  } else if (i <= 3 * ns) {
+    count = 4 * ns;
+    first = 2 * ns * (ns - 1) + (i - ns) * 4 * ns;
+    phase = (((i - ns) & 1) == 0) ? 0.5f : 0.f;
+  } else {
+    const int k = 4 * ns - i;
+    count = 4 * k;
+    first = 12 * ns * ns - 2 * k * (k + 1);
+  }
+  const float dphi = 2.f * kPiF / (float)count;
+  const float ta = ring_colat(ns, i - 1), tb = ring_colat(ns, i + 1);
   bool any = false, full = false;
-  double lo = 0.0, hi = 0.0;   // hull of [pc - W, pc + W], unwrapped near the first disc
+  float lo = 0.f, hi = 0.f;   // hull of [pc - W, pc + W], unwrapped near the first disc
   for (int q = 0; q < nd && !full; ++q) {
-    if (discs[q].R < 0.0) continue;   // empty group
-    const double hw = disc_halfwidth(discs[q].tc, discs[q].R, ta, tb);
-    if (hw < 0.0) continue;
-    const double W = hw + 0.5 * dphi + 1e-12;
-    if (W >= kPi) { full = true; break; }
-    double c = discs[q].pc;
-    if (any) {  // move c to within pi of the hull's first centre
-      const double ref = 0.5 * (lo + hi);
-      while (c - ref > kPi) c -= 2.0 * kPi;
-      while (ref - c > kPi) c += 2.0 * kPi;
-      lo = fmin(lo, c - W);
-      hi = fmax(hi, c + W);
+    if (discs[q].R < 0.f) continue;   // empty group
+    const float hw = disc_halfwidth(discs[q], ta, tb);
+    if (hw < 0.f) continue;
+    const float W = hw + 0.5f * dphi + 2e-6f;
+    if (W >= kPiF) { full = true; break; }
+    float c = discs[q].pc;
+    if (any) {  // move c to within pi of the hull's centre
+      const float ref = 0.5f * (lo + hi);
+      if (c - ref > kPiF) c -= 2.f * kPiF;
+      if (ref - c > kPiF) c += 2.f * kPiF;
+      lo = fminf(lo, c - W);
+      hi = fmaxf(hi, c + W);
+      if (hi - lo >= 2.f * kPiF) full = true;
     } else {
       lo = c - W;
       hi = c + W;
@@ -117,40 +144,30 @@ __device__ int ring_ranges(int64_t ns, int64_t i, const Disc* discs, int nd, Ran
     }
   }
   if (!any && !full) return 0;
-  int64_t jlo = 0, jhi = g.count - 1;
-  if (!full && hi - lo >= 2.0 * kPi) full = true;
+  int jlo = 0, jhi = count - 1;
   if (!full) {
-    jlo = (int64_t)ceil(lo / dphi - g.phase);
-    jhi = (int64_t)floor(hi / dphi - g.phase);
+    // interval ends in pixels: good to ~1e-2 of a pixel at nside 8192, and
+    // the half pixel in W reaches to the pixel centres
+    jlo = (int)ceilf(lo / dphi - phase - 0.02f);
+    jhi = (int)floorf(hi / dphi - phase + 0.02f);
     if (jhi < jlo) return 0;
-    if (jhi - jlo + 1 >= g.count) full = true;
+    if (jhi - jlo + 1 >= count) full = true;
   }
   if (full) {
-    if (out) out[0] = Range{(int32_t)g.first, (int32_t)(g.first + g.count - 1), (int32_t)i, 0};
+    out[0] = Range{first, first + count - 1, i, 0};
     return 1;
   }
-  int64_t a = jlo % g.count, b = jhi % g.count;
-  if (a < 0) a += g.count;
-  if (b < 0) b += g.count;
+  int a = jlo % count, b = jhi % count;
+  if (a < 0) a += count;
+  if (b < 0) b += count;
   if (a <= b) {
-    if (out) out[0] = Range{(int32_t)(g.first + a), (int32_t)(g.first + b), (int32_t)i, 0};
+    out[0] = Range{first + a, first + b, i, 0};
     return 1;
   }
-  if (out) {
-    out[0] = Range{(int32_t)g.first, (int32_t)(g.first + b), (int32_t)i, 0};
-    out[1] = Range{(int32_t)(g.first + a), (int32_t)(g.first + g.count - 1), (int32_t)i, 0};
-  }
+  out[0] = Range{first, first + b, i, 0};
+  out[1] = Range{first + a, first + count - 1, i, 0};
   return 2;
 }
-
-__device__ __forceinline__ Disc make_disc(double4 c, double r_rad) {
-  Disc d;
-  d.tc = acos(fmin(1.0, fmax(-1.0, c.z)));
-  d.pc = atan2(c.y, c.x);
-  d.R = c.w + r_rad;
-  return d;
-}
-
 
 __device__ __forceinline__ bool valid_coord(double lon, double lat) {
   return isfinite(lon) && isfinite(lat) && lat >= -90.0 && lat <= 90.0;
@@ -305,15 +322,6 @@ __device__ __forceinline__ int64_t ang2pix_ring_dual(int64_t ns, double lon, dou
   return ok ? p : ang2pix_ring_f64(ns, lon, lat);
 }
 
-// Ring number of pixel p (RING scheme); the belt division by 4 ns is a
-// shift when nside is a power of two (log2 given, else -1).
-__device__ __forceinline__ int64_t ring_of_key(int64_t ns, int lg, int64_t p) {
-  const int64_t ncap = 2 * ns * (ns - 1);
-  if (p >= ncap && p < 12 * ns * ns - ncap)
-    return ns + (lg >= 0 ? ((p - ncap) >> (lg + 2)) : (p - ncap) / (4 * ns));
-  return ring_of_pix(ns, p);
-}
-
 __device__ __forceinline__ int32_t lower_bound_u32(const uint32_t* __restrict__ a, int32_t lo,
                                                    int32_t hi, uint32_t v) {
   while (lo < hi) {
@@ -321,6 +329,14 @@ __device__ __forceinline__ int32_t lower_bound_u32(const uint32_t* __restrict__ 
     if (a[mid] < v) lo = mid + 1; else hi = mid;
   }
   return lo;
+}
+
+// First pixel of ring i = 0 .. 4 ns (ring 0 is empty, ring 4 ns past the end).
+__device__ __forceinline__ int64_t ring_first(int64_t ns, int64_t i) {
+  if (i < ns) return i < 1 ? 0 : 2 * i * (i - 1);
+  if (i <= 3 * ns) return 2 * ns * (ns - 1) + (i - ns) * 4 * ns;
+  const int64_t k = 4 * ns - i;
+  return 12 * ns * ns - 2 * k * (k + 1);
 }
 
 }  // namespace

@@ -47,7 +47,6 @@ struct Tiling {           // geometry of one tiling of the targets
   int64_t n_tiles = 0;
   float4* chi = nullptr;          // [n_tiles] centre hi (xyz), w = radius (rad)
   float4* clo = nullptr;          // [n_tiles] centre lo (xyz)
-  double4* c64 = nullptr;         // [n_tiles] FP64 centre, w = radius
   float4* a = nullptr;            // [n_tiles*T] u_t - centre (FP32)
   int64_t n_ranges = 0;
   int64_t* range_off = nullptr;   // [n_tiles + 1]
@@ -321,7 +320,6 @@ struct BatchIndexJob {
   int64_t n;              // samples
   int64_t off;            // first position of the job in the batch sample arrays
   int64_t nside;
-  int lg;                 // log2 nside (-1: not a power of two)
   uint64_t key_base;
   int64_t ring_base;      // first of the job's 4 nside + 1 ring offsets
   // the tiling of the job's gridder form: its candidate ranges are written
@@ -341,7 +339,7 @@ struct BatchIndex {
   BatchIndexJob* jobs = nullptr;    // device [n_jobs]
   int64_t* key_blk = nullptr;       // device [n_jobs + 1]: prefix of ceil(n / 256)
   int64_t n_key_blk = 0;
-  int64_t* gth_blk = nullptr;       // device [n_jobs + 1]: prefix of ceil((n + 1) / 256)
+  int64_t* gth_blk = nullptr;       // prefix of ceil(n / 256) + ceil((4 nside + 1) / 256)
   int64_t n_gth_blk = 0;
   int64_t* tile_off = nullptr;      // device [n_jobs + 1]: prefix of n_tiles
   uint64_t* key = nullptr;          // [N] composite keys, input order

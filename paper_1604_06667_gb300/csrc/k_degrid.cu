@@ -185,24 +185,18 @@ __global__ void __launch_bounds__(256) k_degrid(DegridArgs a) {
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ch = fmaxf(ch, __shfl_xor_sync(0xffffffffu, ch, o));
-    const double rt = 2.0 * asin(fmin(1.0, 0.5 * (double)ch)) * (1.0 + 1e-5) + 1e-6;
-    Disc disc;
-    disc.tc = acos(fmin(1.0, fmax(-1.0, (double)cz)));
-    disc.pc = atan2((double)cy, (double)cx);
-    disc.R = rt + a.kd.r_rad + 1e-6;
-    const double tlo = fmax(0.0, disc.tc - disc.R), thi = fmin(kPi, disc.tc + disc.R);
-    int64_t ilo = (int64_t)floor(ring_coord(a.ns, cos(tlo))) - 2;
-    int64_t ihi = (int64_t)ceil(ring_coord(a.ns, cos(thi))) + 2;
-    ilo = ilo < 1 ? 1 : ilo;
-    ihi = ihi > 4 * a.ns - 1 ? 4 * a.ns - 1 : ihi;
+    const float rt = 2.f * asinf(fminf(1.f, 0.5f * ch)) * (1.f + 1e-5f) + 1e-6f;
+    const Disc disc = make_disc_f(cx, cy, cz, rt + (float)a.kd.r_rad);
+    int ilo, ihi;
+    ring_span((int)a.ns, disc.tc - disc.R, disc.tc + disc.R, ilo, ihi);
     const float q1 = a.kd.k1, q2 = a.kd.k2;
-    for (int64_t base = ilo; base <= ihi; base += 32) {
+    for (int base = ilo; base <= ihi; base += 32) {
       // lane j: the target interval(s) of ring base + j
-      const int64_t ring = base + lane;
+      const int ring = base + lane;
       int2 iv[2] = {make_int2(0, 0), make_int2(0, 0)};
       if (ring <= ihi) {
         Range rr[2];
-        const int nr = ring_ranges(a.ns, ring, &disc, 1, rr);
+        const int nr = ring_ranges((int)a.ns, ring, &disc, 1, rr);
         const int32_t ta = a.t_ring_off[ring], tb = a.t_ring_off[ring + 1];
         for (int q = 0; q < nr && tb > ta; ++q) {
           const int32_t lo = lower_bound_u32(a.t_key, ta, tb, (uint32_t)rr[q].pix_lo);

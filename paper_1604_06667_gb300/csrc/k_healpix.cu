@@ -23,51 +23,45 @@ namespace {
 // (radius group radius + r): per ring, the hull of those discs' pixel
 // intervals, which follows the outline of the tile widened by r (one disc of
 // radius tile radius + r around the centre would hold ~1.4x as many samples
-// for a square tile).  Without groups: that one disc.
+// for a square tile).  Bound by the arithmetic of 32 lanes (rings) x 32 discs,
+// in FP32 (cg_healpix.cuh).
 constexpr int kQueryWarps = 8;
 constexpr int kMaxDiscs = 32;
 
 __global__ void __launch_bounds__(32 * kQueryWarps) k_tile_query(
-    const double4* __restrict__ tc64, const double4* __restrict__ grp64, int n_grp,
-    int64_t n_tiles, int64_t ns, double r_rad, int64_t* __restrict__ counts,
+    const double4* __restrict__ grp64, int n_grp,
+    int64_t n_tiles, int ns, double r_rad, int64_t* __restrict__ counts,
     const int64_t* __restrict__ offs, Range* __restrict__ out, int mode) {
   __shared__ Disc sdisc[kQueryWarps][kMaxDiscs];
   const int64_t tile = (int64_t)blockIdx.x * kQueryWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
   if (tile >= n_tiles) return;
   Disc* discs = sdisc[wq];
-  int nd = 1;
-  if (grp64) {
-    nd = n_grp;
-    if (lane < nd) {
-      const double4 gc = grp64[tile * nd + lane];
-      Disc d = make_disc(gc, r_rad);
-      if (gc.w < 0.0) d.R = -1.0;   // empty group
-      discs[lane] = d;
-    }
-  } else if (lane == 0) {
-    discs[0] = make_disc(tc64[tile], r_rad);
+  const int nd = n_grp;
+  if (lane < nd) {
+    const double4 gc = grp64[tile * nd + lane];
+    Disc d = make_disc_f((float)gc.x, (float)gc.y, (float)gc.z, (float)(gc.w + r_rad));
+    if (gc.w < 0.0) d.R = -1.f;   // empty group
+    discs[lane] = d;
   }
   __syncwarp();
   // colatitude span of all discs
-  double tlo = kPi, thi = 0.0;
+  float tlo = kPiF, thi = 0.f;
   for (int q = 0; q < nd; ++q) {
-    if (discs[q].R < 0.0) continue;
-    tlo = fmin(tlo, fmax(0.0, discs[q].tc - discs[q].R));
-    thi = fmax(thi, fmin(kPi, discs[q].tc + discs[q].R));
+    if (discs[q].R < 0.f) continue;
+    tlo = fminf(tlo, discs[q].tc - discs[q].R);
+    thi = fmaxf(thi, discs[q].tc + discs[q].R);
   }
   if (thi < tlo) {  // no member at all
     if (mode == 0 && lane == 0) counts[tile] = 0;
     return;
   }
-  int64_t ilo = (int64_t)floor(ring_coord(ns, cos(tlo))) - 2;
-  int64_t ihi = (int64_t)ceil(ring_coord(ns, cos(thi))) + 2;
-  ilo = ilo < 1 ? 1 : ilo;
-  ihi = ihi > 4 * ns - 1 ? 4 * ns - 1 : ihi;
+  int ilo, ihi;
+  ring_span(ns, tlo, thi, ilo, ihi);
   int64_t pos = (mode == 1) ? offs[tile] : 0;
   int64_t total = 0;
-  for (int64_t base = ilo; base <= ihi; base += 32) {
-    const int64_t i = base + lane;
+  for (int base = ilo; base <= ihi; base += 32) {
+    const int i = base + lane;
     Range rr[2];
     const int n = (i <= ihi) ? ring_ranges(ns, i, discs, nd, rr) : 0;
     int incl = n;
@@ -179,37 +173,28 @@ __global__ void k_sample_keys(int64_t ns, const double* __restrict__ lon,
 }
 
 
-// Sorted order: gather the unit vectors, and ring_off[i] = first sorted
-// position with ring >= i, i = 0 .. 4 ns (thread s writes the entries for
-// the rings after its predecessor's ring up to its own).
-__global__ void k_sample_gather(int64_t ns, int lg, const uint32_t* __restrict__ skey,
-                                const uint32_t* __restrict__ sval,
-                                const float4* __restrict__ u_hi,
-                                const float4* __restrict__ u_lo, int stride, int64_t n,
-                                float4* __restrict__ s_hi, float4* __restrict__ s_lo,
-                                int32_t* __restrict__ ring_off) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const int64_t npix = 12 * ns * ns;
-  const int64_t end = 4 * ns;
-  int64_t rc = end;
-  if (s < n) {
-    const int64_t idx = (int64_t)sval[s] * stride;
-    s_hi[s] = u_hi[idx];
-    s_lo[s] = u_lo[idx];
-    const int64_t k = skey[s];
-    rc = (k >= npix) ? end : ring_of_key(ns, lg, k);
+// Sorted order: gather the unit vectors (CTAs 0 .. nb - 1, one thread per
+// sample), and ring_off[i] = first sorted position with ring >= i, i = 0 ..
+// 4 ns (the CTAs after them, one thread per ring: a binary search for the
+// ring's first pixel).  Latency-bound: when the thread at a gap of the
+// coverage filled the entries of all the rings in the gap one by one, a small
+// field (thousands of empty rings before its first sample) paid for a serial
+// chain of thousands of stores: 2e4 samples at nside 4096 took 29.7 us, 1e6
+// samples 47 us; the searches run side by side with the gather.
+__global__ void __launch_bounds__(256) k_sample_gather(
+    int64_t ns, int64_t nb, const uint32_t* __restrict__ skey, const uint32_t* __restrict__ sval,
+    const float4* __restrict__ u_hi, const float4* __restrict__ u_lo, int stride, int64_t n,
+    float4* __restrict__ s_hi, float4* __restrict__ s_lo, int32_t* __restrict__ ring_off) {
+  if (blockIdx.x >= nb) {
+    const int64_t i = (int64_t)(blockIdx.x - nb) * 256 + threadIdx.x;
+    if (i <= 4 * ns) ring_off[i] = lower_bound_u32(skey, 0, (int32_t)n, (uint32_t)ring_first(ns, i));
+    return;
   }
-  int64_t rp = __shfl_up_sync(0xffffffffu, rc, 1);
-  if (lane == 0) {
-    rp = -1;
-    if (s > 0 && s - 1 < n) {
-      const int64_t k = skey[s - 1];
-      rp = (k >= npix) ? end : ring_of_key(ns, lg, k);
-    }
-  }
-  if (s > n) return;
-  for (int64_t i = rp + 1; i <= rc; ++i) ring_off[i] = (int32_t)s;
+  const int64_t s = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (s >= n) return;
+  const int64_t idx = (int64_t)sval[s] * stride;
+  s_hi[s] = u_hi[idx];
+  s_lo[s] = u_lo[idx];
 }
 
 
@@ -329,10 +314,20 @@ __global__ void __launch_bounds__(256) k_batch_keys(const BatchIndexJob* __restr
   u[2 * i + 1] = make_float4(x.lo, y.lo, sb.lo, 0.f);
 }
 
-// k_sample_gather for every job: each thread covers one position s = 0 .. n
-// of its job's segment (CTA b serves 256 of them, blk: prefix of the jobs'
-// CTA counts for n + 1 positions); ring offsets are relative to the segment,
-// so that each job sees its own index as if it ran alone.
+// First of the sorted composite keys [lo, hi) that is at least v.
+__device__ __forceinline__ int64_t lower_bound_u64(const uint64_t* __restrict__ a, int64_t lo,
+                                                   int64_t hi, uint64_t v) {
+  while (lo < hi) {
+    const int64_t mid = lo + ((hi - lo) >> 1);
+    if (a[mid] < v) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// k_sample_gather for every job: a job's CTAs (blk: prefix of the jobs' CTA
+// counts) serve its ceil(n / 256) blocks of samples and then its 4 nside + 1
+// ring offsets, which are relative to the job's segment, so that each job
+// sees its own index as if it ran alone.
 __global__ void __launch_bounds__(256) k_batch_gather(const BatchIndexJob* __restrict__ jobs,
                                                       const int64_t* __restrict__ blk, int n_jobs,
                                                       const uint64_t* __restrict__ skey64,
@@ -347,28 +342,24 @@ __global__ void __launch_bounds__(256) k_batch_gather(const BatchIndexJob* __res
   __syncthreads();
   const int j = s_job;
   const BatchIndexJob& J = jobs[j];
-  const int64_t s = (int64_t)(blockIdx.x - blk[j]) * 256 + threadIdx.x;   // 0 .. n
-  if (s > J.n) return;
-  const int64_t ns = J.nside;
-  const int64_t npix = 12 * ns * ns;
-  const int64_t end = 4 * ns;
-  int64_t rc = end;
-  if (s < J.n) {
-    const int64_t gs = J.off + s;
-    const int64_t rec = 2 * (J.off + (int64_t)sval[gs]);
-    s_hi[gs] = u[rec];
-    s_lo[gs] = u[rec + 1];
-    const int64_t k = (int64_t)(skey64[gs] - J.key_base);
-    skey[gs] = (uint32_t)k;
-    rc = (k >= npix) ? end : ring_of_key(ns, J.lg, k);
+  const int64_t b = (int64_t)blockIdx.x - blk[j];
+  const int64_t nb = (J.n + 255) / 256;
+  if (b >= nb) {
+    const int64_t i = (b - nb) * 256 + threadIdx.x;
+    if (i <= 4 * J.nside)
+      ring_off[J.ring_base + i] =
+          (int32_t)(lower_bound_u64(skey64, J.off, J.off + J.n,
+                                    J.key_base + (uint64_t)ring_first(J.nside, i)) -
+                    J.off);
+    return;
   }
-  int64_t rp = -1;
-  if (s > 0) {
-    const int64_t k = (int64_t)(skey64[J.off + s - 1] - J.key_base);
-    rp = (k >= npix) ? end : ring_of_key(ns, J.lg, k);
-  }
-  int32_t* ro = ring_off + J.ring_base;
-  for (int64_t i = rp + 1; i <= rc; ++i) ro[i] = (int32_t)s;
+  const int64_t s = b * 256 + threadIdx.x;
+  if (s >= J.n) return;
+  const int64_t gs = J.off + s;
+  const int64_t rec = 2 * (J.off + (int64_t)sval[gs]);
+  s_hi[gs] = u[rec];
+  s_lo[gs] = u[rec + 1];
+  skey[gs] = (uint32_t)(skey64[gs] - J.key_base);
 }
 
 // k_tile_ranges for the tiles of every job (one warp per tile).
@@ -499,7 +490,6 @@ cudaError_t unit_vectors(const double* lon, const double* lat, int64_t n, double
 void tiling_free(Tiling& t, cudaStream_t s) {
   dfree(t.chi, s);
   dfree(t.clo, s);
-  dfree(t.c64, s);
   dfree(t.a, s);
   dfree(t.tile_cand, s);
   dfree(t.order, s);
@@ -527,7 +517,7 @@ cudaError_t tiles_query(cg_grid* g, Tiling& t) {
   if ((e = dalloc(&counts, (size_t)nt, s)) != cudaSuccess) return e;
   const int n_grp = t.T / 4;
   k_tile_query<<<ceil_div(nt, kQueryWarps), 32 * kQueryWarps, 0, s>>>(
-      t.c64, t.grp64, n_grp, nt, g->nside, r, counts, nullptr, nullptr, 0);
+      t.grp64, n_grp, nt, g->nside, r, counts, nullptr, nullptr, 0);
   g->n_launches += 1;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   int64_t* h = (int64_t*)malloc(sizeof(int64_t) * (size_t)(nt + 1));
@@ -548,7 +538,7 @@ cudaError_t tiles_query(cg_grid* g, Tiling& t) {
   free(h);
   if (e != cudaSuccess) return e;
   k_tile_query<<<ceil_div(nt, kQueryWarps), 32 * kQueryWarps, 0, s>>>(
-      t.c64, t.grp64, n_grp, nt, g->nside, r, nullptr, t.range_off, t.ranges, 1);
+      t.grp64, n_grp, nt, g->nside, r, nullptr, t.range_off, t.ranges, 1);
   g->n_launches += 1;
   dfree(counts, s);
   dfree(g->ring_off, s);
@@ -599,12 +589,9 @@ cudaError_t samples_sort(cg_grid* g, int64_t n) {
 cudaError_t sorted_gather(int64_t ns, const uint32_t* skey, const uint32_t* sval,
                           const float4* u_hi, const float4* u_lo, int stride, int64_t n,
                           float4* s_hi, float4* s_lo, int32_t* ring_off, cudaStream_t s) {
-  int lg = -1;
-  if ((ns & (ns - 1)) == 0)
-    for (lg = 0; ((int64_t)1 << lg) < ns; ++lg) {
-    }
-  k_sample_gather<<<ceil_div(n + 1, 256), 256, 0, s>>>(ns, lg, skey, sval, u_hi, u_lo, stride, n, s_hi,
-                                                       s_lo, ring_off);
+  const int64_t nb = ceil_div(n, 256);
+  k_sample_gather<<<(unsigned)(nb + ceil_div(4 * ns + 1, 256)), 256, 0, s>>>(
+      ns, nb, skey, sval, u_hi, u_lo, stride, n, s_hi, s_lo, ring_off);
   return cudaGetLastError();
 }
 

@@ -132,7 +132,7 @@ template <int T>
 __global__ void __launch_bounds__(T) k_tile_build(
     const double* __restrict__ lon, const double* __restrict__ lat, int64_t P,
     const uint32_t* __restrict__ order, float4* __restrict__ tile_chi,
-    float4* __restrict__ tile_clo, double4* __restrict__ tile_c64, float4* __restrict__ tgt_a,
+    float4* __restrict__ tile_clo, float4* __restrict__ tgt_a,
     uint32_t* __restrict__ tgt_perm, float4* __restrict__ tgt_e, float4* __restrict__ tgt_n,
     double2* __restrict__ tgt_ll, double4* __restrict__ sub64, float4* __restrict__ subf,
     double4* __restrict__ grp64) {
@@ -266,7 +266,6 @@ __global__ void __launch_bounds__(T) k_tile_build(
     split_f64(cz, hz, lz);
     tile_chi[tile] = make_float4(hx, hy, hz, (float)radius);
     tile_clo[tile] = make_float4(lx, ly, lz, 0.f);
-    tile_c64[tile] = make_double4(cx, cy, cz, radius);
   }
 }
 
@@ -289,7 +288,6 @@ static cudaError_t tiling_alloc(Tiling& t, int T, int64_t P, cudaStream_t s) {
   cudaError_t e;
   if ((e = dalloc(&t.chi, (size_t)t.n_tiles, s)) != cudaSuccess) return e;
   if ((e = dalloc(&t.clo, (size_t)t.n_tiles, s)) != cudaSuccess) return e;
-  if ((e = dalloc(&t.c64, (size_t)t.n_tiles, s)) != cudaSuccess) return e;
   if ((e = dalloc(&t.a, (size_t)(t.n_tiles * T), s)) != cudaSuccess) return e;
   if ((e = dalloc(&t.tile_cand, (size_t)t.n_tiles, s)) != cudaSuccess) return e;
   if ((e = dalloc(&t.grp64, (size_t)(t.n_tiles * (T / 4)), s)) != cudaSuccess) return e;
@@ -364,10 +362,10 @@ cudaError_t targets_build(cg_grid* g, const double* lon, const double* lat) {
   }
   if (e == cudaSuccess) {
     k_tile_build<kTile2><<<(unsigned)g->t128.n_tiles, kTile2, 0, s>>>(
-        lon, lat, P, ord, g->t128.chi, g->t128.clo, g->t128.c64, g->t128.a, g->tgt_perm,
+        lon, lat, P, ord, g->t128.chi, g->t128.clo, g->t128.a, g->tgt_perm,
         g->tgt_e, g->tgt_n, g->tgt_ll, g->t128.sub64, g->t128.subf, g->t128.grp64);
     k_tile_build<kTile><<<(unsigned)g->t64.n_tiles, kTile, 0, s>>>(
-        lon, lat, P, ord, g->t64.chi, g->t64.clo, g->t64.c64, g->t64.a, nullptr, nullptr,
+        lon, lat, P, ord, g->t64.chi, g->t64.clo, g->t64.a, nullptr, nullptr,
         nullptr, nullptr, nullptr, nullptr, g->t64.grp64);
     g->n_launches += 2;
     e = cudaGetLastError();
