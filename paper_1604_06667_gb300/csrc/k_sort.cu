@@ -359,6 +359,7 @@ __global__ void __launch_bounds__(kThreads) k_os_pass_warp(
     st[(size_t)b * kRadix + tid] = os_word(epoch, kInc, prefix + c);
     blk_off[tid] = g_excl + prefix;
   }
+  __syncthreads();   // every digit's t_start (and blk_off) is written
   // the tile in sorted order in shared memory, then written out in runs per
   // digit (consecutive threads, consecutive positions)
 #pragma unroll
