@@ -138,6 +138,8 @@ void free_all(cg_grid* g) {
   dfree(g->pcw_acc, s);
   dfree(g->pcw_w, s);
   g->pcw_cap_data = 0;
+  dfree(g->rows, s);
+  g->rows_cap = 0;
   dfree(g->part_num, s);
   dfree(g->part_w, s);
   dfree(g->acc_num, s);
@@ -215,7 +217,10 @@ cg_status do_add(cg_grid* g, const double* lon, const double* lat, const void* d
   cudaEvent_t t0 = tmark(g);
   if (!reuse) {
     g->index_valid = false;
-    CG_CUDA(samples_keys(g, lon, lat, weights, n), where);
+    // a single channel's values travel with the records when they are there
+    // already (host-buffer calls still copy them) and the FP32 form reads them
+    g->rec_values = g->C == 1 && !tc && g->f32_cfg < 0 && !g->data_ready;
+    CG_CUDA(samples_keys(g, lon, lat, weights, n, g->rec_values ? data : nullptr, dtype), where);
   }
   cudaEvent_t t1 = tmark(g);
   if (!reuse) CG_CUDA(samples_sort(g, n), where);
@@ -241,8 +246,10 @@ cg_status do_add(cg_grid* g, const double* lon, const double* lat, const void* d
     // one-shot calls: the gridder writes R = N / W itself where it can
     const bool want = out != nullptr && g->acc_empty;
     bool direct = false;
-    CG_CUDA(grid_tiles_f32(g, data, dtype, want ? out : nullptr, want ? out_w : nullptr, &direct),
-            where);
+    const cudaError_t eg = grid_tiles_f32(g, data, dtype, want ? out : nullptr,
+                                          want ? out_w : nullptr, &direct);
+    g->rec_values = false;   // later passes bring values of their own
+    CG_CUDA(eg, where);
     if (fused) *fused = direct;
   }
   cudaEvent_t t4 = tmark(g);

@@ -183,6 +183,9 @@ struct cg_grid {
   float* part_num = nullptr;      // [n_split][slots][C]
   float2* part_w = nullptr;       // [n_split][slots]
   size_t part_cap_num = 0, part_cap_w = 0;
+  float* rows = nullptr;          // channel rows in sorted order (at most 8 channels)
+  size_t rows_cap = 0;
+  bool rec_values = false;        // this call's single-channel values lie in s_lo.w
 
   // accumulators (tile order)
   float* acc_num = nullptr;       // [slots][C]
@@ -235,8 +238,9 @@ cudaError_t targets_set_axes(cg_grid* g, double pa_deg);
 // k_healpix.cu -- ang2pix, ring offsets, tile disc queries, sample ranges.
 cudaError_t ang2pix_export(int nside, const double* lon, const double* lat, int64_t n,
                            int64_t* pix, cudaStream_t s);
+// values: null, or one channel value per sample (dtype) to travel with its record (s_lo.w)
 cudaError_t samples_keys(cg_grid* g, const double* lon, const double* lat, const float* weights,
-                         int64_t n);
+                         int64_t n, const void* values = nullptr, int dtype = CG_F32);
 cudaError_t unit_vectors(const double* lon, const double* lat, int64_t n, double* out,
                          cudaStream_t s);
 cudaError_t samples_sort(cg_grid* g, int64_t n);
@@ -298,6 +302,13 @@ struct GridArgs {
 // accumulators as usual.
 cudaError_t grid_tiles_f32(cg_grid* g, const void* data, int dtype, float* out = nullptr,
                            float* out_w = nullptr, bool* direct = nullptr);
+// k_grid_narrow.cu -- at most 8 channels: lanes over candidates.  rows: scratch
+// of n * narrow_width(C) floats (null: one channel, values in s_lo.w).
+constexpr int kNarrowMaxC = 8;
+int narrow_width(int C);
+int narrow_splits(int64_t n_tiles, int64_t n, int n_sms);
+cudaError_t grid_narrow(const GridArgs& a, const Tiling& t, int64_t n, int dtype, float* rows,
+                        cudaStream_t s);
 constexpr int kF32Configs = 7;   // register-blocking shapes of the FP32 gridder
 int f32_default_config(int C);
 // the same into given accumulators; dscale != 0 evaluates w d^2 dscale
@@ -427,6 +438,7 @@ struct NonfiniteRows {
   int cp;                 // channels per slab (<= 256)
   int n_slabs;
   int mode;               // 0 store, 1 add (into acc_num), 2 divide by W into out
+  bool skip_zero;         // pairs of weight zero take part only in a sum that is non-finite anyway
   float* out;             // mode 2: user-order map
   float* acc_num;         // modes 0, 1: slot-order numerator
   KernelDev kd;

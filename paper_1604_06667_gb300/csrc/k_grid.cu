@@ -711,19 +711,10 @@ cudaError_t launch(const GridArgs& a, int64_t n_tiles, int dtype, cudaStream_t s
   return cudaGetLastError();
 }
 
-// One FP32 gridder pass: choose the candidate splits, grow the partial-sum
-// scratch if needed, launch, reduce the splits, and compute the flagged
-// non-finite rows again.  A one-shot output (a.out) is kept only without
-// candidate splits; *direct tells whether the map was written.
-template <int PB, int CB, int NCG>
-cudaError_t run(cg_grid* g, GridArgs& a, int dtype, bool* direct) {
-  constexpr int CPAD = CB * NCG;
-  const int64_t nt = g->t64.n_tiles;
+// Scratch of a pass with a.n_split candidate shares, and whether it writes
+// the one-shot map itself (a.out is kept only without candidate splits).
+cudaError_t begin_pass(cg_grid* g, GridArgs& a, int n_slabs, bool* direct) {
   cudaStream_t s = g->stream;
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  a.n_split = splits_for<PB, CB, NCG>(nt, a.C, nsm);
   a.part_num = nullptr;
   a.part_w = nullptr;
   if (a.n_split > 1 || a.accumulate) {
@@ -750,19 +741,24 @@ cudaError_t run(cg_grid* g, GridArgs& a, int dtype, bool* direct) {
     a.part_num = g->part_num;
     a.part_w = g->part_w;
   }
-  const int n_slabs = (a.C + CPAD - 1) / CPAD;
   cudaError_t e = nonfinite_prepare(g, g->n_slots * (int64_t)n_slabs);
   if (e != cudaSuccess) return e;
   a.nf_bits = g->nf_bits;
   a.nf_any = g->nf_any;
   g->n_launches += 1;
-  e = launch<PB, CB, NCG>(a, nt, dtype, s);
-  if (e != cudaSuccess || nt == 0) return e;
+  return cudaSuccess;
+}
+
+// After the gridder: the splits' sum and the flagged non-finite rows
+// (bitmap rows of cpad channels).
+cudaError_t end_pass(cg_grid* g, const GridArgs& a, int dtype, int cpad, int n_slabs,
+                     bool skip_zero) {
+  cudaError_t e;
   if (a.n_split > 1) {
     const int64_t m = g->n_slots * (int64_t)(a.C + 1);
-    k_split_reduce<<<ceil_div(m, 256), 256, 0, s>>>(a.part_num, a.part_w, a.tgt_perm, g->n_slots,
-                                                    a.C, a.n_split, a.accumulate, a.acc_num,
-                                                    a.acc_w, a.nf_bits, CPAD, n_slabs);
+    k_split_reduce<<<ceil_div(m, 256), 256, 0, g->stream>>>(
+        a.part_num, a.part_w, a.tgt_perm, g->n_slots, a.C, a.n_split, a.accumulate, a.acc_num,
+        a.acc_w, a.nf_bits, cpad, n_slabs);
     g->n_launches += 1;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -771,13 +767,57 @@ cudaError_t run(cg_grid* g, GridArgs& a, int dtype, bool* direct) {
   rows.data = a.data;
   rows.dtype = dtype;
   rows.C = a.C;
-  rows.cp = CPAD;
+  rows.cp = cpad;
   rows.n_slabs = n_slabs;
   rows.mode = a.out ? 2 : (a.accumulate ? 1 : 0);
+  rows.skip_zero = skip_zero;
   rows.out = a.out;
   rows.acc_num = a.acc_num;
   rows.kd = a.kd;
   return nonfinite_fixup(g, rows);
+}
+
+int sm_count() {
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  return nsm;
+}
+
+// One FP32 gridder pass in a register-blocking shape: choose the candidate
+// splits, launch, reduce the splits, compute the flagged non-finite rows again.
+template <int PB, int CB, int NCG>
+cudaError_t run(cg_grid* g, GridArgs& a, int dtype, bool* direct) {
+  constexpr int CPAD = CB * NCG;
+  const int64_t nt = g->t64.n_tiles;
+  const int n_slabs = (a.C + CPAD - 1) / CPAD;
+  a.n_split = splits_for<PB, CB, NCG>(nt, a.C, sm_count());
+  cudaError_t e = begin_pass(g, a, n_slabs, direct);
+  if (e == cudaSuccess) e = launch<PB, CB, NCG>(a, nt, dtype, g->stream);
+  if (e != cudaSuccess || nt == 0) return e;
+  return end_pass(g, a, dtype, CPAD, n_slabs, false);
+}
+
+// The same pass for at most 8 channels (k_grid_narrow.cu).
+cudaError_t run_narrow(cg_grid* g, GridArgs& a, int dtype, bool* direct) {
+  const int64_t nt = g->t64.n_tiles;
+  const int cw = narrow_width(a.C);
+  const bool own_rows = !(g->rec_values && cw == 1);
+  const size_t need = (size_t)g->last_n * (size_t)cw;
+  if (own_rows && g->rows_cap < need) {
+    dfree(g->rows, g->stream);
+    g->rows_cap = 0;
+    const cudaError_t e = dalloc(&g->rows, need, g->stream);
+    if (e != cudaSuccess) return e;
+    g->rows_cap = need;
+  }
+  a.n_split = narrow_splits(nt, g->last_n, sm_count());
+  cudaError_t e = begin_pass(g, a, 1, direct);
+  if (e == cudaSuccess) e = grid_narrow(a, g->t64, g->last_n, dtype, own_rows ? g->rows : nullptr,
+                                         g->stream);
+  if (e != cudaSuccess) return e;
+  g->n_launches += own_rows ? 1 : 0;   // the rows' gather
+  return end_pass(g, a, dtype, cw, 1, true);
 }
 
 }  // namespace
@@ -823,7 +863,12 @@ cudaError_t grid_tiles_f32_to(cg_grid* g, const void* data, int dtype, float* ac
   a.tile_cand = g->t64.tile_cand;
   a.n_slots = g->n_slots;
   int cfg = g->f32_cfg;
-  if (cfg < 0 || cfg >= kF32Configs || C != g->C) cfg = f32_default_config(C);
+  if (cfg < 0 || cfg >= kF32Configs || C != g->C) {
+    // at most 8 channels: lanes over candidates (the register-blocked shapes
+    // stay for wider rows, for shapes asked for and for fused batches)
+    if (C <= kNarrowMaxC) return run_narrow(g, a, dtype, direct);
+    cfg = f32_default_config(C);
+  }
   switch (cfg) {
     case 0: return run<1, 4, 1>(g, a, dtype, direct);
     case 1: return run<1, 8, 1>(g, a, dtype, direct);
@@ -863,7 +908,7 @@ struct FixArgs {
   KernelDev kd;
   const void* data;
   int bf16;
-  int C, cp, n_slabs, mode;
+  int C, cp, n_slabs, mode, skip_zero;
   float* out;
   float* acc_num;
   const uint32_t* perm_t;
@@ -910,7 +955,7 @@ __device__ __forceinline__ void fix_word(const FixArgs& a, int64_t wd, FixShared
     const float4 chi = a.chi[tile], clo = a.clo[tile];
     const int c = slab * a.cp + tid;
     const bool mine = tid < a.cp && c < a.C;
-    float acc = 0.f;
+    float acc = 0.f, acc_nz = 0.f;   // all pairs, those of non-zero weight
     double wsum = 0.0;
     for (int64_t r = a.range_off[tile]; r < a.range_off[tile + 1]; ++r) {
       const int2 rg = a.range_s[r];
@@ -935,9 +980,14 @@ __device__ __forceinline__ void fix_word(const FixArgs& a, int64_t wd, FixShared
         const int n = min(kFixThreads, rg.y - j0);
         if (mine)
           for (int k = 0; k < n; ++k)
-            if (takes_part(F.w[k])) acc = fmaf(F.w[k], fix_load(a, (size_t)F.idx[k] * a.C + c), acc);
+            if (takes_part(F.w[k])) {
+              const float v = fix_load(a, (size_t)F.idx[k] * a.C + c);
+              acc = fmaf(F.w[k], v, acc);
+              if (F.w[k] != 0.f) acc_nz = fmaf(F.w[k], v, acc_nz);
+            }
       }
     }
+    if (a.skip_zero && isfinite(acc_nz)) acc = acc_nz;
     double W = 0.0;
     if (a.mode == 2) {
       F.wsum[tid] = wsum;
@@ -1010,6 +1060,7 @@ cudaError_t nonfinite_fixup(cg_grid* g, const NonfiniteRows& j) {
   a.cp = j.cp;
   a.n_slabs = j.n_slabs;
   a.mode = j.mode;
+  a.skip_zero = j.skip_zero ? 1 : 0;
   a.out = j.out;
   a.acc_num = j.acc_num;
   a.perm_t = g->tgt_perm;
@@ -1244,6 +1295,7 @@ __global__ void __launch_bounds__(kFixThreads) k_multi_fixup(const __grid_consta
     f.cp = J.pad;
     f.n_slabs = J.n_slabs;
     f.mode = J.a.out ? 2 : 0;
+    f.skip_zero = 0;
     f.out = J.a.out;
     f.acc_num = J.a.acc_num;
     f.perm_t = J.a.tgt_perm;

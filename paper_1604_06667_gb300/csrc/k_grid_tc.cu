@@ -1201,6 +1201,7 @@ cudaError_t grid_tiles_tc(cg_grid* g, const void* data, int mode, float* out, fl
   rows.cp = a.cp;
   rows.n_slabs = a.n_slabs;
   rows.mode = mode;
+  rows.skip_zero = false;
   rows.out = out;
   rows.acc_num = g->acc_num;
   rows.kd = g->kdev;
