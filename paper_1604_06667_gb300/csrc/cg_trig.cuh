@@ -93,7 +93,8 @@ __device__ __forceinline__ void df_sincos_deg(double a, df32& s, df32& c) {
   const float rh = __double2float_rn(r);
   const float rl = __double2float_rn(r - (double)rh);
   const df32 x = df_mul(df32{rh, rl}, df32{kD2R_hi, kD2R_lo});
-  const int j = __float2int_rn(x.hi * 64.f);
+  // (angles beyond 2^40 deg keep no exact remainder: stay inside the table)
+  const int j = max(-(kTrigTab - 1), min(kTrigTab - 1, __float2int_rn(x.hi * 64.f)));
   const int ja = j < 0 ? -j : j;
   const float4 tab = *reinterpret_cast<const float4*>(&kTrigTable.v[4 * ja]);
   const df32 S = (j < 0) ? df32{-tab.x, -tab.y} : df32{tab.x, tab.y};
