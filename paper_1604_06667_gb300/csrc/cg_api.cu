@@ -434,8 +434,7 @@ cg_status cg_set_kernel(cg_grid* g, int32_t kernel_type, const double* params, i
   kd.big_support = chord > 0.1 ? 1 : 0;
   g->kdev = kd;
   if (kernel_type == CG_GAUSS2D) CG_CUDA(targets_set_axes(g, pa), "cg_set_kernel");
-  CG_CUDA(tiles_query(g, g->t64), "cg_set_kernel");
-  CG_CUDA(tiles_query(g, g->t128), "cg_set_kernel");
+  CG_CUDA(tiles_query(g), "cg_set_kernel");
   // nside and tiles may have changed: the sample and target indices are stale
   g->index_valid = false;
   g->t64.ranges_gen = g->t128.ranges_gen = -1;

@@ -45,7 +45,7 @@ struct KernelDev {        // kernel constants used by the gridder
 struct Tiling {           // geometry of one tiling of the targets
   int T = 0;
   int64_t n_tiles = 0;
-  float4* chi = nullptr;          // [n_tiles] centre hi (xyz), w = radius (rad)
+  float4* chi = nullptr;          // [n_tiles] centre hi (xyz)
   float4* clo = nullptr;          // [n_tiles] centre lo (xyz)
   float4* a = nullptr;            // [n_tiles*T] u_t - centre (FP32)
   int64_t n_ranges = 0;
@@ -57,13 +57,11 @@ struct Tiling {           // geometry of one tiling of the targets
   int32_t* order = nullptr;       // [cap_order] persistent schedule: waves of neighbouring items
   int64_t cap_order = 0;
   // 128-target tiles only: the four 32-target quarters (one TMEM lane quarter
-  // each; k-d leaves), FP64 centre + radius, and the centre relative to the
-  // tile centre in FP32 with the radius as a chord
-  double4* sub64 = nullptr;       // [n_tiles * 4]
+  // each; k-d leaves), centre relative to the tile centre and radius (chord)
   float4* subf = nullptr;         // [n_tiles * 4]
-  // every tile: its 4-target groups (compact k-d leaves), FP64 centre + radius
-  // (radius < 0: an empty group); the candidate query's discs
-  double4* grp64 = nullptr;       // [n_tiles * T / 4]
+  // every tile: its 4-target groups (compact k-d leaves), centre and radius
+  // (rad; < 0: an empty group); the candidate query's discs
+  float4* grp = nullptr;          // [n_tiles * T / 4]
   int64_t ranges_gen = -1;        // sample index the per-add ranges belong to
 };
 
@@ -252,7 +250,7 @@ cudaError_t sorted_gather(int64_t ns, const uint32_t* skey, const uint32_t* sval
                           const float4* u_hi, const float4* u_lo, int stride, int64_t n,
                           float4* s_hi, float4* s_lo, int32_t* ring_off, cudaStream_t s);
 cudaError_t tiles_ranges(cg_grid* g, Tiling& t);
-cudaError_t tiles_query(cg_grid* g, Tiling& t);
+cudaError_t tiles_query(cg_grid* g);   // both tilings
 void tiling_free(Tiling& t, cudaStream_t s);
 cudaError_t export_index(cg_grid* g, int64_t* sorted_pix, int64_t* perm, int64_t* ring_off,
                          int64_t n);

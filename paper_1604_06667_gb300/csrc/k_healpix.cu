@@ -29,8 +29,8 @@ constexpr int kQueryWarps = 8;
 constexpr int kMaxDiscs = 32;
 
 __global__ void __launch_bounds__(32 * kQueryWarps) k_tile_query(
-    const double4* __restrict__ grp64, int n_grp,
-    int64_t n_tiles, int ns, double r_rad, int64_t* __restrict__ counts,
+    const float4* __restrict__ grp, int n_grp,
+    int64_t n_tiles, int ns, float r_rad, int64_t* __restrict__ counts,
     const int64_t* __restrict__ offs, Range* __restrict__ out, int mode) {
   __shared__ Disc sdisc[kQueryWarps][kMaxDiscs];
   const int64_t tile = (int64_t)blockIdx.x * kQueryWarps + (threadIdx.x >> 5);
@@ -39,9 +39,9 @@ __global__ void __launch_bounds__(32 * kQueryWarps) k_tile_query(
   Disc* discs = sdisc[wq];
   const int nd = n_grp;
   if (lane < nd) {
-    const double4 gc = grp64[tile * nd + lane];
-    Disc d = make_disc_f((float)gc.x, (float)gc.y, (float)gc.z, (float)(gc.w + r_rad));
-    if (gc.w < 0.0) d.R = -1.f;   // empty group
+    const float4 gc = grp[tile * nd + lane];
+    Disc d = make_disc_f(gc.x, gc.y, gc.z, gc.w + r_rad);
+    if (gc.w < 0.f) d.R = -1.f;   // empty group
     discs[lane] = d;
   }
   __syncwarp();
@@ -83,6 +83,50 @@ __global__ void __launch_bounds__(32 * kQueryWarps) k_tile_query(
   if (mode == 0 && lane == 0) counts[tile] = total;
 }
 
+
+// off[i] = sum of counts[0 .. i), i = 0 .. n: one CTA, a run of consecutive
+// counts per thread and step (n is the number of tiles, at most ~1e5 in use).
+constexpr int kScanThreads = 1024;
+constexpr int kScanPer = 8;
+__global__ void __launch_bounds__(kScanThreads) k_count_scan(const int64_t* __restrict__ counts,
+                                                             int64_t n, int64_t* __restrict__ off) {
+  __shared__ int64_t wsum[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int64_t carry = 0;
+  for (int64_t base = 0; base < n; base += kScanThreads * kScanPer) {
+    int64_t v[kScanPer], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) {
+      const int64_t i = base + (int64_t)tid * kScanPer + k;
+      v[k] = i < n ? counts[i] : 0;
+      sum += v[k];
+    }
+    int64_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    int64_t before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < 32; ++w) {
+      if (w < warp) before += wsum[w];
+      all += wsum[w];
+    }
+    int64_t x = carry + before + incl - sum;
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) {
+      const int64_t i = base + (int64_t)tid * kScanPer + k;
+      if (i < n) off[i] = x;
+      x += v[k];
+    }
+    carry += all;
+    __syncthreads();   // wsum is rewritten by the next step
+  }
+  if (tid == 0) off[n] = carry;
+}
 
 // RING index of a valid direction and the double-float sine / cosine of its
 // latitude and longitude.  Ordinary angles (|lon| < 2048 deg) take an FP64-free
@@ -502,8 +546,7 @@ void tiling_free(Tiling& t, cudaStream_t s) {
   dfree(t.tile_cand, s);
   dfree(t.order, s);
   t.cap_order = 0;
-  dfree(t.sub64, s);
-  dfree(t.grp64, s);
+  dfree(t.grp, s);
   dfree(t.subf, s);
   dfree(t.range_off, s);
   dfree(t.ranges, s);
@@ -512,46 +555,47 @@ void tiling_free(Tiling& t, cudaStream_t s) {
   t.n_ranges = 0;
 }
 
-cudaError_t tiles_query(cg_grid* g, Tiling& t) {
+// Both tilings' candidate ranges: count, exclusive scan, write.  The host
+// waits once, for the two totals that size the range arrays.
+cudaError_t tiles_query(cg_grid* g) {
   cudaStream_t s = g->stream;
-  const int64_t nt = t.n_tiles;
-  const double r = g->support_deg * kDeg2Rad;
-  int64_t* counts = nullptr;
-  cudaError_t e;
-  dfree(t.range_off, s);
-  dfree(t.ranges, s);
-  dfree(t.range_s, s);
-  dfree(t.range_c, s);
-  if ((e = dalloc(&counts, (size_t)nt, s)) != cudaSuccess) return e;
-  const int n_grp = t.T / 4;
-  k_tile_query<<<ceil_div(nt, kQueryWarps), 32 * kQueryWarps, 0, s>>>(
-      t.grp64, n_grp, nt, g->nside, r, counts, nullptr, nullptr, 0);
-  g->n_launches += 1;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  int64_t* h = (int64_t*)malloc(sizeof(int64_t) * (size_t)(nt + 1));
-  if (!h) return cudaErrorMemoryAllocation;
-  e = cudaMemcpyAsync(h + 1, counts, sizeof(int64_t) * (size_t)nt, cudaMemcpyDeviceToHost, s);
+  const float r = (float)(g->support_deg * kDeg2Rad);
+  Tiling* ts[2] = {&g->t64, &g->t128};
+  int64_t* counts[2] = {nullptr, nullptr};
+  int64_t total[2] = {0, 0};
+  cudaError_t e = cudaSuccess;
+  for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+    Tiling& t = *ts[q];
+    dfree(t.range_off, s);
+    dfree(t.ranges, s);
+    dfree(t.range_s, s);
+    dfree(t.range_c, s);
+    t.n_ranges = 0;
+    e = dalloc(&counts[q], (size_t)t.n_tiles, s);
+    if (e == cudaSuccess) e = dalloc(&t.range_off, (size_t)t.n_tiles + 1, s);
+    if (e != cudaSuccess) break;
+    k_tile_query<<<ceil_div(t.n_tiles, kQueryWarps), 32 * kQueryWarps, 0, s>>>(
+        t.grp, t.T / 4, t.n_tiles, g->nside, r, counts[q], nullptr, nullptr, 0);
+    k_count_scan<<<1, kScanThreads, 0, s>>>(counts[q], t.n_tiles, t.range_off);
+    g->n_launches += 2;
+    e = cudaMemcpyAsync(&total[q], t.range_off + t.n_tiles, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) { free(h); return e; }
-  h[0] = 0;
-  for (int64_t i = 0; i < nt; ++i) h[i + 1] += h[i];
-  t.n_ranges = h[nt];
-  if ((e = dalloc(&t.range_off, (size_t)nt + 1, s)) != cudaSuccess) { free(h); return e; }
-  if ((e = dalloc(&t.ranges, (size_t)t.n_ranges, s)) != cudaSuccess) { free(h); return e; }
-  if ((e = dalloc(&t.range_s, (size_t)t.n_ranges, s)) != cudaSuccess) { free(h); return e; }
-  if ((e = dalloc(&t.range_c, (size_t)t.n_ranges, s)) != cudaSuccess) { free(h); return e; }
-  e = cudaMemcpyAsync(t.range_off, h, sizeof(int64_t) * (size_t)(nt + 1),
-                      cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  free(h);
+  for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+    Tiling& t = *ts[q];
+    t.n_ranges = total[q];
+    if ((e = dalloc(&t.ranges, (size_t)t.n_ranges, s)) != cudaSuccess) break;
+    if ((e = dalloc(&t.range_s, (size_t)t.n_ranges, s)) != cudaSuccess) break;
+    if ((e = dalloc(&t.range_c, (size_t)t.n_ranges, s)) != cudaSuccess) break;
+    k_tile_query<<<ceil_div(t.n_tiles, kQueryWarps), 32 * kQueryWarps, 0, s>>>(
+        t.grp, t.T / 4, t.n_tiles, g->nside, r, nullptr, t.range_off, t.ranges, 1);
+    g->n_launches += 1;
+    e = cudaGetLastError();
+  }
+  for (int q = 0; q < 2; ++q) dfree(counts[q], s);
   if (e != cudaSuccess) return e;
-  k_tile_query<<<ceil_div(nt, kQueryWarps), 32 * kQueryWarps, 0, s>>>(
-      t.grp64, n_grp, nt, g->nside, r, nullptr, t.range_off, t.ranges, 1);
-  g->n_launches += 1;
-  dfree(counts, s);
   dfree(g->ring_off, s);
-  if ((e = dalloc(&g->ring_off, (size_t)(4 * g->nside + 1), s)) != cudaSuccess) return e;
-  return cudaGetLastError();
+  return dalloc(&g->ring_off, (size_t)(4 * g->nside + 1), s);
 }
 
 static cudaError_t ensure_samples(cg_grid* g, int64_t n) {

@@ -3,199 +3,385 @@
 // The paper grids onto the pixel centres of a WCS map or onto a list of sight
 // lines (Sect. 3.5, WcsGrid / SlGrid).  Here targets are always a list of
 // directions.  To give each CTA a compact group of targets (its "tile"), the
-// targets are split by a k-d tree over their unit vectors: every node is cut
-// along its widest axis at a multiple of the leaf size, so all leaves hold
-// exactly that many targets (except the last) and each leaf is a compact box.
-// The tree is cut to 128-target leaves, then each leaf into 64 + 64, 32 + 32
-// and on down to groups of 4, so a 128-tile is two 64-tiles, four 32-target
-// quarters and thirty-two 4-target groups, all compact (consecutive slots).
-// The tree is built level by level with one stable 64-bit radix sort per
-// level keyed by (child node, coordinate along the child's widest axis).
+// targets are split by a k-d tree over their unit vectors: every node is
+// sorted along its widest axis and cut at a multiple of the leaf size, so all
+// leaves hold exactly that many targets (except the last) and each leaf is a
+// compact box.  The tree is cut to 128-target leaves, then each leaf into
+// 64 + 64, 32 + 32 and on down to groups of 4, so a 128-tile is two 64-tiles,
+// four 32-target quarters and thirty-two 4-target groups, all compact
+// (consecutive slots).  A position's node at any level follows from its index
+// alone (the cuts depend on counts only).
+//
+// A new set of targets is part of every new map, so the build is a path of its
+// own: levels of nodes above 4096 targets run over the whole array (bounding
+// boxes, 16-bit coordinates within the node's box, one radix sort of the
+// 32-bit (node, coordinate) keys per level), all levels below in shared
+// memory, one CTA per node.  786,432 sight lines: 18 levels of 64-bit
+// three-kernel sort passes with per-target atomics and FP64 geometry took
+// 18 ms of kernels.
 // Each tile stores
-//   - its centre e_c (FP64, and as a double-float pair) and angular radius;
-//   - for every member, u_t - e_c in FP32 (accurate relative to its size);
+//   - its centre e_c (near the targets' mean) and, for every member,
+//     u_t - e_c in FP32 (accurate relative to its size; u_t as a double-float);
 //   - the local east / north unit vectors (for the elliptical kernel);
-//   - the member's longitude / latitude in FP64 (guard-band recomputation).
-// FP64 is acceptable here: this runs once per target set, not per sample.
+//   - the member's longitude / latitude in FP64 (guard-band recomputation);
+//   - the discs of its 4-target groups and (128-tiles) 32-target quarters.
+#include <algorithm>
+
 #include "cg_common.cuh"
 #include "cg_internal.h"
+#include "cg_trig.cuh"
 
 namespace cg {
 namespace {
 
-__device__ __forceinline__ uint32_t orderable(float f) {
-  const uint32_t b = __float_as_uint(f);
+__host__ __device__ __forceinline__ uint32_t orderable_bits(uint32_t b) {
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ uint32_t orderable(float f) { return orderable_bits(__float_as_uint(f)); }
+__device__ __forceinline__ float from_orderable(uint32_t u) {
+  return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
 __device__ __forceinline__ bool valid_coord(double lon, double lat) {
   return isfinite(lon) && isfinite(lat) && lat >= -90.0 && lat <= 90.0;
 }
 
-__device__ __forceinline__ void unit_vec(double lon, double lat, double& x, double& y,
-                                         double& z) {
-  double sb, cb, sl, cl;
-  sincos(lat * kDeg2Rad, &sb, &cb);
-  sincos(lon * kDeg2Rad, &sl, &cl);
-  x = cb * cl;
-  y = cb * sl;
-  z = sb;
+// Double-float sine and cosine of a longitude or latitude in degrees (FP64
+// operations only for angles beyond the split's range).
+__device__ __forceinline__ void sincos_deg(double a, df32& s, df32& c) {
+  if (df_split_ok(a) && fabs(a) < 2048.0) {
+    df_sincos_deg_df(df_split(a), s, c);
+  } else {
+    double sd, cd;
+    sincos(a * kDeg2Rad, &sd, &cd);
+    split_f64(sd, s.hi, s.lo);
+    split_f64(cd, c.hi, c.lo);
+  }
 }
 
-__global__ void k_target_init(const double* __restrict__ lon, const double* __restrict__ lat,
-                              int64_t P, float4* __restrict__ pos, uint32_t* __restrict__ ord,
-                              uint32_t* __restrict__ nid, unsigned* err) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) k_target_init(const double* __restrict__ lon,
+                                                     const double* __restrict__ lat, int64_t P,
+                                                     float4* __restrict__ u_hi,
+                                                     float4* __restrict__ u_lo,
+                                                     uint32_t* __restrict__ ord, unsigned* err) {
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= P) return;
   const double lo = lon[i], la = lat[i];
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 h = make_float4(0.f, 0.f, 0.f, 0.f), l = h;
   if (valid_coord(lo, la)) {
-    double x, y, z;
-    unit_vec(lo, la, x, y, z);
-    v = make_float4((float)x, (float)y, (float)z, 0.f);
+    df32 sb, cb, sl, cl;
+    sincos_deg(la, sb, cb);
+    sincos_deg(lo, sl, cl);
+    const df32 x = df_mul(cb, cl), y = df_mul(cb, sl);
+    h = make_float4(x.hi, y.hi, sb.hi, 0.f);
+    l = make_float4(x.lo, y.lo, sb.lo, 0.f);
   } else {
     set_error(err, ERR_BAD_TARGET);
   }
-  pos[i] = v;
+  u_hi[i] = h;
+  u_lo[i] = l;
   ord[i] = (uint32_t)i;
-  nid[i] = 0;
 }
 
-// First / one-past-last position of every node in the current order.
-__global__ void k_node_bounds(const uint32_t* __restrict__ nid, int64_t P,
-                              uint32_t* __restrict__ nstart, uint32_t* __restrict__ nend) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= P) return;
-  const uint32_t n = nid[s];
-  if (s == 0 || nid[s - 1] != n) nstart[n] = (uint32_t)s;
-  if (s == P - 1 || nid[s + 1] != n) nend[n] = (uint32_t)(s + 1);
-}
+// ---- k-d tree ----
+constexpr int kNodeCap = 4096;     // targets of a node finished in shared memory
+constexpr int kNodeThreads = 1024;
 
-// Child of every position (left part = a multiple of kTile targets) and the
-// bounding box of every child (order-preserving integer min / max).
-__global__ void k_node_split(const uint32_t* __restrict__ nid, const uint32_t* __restrict__ ord,
-                             const float4* __restrict__ pos, int64_t P, uint32_t leaf,
-                             const uint32_t* __restrict__ nstart,
-                             const uint32_t* __restrict__ nend, uint32_t* __restrict__ child,
-                             uint32_t* __restrict__ bmin, uint32_t* __restrict__ bmax) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= P) return;
-  const uint32_t n = nid[s];
-  const uint32_t st = nstart[n], cnt = nend[n] - st;
-  uint32_t c = 2u * n;
-  if (cnt > leaf) {
-    const uint32_t m = (cnt + leaf - 1) / leaf;
-    const uint32_t left = leaf * (m / 2);
-    if ((uint32_t)s - st >= left) c += 1u;
+struct Node {
+  uint32_t id, start, cnt;         // id: path from the root (0 left, 1 right)
+};
+
+// The part of node q that holds position s after its cut at a multiple of leaf.
+__device__ __forceinline__ void descend(Node& q, uint32_t s, uint32_t leaf) {
+  q.id *= 2u;
+  if (q.cnt <= leaf) return;
+  const uint32_t left = leaf * (((q.cnt + leaf - 1) / leaf) / 2);
+  if (s - q.start >= left) {
+    q.id += 1u;
+    q.start += left;
+    q.cnt -= left;
+  } else {
+    q.cnt = left;
   }
-  child[s] = c;
-  const float4 v = pos[ord[s]];
-  atomicMin(&bmin[3 * c + 0], orderable(v.x));
-  atomicMin(&bmin[3 * c + 1], orderable(v.y));
-  atomicMin(&bmin[3 * c + 2], orderable(v.z));
-  atomicMax(&bmax[3 * c + 0], orderable(v.x));
-  atomicMax(&bmax[3 * c + 1], orderable(v.y));
-  atomicMax(&bmax[3 * c + 2], orderable(v.z));
 }
 
-__device__ __forceinline__ float from_orderable(uint32_t u) {
-  return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
+__device__ __forceinline__ Node node_at(uint32_t s, uint32_t P, int level) {
+  Node q{0u, 0u, P};
+  for (int l = 0; l < level; ++l) descend(q, s, (uint32_t)kTile2);
+  return q;
 }
 
-// Sort key: (child node, coordinate along the child's widest axis).
-__global__ void k_node_keys(const uint32_t* __restrict__ child, const uint32_t* __restrict__ ord,
-                            const float4* __restrict__ pos, int64_t P,
-                            const uint32_t* __restrict__ bmin, const uint32_t* __restrict__ bmax,
-                            uint64_t* __restrict__ key, uint32_t* __restrict__ val) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Bounding boxes of the nodes of a level: box[6 n] = min x, y, z, then the
+// complements of max x, y, z (order-preserving integers, so one fill of ones
+// and one atomic minimum serve both).  A warp covers 256 positions and
+// reduces before its atomics (nodes start at multiples of 128): with one
+// atomic per target and side the first levels serialised on a few addresses
+// (13 ms for 786,432 targets).
+__global__ void __launch_bounds__(256) k_kd_box(const float4* __restrict__ pos,
+                                                const uint32_t* __restrict__ ord, uint32_t P,
+                                                int level, uint32_t* __restrict__ box) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t s0 = (blockIdx.x * 8u + (threadIdx.x >> 5)) * 256u;
+  uint32_t b[6], cur = 0xffffffffu;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) b[k] = 0xffffffffu;
+  auto flush = [&]() {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const uint32_t m = __reduce_min_sync(0xffffffffu, b[k]);
+      if (lane == 0) atomicMin(&box[6 * cur + k], m);
+      b[k] = 0xffffffffu;
+    }
+  };
+  for (int r = 0; r < 8; ++r) {
+    const uint32_t sw = s0 + 32u * r;   // uniform over the warp
+    if (sw >= P) break;
+    const uint32_t id = node_at(sw, P, level).id;
+    if (id != cur && cur != 0xffffffffu) flush();
+    cur = id;
+    const uint32_t s = sw + lane;
+    if (s < P) {
+      const float4 v = pos[ord[s]];
+      const uint32_t x = orderable(v.x), y = orderable(v.y), z = orderable(v.z);
+      b[0] = min(b[0], x);
+      b[1] = min(b[1], y);
+      b[2] = min(b[2], z);
+      b[3] = min(b[3], ~x);
+      b[4] = min(b[4], ~y);
+      b[5] = min(b[5], ~z);
+    }
+  }
+  if (cur != 0xffffffffu) flush();
+}
+
+// Sort key: (node, 16-bit coordinate within the node's box along its widest
+// axis).
+__global__ void __launch_bounds__(256) k_kd_keys(const float4* __restrict__ pos,
+                                                 const uint32_t* ord, uint32_t P, int level,
+                                                 const uint32_t* __restrict__ box,
+                                                 uint32_t* __restrict__ key, uint32_t* val) {
+  const uint32_t s = blockIdx.x * 256u + threadIdx.x;
   if (s >= P) return;
-  const uint32_t c = child[s];
-  const float ex = from_orderable(bmax[3 * c + 0]) - from_orderable(bmin[3 * c + 0]);
-  const float ey = from_orderable(bmax[3 * c + 1]) - from_orderable(bmin[3 * c + 1]);
-  const float ez = from_orderable(bmax[3 * c + 2]) - from_orderable(bmin[3 * c + 2]);
+  const uint32_t id = node_at(s, P, level).id;
+  float lo[3], ext[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    lo[k] = from_orderable(box[6 * id + k]);
+    ext[k] = from_orderable(~box[6 * id + 3 + k]) - lo[k];
+  }
   const uint32_t o = ord[s];
   const float4 v = pos[o];
-  const float coord = (ex >= ey && ex >= ez) ? v.x : ((ey >= ez) ? v.y : v.z);
-  key[s] = ((uint64_t)c << 32) | orderable(coord);
+  const int ax = (ext[0] >= ext[1] && ext[0] >= ext[2]) ? 0 : (ext[1] >= ext[2] ? 1 : 2);
+  const float c = ax == 0 ? v.x - lo[0] : (ax == 1 ? v.y - lo[1] : v.z - lo[2]);
+  const float q = ext[ax] > 0.f ? c / ext[ax] * 65535.f : 0.f;
+  key[s] = (id << 16) | min((uint32_t)q, 65535u);
   val[s] = o;
 }
 
-__global__ void k_node_unpack(const uint64_t* __restrict__ key, int64_t P,
-                              uint32_t* __restrict__ nid) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < P) nid[s] = (uint32_t)(key[s] >> 32);
+struct NodeSmem {
+  uint64_t key[kNodeCap];          // (segment, coordinate, place in the node)
+  float pos[3][kNodeCap];
+  uint32_t box[128][6];            // segments of at least 32 targets
+};
+
+// All levels below `level` of node blockIdx.x, down to groups of 4: per level
+// the segments' boxes, then a sort along each segment's widest axis.  Bound by
+// the barriers of the bitonic sorts; segments of at most 128 targets start at
+// multiples of their power-of-two size, so only their own steps run.
+__global__ void __launch_bounds__(kNodeThreads) k_kd_node(const float4* __restrict__ pos,
+                                                          const uint32_t* __restrict__ ord,
+                                                          uint32_t P, int level, int levels2,
+                                                          uint32_t* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  NodeSmem& S = *reinterpret_cast<NodeSmem*>(raw);
+  const int tid = threadIdx.x, lane = tid & 31;
+  // the node: descend along the bits of its id
+  Node nd{0u, 0u, P};
+  for (int l = 0; l < level; ++l) {
+    const uint32_t leaf = (uint32_t)kTile2;
+    const uint32_t left = nd.cnt > leaf ? leaf * (((nd.cnt + leaf - 1) / leaf) / 2) : nd.cnt;
+    if ((blockIdx.x >> (level - 1 - l)) & 1u) {
+      nd.start += left;
+      nd.cnt -= left;
+    } else {
+      nd.cnt = left;
+    }
+  }
+  const uint32_t n = nd.cnt;
+  uint32_t np = 128;
+  while (np < n) np <<= 1;
+  constexpr int kPer = kNodeCap / kNodeThreads;
+  Node seg[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const uint32_t i = tid + k * kNodeThreads;
+    seg[k] = Node{0u, 0u, n};
+    if (i < np) S.key[i] = i < n ? (uint64_t)i : ~0ull;
+    if (i < n) {
+      const float4 v = pos[ord[nd.start + i]];
+      S.pos[0][i] = v.x;
+      S.pos[1][i] = v.y;
+      S.pos[2][i] = v.z;
+    }
+  }
+  __syncthreads();
+  for (int l = level; l < levels2 + 5; ++l) {
+    // size of the level's segments: multiples of 128 down to tiles, then halves
+    const uint32_t cap = l <= levels2 ? 128u : (128u >> (l - levels2));
+    const bool small = l >= levels2;     // segments of at most cap targets, aligned to cap
+    if (cap >= 32u) {
+      for (int i = tid; i < 128 * 6; i += kNodeThreads) S.box[i / 6][i % 6] = 0xffffffffu;
+      __syncthreads();
+    }
+    uint32_t lo[kPer][3], hc[kPer][3];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t i = tid + k * kNodeThreads;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) lo[k][d] = hc[k][d] = 0xffffffffu;
+      if (i < n) {
+        const uint32_t e = (uint32_t)S.key[i] & 0xfffu;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          const uint32_t x = orderable(S.pos[d][e]);
+          lo[k][d] = x;
+          hc[k][d] = ~x;
+        }
+      }
+      const int width = cap < 32u ? (int)cap : 32;
+      for (int o = width >> 1; o > 0; o >>= 1) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          lo[k][d] = min(lo[k][d], __shfl_xor_sync(0xffffffffu, lo[k][d], o));
+          hc[k][d] = min(hc[k][d], __shfl_xor_sync(0xffffffffu, hc[k][d], o));
+        }
+      }
+      if (cap >= 32u && lane == 0 && i < n) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          atomicMin(&S.box[seg[k].id][d], lo[k][d]);
+          atomicMin(&S.box[seg[k].id][3 + d], hc[k][d]);
+        }
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t i = tid + k * kNodeThreads;
+      if (i >= n) continue;
+      if (cap >= 32u) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          lo[k][d] = S.box[seg[k].id][d];
+          hc[k][d] = S.box[seg[k].id][3 + d];
+        }
+      }
+      const float ex = from_orderable(~hc[k][0]) - from_orderable(lo[k][0]);
+      const float ey = from_orderable(~hc[k][1]) - from_orderable(lo[k][1]);
+      const float ez = from_orderable(~hc[k][2]) - from_orderable(lo[k][2]);
+      const int ax = (ex >= ey && ex >= ez) ? 0 : (ey >= ez ? 1 : 2);
+      const uint32_t e = (uint32_t)S.key[i] & 0xfffu;
+      S.key[i] = ((uint64_t)seg[k].id << 44) | ((uint64_t)orderable(S.pos[ax][e]) << 12) | e;
+    }
+    __syncthreads();
+    const uint32_t top = small ? cap : np;
+    for (uint32_t kk = 2; kk <= top; kk <<= 1) {
+      for (uint32_t jj = kk >> 1; jj > 0; jj >>= 1) {
+        for (uint32_t t = tid; t < np / 2; t += kNodeThreads) {
+          const uint32_t i = 2u * t - (t & (jj - 1u)), m = i + jj;
+          const bool up = kk == top || (i & kk) == 0u;
+          const uint64_t x = S.key[i], y = S.key[m];
+          if ((x > y) == up) {
+            S.key[i] = y;
+            S.key[m] = x;
+          }
+        }
+        __syncthreads();
+      }
+    }
+    const uint32_t leaf = l < levels2 ? (uint32_t)kTile2 : ((uint32_t)kTile >> (l - levels2));
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) descend(seg[k], tid + k * kNodeThreads, leaf);
+  }
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const uint32_t i = tid + k * kNodeThreads;
+    if (i < n) out[nd.start + i] = ord[nd.start + ((uint32_t)S.key[i] & 0xfffu)];
+  }
 }
 
-// One CTA of T threads per tile: centre, radius and tile-relative vectors.
-// The T = kTile2 build also writes the per-slot data shared by both tilings.
+// One CTA of T threads per tile: centre and tile-relative vectors, the discs
+// of its groups.  The T = kTile2 build also writes the per-slot data shared by
+// both tilings and the quarters' discs.  FP32 throughout: the unit vectors are
+// double-float, and the centre may be any point near the targets.
 template <int T>
 __global__ void __launch_bounds__(T) k_tile_build(
     const double* __restrict__ lon, const double* __restrict__ lat, int64_t P,
-    const uint32_t* __restrict__ order, float4* __restrict__ tile_chi,
-    float4* __restrict__ tile_clo, float4* __restrict__ tgt_a,
-    uint32_t* __restrict__ tgt_perm, float4* __restrict__ tgt_e, float4* __restrict__ tgt_n,
-    double2* __restrict__ tgt_ll, double4* __restrict__ sub64, float4* __restrict__ subf,
-    double4* __restrict__ grp64) {
-  __shared__ double red[3][T];
+    const uint32_t* __restrict__ order, const float4* __restrict__ u_hi,
+    const float4* __restrict__ u_lo, float4* __restrict__ tile_chi,
+    float4* __restrict__ tile_clo, float4* __restrict__ tgt_a, uint32_t* __restrict__ tgt_perm,
+    float4* __restrict__ tgt_e, float4* __restrict__ tgt_n, double2* __restrict__ tgt_ll,
+    float4* __restrict__ subf, float4* __restrict__ grp) {
+  __shared__ float red[3][T / 32];
   const int64_t tile = blockIdx.x;
-  const int j = threadIdx.x;
+  const int j = threadIdx.x, lane = j & 31;
   const int64_t s = tile * T + j;
   const bool valid = s < P;
-  double x = 0, y = 0, z = 0, lo = 0, la = 0;
+  float4 h = make_float4(0.f, 0.f, 0.f, 0.f), l = h;
   uint32_t u = 0xffffffffu;
   if (valid) {
     u = order[s];
-    lo = lon[u];
-    la = lat[u];
-    unit_vec(lo, la, x, y, z);
+    h = u_hi[u];
+    l = u_lo[u];
   }
-  red[0][j] = x;
-  red[1][j] = y;
-  red[2][j] = z;
-  __syncthreads();
-  for (int o = T / 2; o > 0; o >>= 1) {
-    if (j < o) {
-      red[0][j] += red[0][j + o];
-      red[1][j] += red[1][j + o];
-      red[2][j] += red[2][j + o];
+  auto warp_sum = [](float v, int width) {
+    for (int o = width >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  auto warp_max = [](float v, int width) {
+    for (int o = width >> 1; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+  };
+  {
+    const float sx = warp_sum(h.x, 32), sy = warp_sum(h.y, 32), sz = warp_sum(h.z, 32);
+    if (lane == 0) {
+      red[0][j >> 5] = sx;
+      red[1][j >> 5] = sy;
+      red[2][j >> 5] = sz;
     }
-    __syncthreads();
   }
-  double cx = red[0][0], cy = red[1][0], cz = red[2][0];
-  double nrm = sqrt(cx * cx + cy * cy + cz * cz);
   __syncthreads();
-  if (!(nrm > 1e-9)) {  // degenerate spread: use the first member
-    const uint32_t u0 = order[tile * T];
-    unit_vec(lon[u0], lat[u0], cx, cy, cz);
-    nrm = 1.0;
+  float cx = 0.f, cy = 0.f, cz = 0.f;
+#pragma unroll
+  for (int w = 0; w < T / 32; ++w) {
+    cx += red[0][w];
+    cy += red[1][w];
+    cz += red[2][w];
   }
-  cx /= nrm;
-  cy /= nrm;
-  cz /= nrm;
-  const double dx = x - cx, dy = y - cy, dz = z - cz;
-  double ang = 0.0;
-  if (valid) {
-    const double ch = sqrt(dx * dx + dy * dy + dz * dz);
-    ang = 2.0 * asin(fmin(1.0, 0.5 * ch));
+  const float nrm = sqrtf(cx * cx + cy * cy + cz * cz);
+  if (nrm > 1e-3f) {
+    cx /= nrm;
+    cy /= nrm;
+    cz /= nrm;
+  } else {  // targets all over the sphere: the first member
+    const float4 f = u_hi[order[tile * T]];
+    cx = f.x;
+    cy = f.y;
+    cz = f.z;
   }
-  red[0][j] = ang;
-  __syncthreads();
-  for (int o = T / 2; o > 0; o >>= 1) {
-    if (j < o) red[0][j] = fmax(red[0][j], red[0][j + o]);
-    __syncthreads();
-  }
-  const double radius = red[0][0] * (1.0 + 1e-9) + 1e-12;
+  const float dx = df_diff(h.x, l.x, cx, 0.f), dy = df_diff(h.y, l.y, cy, 0.f),
+              dz = df_diff(h.z, l.z, cz, 0.f);
   // an empty slot sits far outside every support radius
-  tgt_a[s] = valid ? make_float4((float)dx, (float)dy, (float)dz, 0.f)
-                   : make_float4(4.f, 4.f, 4.f, 0.f);
+  tgt_a[s] = valid ? make_float4(dx, dy, dz, 0.f) : make_float4(4.f, 4.f, 4.f, 0.f);
   if (tgt_perm) {
-    tgt_perm[s] = valid ? u : 0xffffffffu;
-    if (valid) {
-      double sl, cl, sb, cb;
-      sincos(lo * kDeg2Rad, &sl, &cl);
-      sincos(la * kDeg2Rad, &sb, &cb);
-      tgt_e[s] = make_float4((float)(-sl), (float)cl, 0.f, 0.f);
-      tgt_n[s] = make_float4((float)(-sb * cl), (float)(-sb * sl), (float)cb, 0.f);
+    tgt_perm[s] = u;
+    const double lo = valid ? lon[u] : 0.0, la = valid ? lat[u] : 0.0;
+    if (valid && valid_coord(lo, la)) {
+      df32 sb, cb, sl, cl;
+      sincos_deg(la, sb, cb);
+      sincos_deg(lo, sl, cl);
+      tgt_e[s] = make_float4(-sl.hi, cl.hi, 0.f, 0.f);
+      tgt_n[s] = make_float4(-sb.hi * cl.hi, -sb.hi * sl.hi, cb.hi, 0.f);
       tgt_ll[s] = make_double2(lo, la);
     } else {
       tgt_e[s] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -203,69 +389,39 @@ __global__ void __launch_bounds__(T) k_tile_build(
       tgt_ll[s] = make_double2(0.0, 0.0);
     }
   }
-  if (sub64) {
-    // 32-target quarters: warp-level centroid and radius (empty slots ignored)
-    double sx = x, sy = y, sz = z;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      sx += __shfl_xor_sync(0xffffffffu, sx, o);
-      sy += __shfl_xor_sync(0xffffffffu, sy, o);
-      sz += __shfl_xor_sync(0xffffffffu, sz, o);
-    }
-    double qn = sqrt(sx * sx + sy * sy + sz * sz);
-    if (!(qn > 1e-9)) {  // empty or degenerate quarter: use the tile centre
-      sx = cx; sy = cy; sz = cz; qn = 1.0;
-    }
-    sx /= qn; sy /= qn; sz /= qn;
-    double qa = 0.0;
-    if (valid) {
-      const double ex = x - sx, ey = y - sy, ez = z - sz;
-      qa = 2.0 * asin(fmin(1.0, 0.5 * sqrt(ex * ex + ey * ey + ez * ez)));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) qa = fmax(qa, __shfl_xor_sync(0xffffffffu, qa, o));
-    qa = qa * (1.0 + 1e-9) + 1e-12;
-    if ((j & 31) == 0) {
-      const int64_t qi = tile * (T / 32) + (j >> 5);
-      sub64[qi] = make_double4(sx, sy, sz, qa);
-      subf[qi] = make_float4((float)(sx - cx), (float)(sy - cy), (float)(sz - cz),
-                             (float)(2.0 * sin(0.5 * qa)));
-    }
+  if (subf) {
+    // 32-target quarters: mean and largest distance, relative to the tile
+    // centre (an empty quarter: the tile centre, radius 0)
+    const float m = warp_sum(valid ? 1.f : 0.f, 32);
+    const float inv = m > 0.f ? 1.f / m : 0.f;
+    const float qx = warp_sum(valid ? dx : 0.f, 32) * inv, qy = warp_sum(valid ? dy : 0.f, 32) * inv,
+                qz = warp_sum(valid ? dz : 0.f, 32) * inv;
+    const float ex = dx - qx, ey = dy - qy, ez = dz - qz;
+    const float r = warp_max(valid ? sqrtf(ex * ex + ey * ey + ez * ez) : 0.f, 32);
+    if (lane == 0) subf[tile * (T / 32) + (j >> 5)] = make_float4(qx, qy, qz, r * (1.f + 1e-6f) + 1e-12f);
   }
-  {
-    // 4-target groups (lanes 4 g .. 4 g + 3): centroid of the valid members
-    // and their largest angular distance from it; empty groups get radius -1
-    double gx = x, gy = y, gz = z;
-    int gv = valid ? 1 : 0;
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-      gx += __shfl_xor_sync(0xffffffffu, gx, o);
-      gy += __shfl_xor_sync(0xffffffffu, gy, o);
-      gz += __shfl_xor_sync(0xffffffffu, gz, o);
-      gv += __shfl_xor_sync(0xffffffffu, gv, o);
-    }
-    double gn = sqrt(gx * gx + gy * gy + gz * gz);
-    if (!(gn > 1e-9)) {  // degenerate spread: the tile centre (radius still covers)
-      gx = cx; gy = cy; gz = cz; gn = 1.0;
-    }
-    gx /= gn; gy /= gn; gz /= gn;
-    double ga = 0.0;
-    if (valid) {
-      const double ex = x - gx, ey = y - gy, ez = z - gz;
-      ga = 2.0 * asin(fmin(1.0, 0.5 * sqrt(ex * ex + ey * ey + ez * ez)));
-    }
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1) ga = fmax(ga, __shfl_xor_sync(0xffffffffu, ga, o));
-    ga = ga * (1.0 + 1e-9) + 1e-12;
-    if ((j & 3) == 0) grp64[tile * (T / 4) + (j >> 2)] = make_double4(gx, gy, gz, gv ? ga : -1.0);
+  // 4-target groups (lanes 4 g .. 4 g + 3): the direction of their mean and
+  // their largest angle from it, widened by the rounding; empty: radius -1
+  const float m = warp_sum(valid ? 1.f : 0.f, 4);
+  float gx = warp_sum(h.x, 4), gy = warp_sum(h.y, 4), gz = warp_sum(h.z, 4);
+  const float gn = sqrtf(gx * gx + gy * gy + gz * gz);
+  if (gn > 1e-3f) {
+    gx /= gn;
+    gy /= gn;
+    gz /= gn;
+  } else {  // degenerate spread: the tile centre (the radius still covers)
+    gx = cx;
+    gy = cy;
+    gz = cz;
   }
+  const float ex = h.x - gx, ey = h.y - gy, ez = h.z - gz;
+  const float ch = warp_max(valid ? sqrtf(ex * ex + ey * ey + ez * ez) : 0.f, 4);
+  if ((j & 3) == 0)
+    grp[tile * (T / 4) + (j >> 2)] = make_float4(
+        gx, gy, gz, m > 0.f ? 2.f * asinf(fminf(1.f, 0.5f * ch)) * (1.f + 1e-5f) + 1e-6f : -1.f);
   if (j == 0) {
-    float hx, lx, hy, ly, hz, lz;
-    split_f64(cx, hx, lx);
-    split_f64(cy, hy, ly);
-    split_f64(cz, hz, lz);
-    tile_chi[tile] = make_float4(hx, hy, hz, (float)radius);
-    tile_clo[tile] = make_float4(lx, ly, lz, 0.f);
+    tile_chi[tile] = make_float4(cx, cy, cz, 0.f);
+    tile_clo[tile] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 
@@ -290,9 +446,8 @@ static cudaError_t tiling_alloc(Tiling& t, int T, int64_t P, cudaStream_t s) {
   if ((e = dalloc(&t.clo, (size_t)t.n_tiles, s)) != cudaSuccess) return e;
   if ((e = dalloc(&t.a, (size_t)(t.n_tiles * T), s)) != cudaSuccess) return e;
   if ((e = dalloc(&t.tile_cand, (size_t)t.n_tiles, s)) != cudaSuccess) return e;
-  if ((e = dalloc(&t.grp64, (size_t)(t.n_tiles * (T / 4)), s)) != cudaSuccess) return e;
+  if ((e = dalloc(&t.grp, (size_t)(t.n_tiles * (T / 4)), s)) != cudaSuccess) return e;
   if (T == kTile2) {
-    if ((e = dalloc(&t.sub64, (size_t)(t.n_tiles * 4), s)) != cudaSuccess) return e;
     if ((e = dalloc(&t.subf, (size_t)(t.n_tiles * 4), s)) != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -313,77 +468,67 @@ cudaError_t targets_build(cg_grid* g, const double* lon, const double* lat) {
   if ((e = dalloc(&g->tgt_f2, slots, s)) != cudaSuccess) return e;
   if ((e = dalloc(&g->tgt_ll, slots, s)) != cudaSuccess) return e;
 
-  // k-d tree levels: leaves of kTile2 targets, then five more levels that split
-  // every leaf into kTile halves, 32-target quarters and on down to groups of 4
-  int levels2 = 0;
+  // levels to 128-target leaves; the first `top` of them over the whole array,
+  // until a node has at most kNodeCap targets
+  int levels2 = 0, top = 0;
   while (((int64_t)1 << levels2) < g->t128.n_tiles) ++levels2;
-  const int levels = levels2 + 5;
-  const int64_t max_nodes = (int64_t)1 << (levels + 1);
-  float4* pos = nullptr;
-  uint32_t *ord = nullptr, *nid = nullptr, *child = nullptr, *val = nullptr;
-  uint32_t *nstart = nullptr, *nend = nullptr, *bmin = nullptr, *bmax = nullptr;
-  uint64_t* key = nullptr;
+  while (((g->t128.n_tiles + ((int64_t)1 << top) - 1) >> top) * kTile2 > kNodeCap) ++top;
+  float4 *u_hi = nullptr, *u_lo = nullptr;
+  uint32_t *ord = nullptr, *key = nullptr, *val = nullptr, *box = nullptr;
   SortWork w;
-  e = dalloc(&pos, (size_t)P, s);
+  w.err = g->d_err;
+  e = dalloc(&u_hi, (size_t)P, s);
+  if (e == cudaSuccess) e = dalloc(&u_lo, (size_t)P, s);
   if (e == cudaSuccess) e = dalloc(&ord, (size_t)P, s);
-  if (e == cudaSuccess) e = dalloc(&nid, (size_t)P, s);
-  if (e == cudaSuccess) e = dalloc(&child, (size_t)P, s);
   if (e == cudaSuccess) e = dalloc(&val, (size_t)P, s);
-  if (e == cudaSuccess) e = dalloc(&key, (size_t)P, s);
-  if (e == cudaSuccess) e = dalloc(&nstart, (size_t)max_nodes, s);
-  if (e == cudaSuccess) e = dalloc(&nend, (size_t)max_nodes, s);
-  if (e == cudaSuccess) e = dalloc(&bmin, (size_t)(3 * max_nodes), s);
-  if (e == cudaSuccess) e = dalloc(&bmax, (size_t)(3 * max_nodes), s);
+  if (e == cudaSuccess && top > 0) e = dalloc(&key, (size_t)P, s);
+  if (e == cudaSuccess && top > 0) e = dalloc(&box, (size_t)6 << (top - 1), s);
   const unsigned nb = ceil_div(P, 256);
   if (e == cudaSuccess) {
-    k_target_init<<<nb, 256, 0, s>>>(lon, lat, P, pos, ord, nid, g->d_err);
+    k_target_init<<<nb, 256, 0, s>>>(lon, lat, P, u_hi, u_lo, ord, g->d_err);
     g->n_launches += 1;
   }
-  for (int l = 0; l < levels && e == cudaSuccess; ++l) {
-    const uint32_t leaf = (l < levels2) ? (uint32_t)kTile2 : ((uint32_t)kTile >> (l - levels2));
-    const int64_t nchild = (int64_t)1 << (l + 1);
-    e = cudaMemsetAsync(bmin, 0xff, sizeof(uint32_t) * (size_t)(3 * nchild), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(bmax, 0x00, sizeof(uint32_t) * (size_t)(3 * nchild), s);
+  uint32_t* cur = ord;   // the targets in the order reached so far
+  for (int l = 0; l < top && e == cudaSuccess; ++l) {
+    e = cudaMemsetAsync(box, 0xff, sizeof(uint32_t) * ((size_t)6 << l), s);
     if (e != cudaSuccess) break;
-    k_node_bounds<<<nb, 256, 0, s>>>(nid, P, nstart, nend);
-    k_node_split<<<nb, 256, 0, s>>>(nid, ord, pos, P, leaf, nstart, nend, child, bmin, bmax);
-    k_node_keys<<<nb, 256, 0, s>>>(child, ord, pos, P, bmin, bmax, key, val);
-    g->n_launches += 3;
-    uint64_t* sk = nullptr;
-    uint32_t* sv = nullptr;
-    const int bits = 32 + l + 1;
-    e = radix_sort_u64(key, val, P, bits, w, s, &sk, &sv);
-    g->n_launches += 3 * ((bits + 7) / 8);
-    if (e != cudaSuccess) break;
-    k_node_unpack<<<nb, 256, 0, s>>>(sk, P, nid);
-    g->n_launches += 1;
-    if (sv != ord) e = cudaMemcpyAsync(ord, sv, sizeof(uint32_t) * (size_t)P,
-                                       cudaMemcpyDeviceToDevice, s);
+    k_kd_box<<<ceil_div(P, 2048), 256, 0, s>>>(u_hi, cur, (uint32_t)P, l, box);
+    k_kd_keys<<<nb, 256, 0, s>>>(u_hi, cur, (uint32_t)P, l, box, key, val);
+    uint32_t* sk = nullptr;
+    const int bits = 16 + l;
+    e = radix_sort_u32(key, val, P, bits, w, s, &sk, &cur);
+    g->n_launches += 3 + (bits + 7) / 8;
   }
   if (e == cudaSuccess) {
-    k_tile_build<kTile2><<<(unsigned)g->t128.n_tiles, kTile2, 0, s>>>(
-        lon, lat, P, ord, g->t128.chi, g->t128.clo, g->t128.a, g->tgt_perm,
-        g->tgt_e, g->tgt_n, g->tgt_ll, g->t128.sub64, g->t128.subf, g->t128.grp64);
-    k_tile_build<kTile><<<(unsigned)g->t64.n_tiles, kTile, 0, s>>>(
-        lon, lat, P, ord, g->t64.chi, g->t64.clo, g->t64.a, nullptr, nullptr,
-        nullptr, nullptr, nullptr, nullptr, g->t64.grp64);
-    g->n_launches += 2;
-    e = cudaGetLastError();
+    // (`ord` is free unless nothing has been sorted: then val takes the result)
+    uint32_t* fin = cur == ord ? val : ord;
+    e = cudaFuncSetAttribute(k_kd_node, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(NodeSmem));
+    if (e == cudaSuccess) {
+      k_kd_node<<<1u << top, kNodeThreads, sizeof(NodeSmem), s>>>(u_hi, cur, (uint32_t)P, top,
+                                                                  levels2, fin);
+      k_tile_build<kTile2><<<(unsigned)g->t128.n_tiles, kTile2, 0, s>>>(
+          lon, lat, P, fin, u_hi, u_lo, g->t128.chi, g->t128.clo, g->t128.a, g->tgt_perm,
+          g->tgt_e, g->tgt_n, g->tgt_ll, g->t128.subf, g->t128.grp);
+      k_tile_build<kTile><<<(unsigned)g->t64.n_tiles, kTile, 0, s>>>(
+          lon, lat, P, fin, u_hi, u_lo, g->t64.chi, g->t64.clo, g->t64.a, nullptr, nullptr,
+          nullptr, nullptr, nullptr, g->t64.grp);
+      g->n_launches += 3;
+      e = cudaGetLastError();
+    }
   }
   if (w.keys_alt) cudaFreeAsync(w.keys_alt, s);
   dfree(w.vals_alt, s);
   dfree(w.hist, s);
   dfree(w.totals, s);
-  dfree(pos, s);
+  dfree(w.status, s);
+  dfree(w.os_meta, s);
+  dfree(u_hi, s);
+  dfree(u_lo, s);
   dfree(ord, s);
-  dfree(nid, s);
-  dfree(child, s);
   dfree(val, s);
   dfree(key, s);
-  dfree(nstart, s);
-  dfree(nend, s);
-  dfree(bmin, s);
-  dfree(bmax, s);
+  dfree(box, s);
   return e;
 }
 
