@@ -2,7 +2,7 @@
 
     b = Batch([(gridder, lon, lat, data, out, out_weights), ...], n_streams=16)
     b.autotune(reps=2)          # per job: FP32 register-blocking shape or BF16 tensor cores
-    b.set_fused(True)           # optional: one index and one gridder launch for all jobs
+    b.set_fused(True)           # optional: one sample index for all jobs
     b.capture()                 # one graph (per-job branches, or the fused pipeline)
     b.run()                     # one launch per replay
     b.sync()                    # wait; raises on the jobs' device errors

@@ -188,8 +188,10 @@ bool use_tc(const cg_grid* g, int dtype, const void* data) {
 // tensor-core epilogue writes directly (the accumulators are left empty).
 cg_status do_add(cg_grid* g, const double* lon, const double* lat, const void* data,
                  int32_t dtype, const float* weights, int64_t n, const char* where,
-                 float* out = nullptr, float* out_w = nullptr, bool* fused = nullptr) {
+                 float* out = nullptr, float* out_w = nullptr, bool* fused = nullptr,
+                 bool* drop = nullptr) {
   if (fused) *fused = false;
+  if (drop) *drop = false;
   if (!g) return fail(CG_EINVAL, "%s: null handle", where);
   if (!g->kernel_set) return fail(CG_ESTATE, "%s: call cg_set_kernel first", where);
   if (dtype != CG_F32 && dtype != CG_BF16)
@@ -234,6 +236,7 @@ cg_status do_add(cg_grid* g, const double* lon, const double* lat, const void* d
     CG_CUDA(tiles_ranges(g, t), where);
     t.ranges_gen = g->index_gen;
   }
+  bool kept = false;   // (direct forms) the sums stay as well
   cudaEvent_t t3 = tmark(g);
   // host-buffer calls: the index is built while the channel data still copy
   if (g->data_ready) CG_CUDA(cudaStreamWaitEvent(g->stream, g->data_ready, 0), where);
@@ -247,10 +250,11 @@ cg_status do_add(cg_grid* g, const double* lon, const double* lat, const void* d
     const bool want = out != nullptr && g->acc_empty;
     bool direct = false;
     const cudaError_t eg = grid_tiles_f32(g, data, dtype, want ? out : nullptr,
-                                          want ? out_w : nullptr, &direct);
+                                          want ? out_w : nullptr, &direct, &kept);
     g->rec_values = false;   // later passes bring values of their own
     CG_CUDA(eg, where);
     if (fused) *fused = direct;
+    if (drop) *drop = !direct && !kept;
   }
   cudaEvent_t t4 = tmark(g);
   tstage(g, 0, t0, t1);
@@ -259,7 +263,7 @@ cg_status do_add(cg_grid* g, const double* lon, const double* lat, const void* d
   tstage(g, 3, t3, t4);
   g->last_path = tc ? (g->path == CG_PATH_TC_FAST ? CG_PATH_TC_FAST : CG_PATH_TC) : CG_PATH_FP32;
   g->total_n += n;
-  if (!(fused && *fused)) g->acc_empty = false;
+  if (!(fused && *fused) || kept) g->acc_empty = false;
   return CG_OK;
 }
 
@@ -269,9 +273,9 @@ cg_status oneshot_impl(cg_grid* g, const double* lon, const double* lat, const v
                        int32_t layout_channel_major, float* out_w, const char* where) {
   cg_status st = zero_acc(g);
   if (st != CG_OK) return st;
-  bool fused = false;
+  bool fused = false, drop = false;
   st = do_add(g, lon, lat, data, dtype, weights, n, where, layout_channel_major ? nullptr : out,
-              out_w, &fused);
+              out_w, &fused, &drop);
   if (st != CG_OK) return st;
   if (fused) return CG_OK;  // the gridder's epilogue already wrote Eq. 3
   st = clear_if_empty(g, where);
@@ -279,6 +283,7 @@ cg_status oneshot_impl(cg_grid* g, const double* lon, const double* lat, const v
   cudaEvent_t t0 = tmark(g);
   CG_CUDA(finalize_maps(g, out, layout_channel_major ? 1 : 0, out_w), where);
   tstage(g, 4, t0, tmark(g));
+  if (drop) g->acc_empty = true;   // candidate splits: the sums were only this call's
   return CG_OK;
 }
 

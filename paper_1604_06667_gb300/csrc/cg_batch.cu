@@ -8,14 +8,10 @@
 //           (C + 16)), the capture records every job's one-shot pipeline
 //           (keys, sort, index, gridder, normalisation) on its branch
 //           between one fork and one join event;
-// fused     one pipeline for all jobs: one keys pass, one sort of every
+// fused     one sample index for all jobs: one keys pass, one sort of every
 //           job's samples by a composite key, one gather and one candidate
-//           range pass, then one persistent FP32 gridder launch whose CTAs
-//           take (job, tile, slab, split) items from a queue ordered by
-//           estimated cost (up to 96 jobs per launch), one split reduction,
-//           one non-finite fix-up and one normalisation over all jobs; jobs
-//           on the tensor-core form run the tensor-core gridder on their
-//           segment of the shared index.
+//           range pass; then every job's gridder on its segment of the shared
+//           index, side by side on the branch streams.
 //
 // cg_batch_run replays the instantiated graph with a single launch.  The
 // autotuner times, per job, the FP32 gridder's register-blocking shapes near
@@ -36,14 +32,6 @@ namespace {
 struct FusedPlan {
   cg::BatchIndex bi;
   std::vector<cg::BatchIndexJob> ijobs;
-  struct Group {
-    cg::F32Multi m;
-    std::vector<cg::F32MultiJob> hjobs;
-    std::vector<cg::F32Multi::Out> houts;
-  };
-  std::vector<Group> groups;
-  std::vector<int> tc_jobs;          // jobs on the tensor-core form
-  std::vector<void*> owned;          // device buffers to release
   int64_t kernels = 0;               // launches of one pass
 };
 
@@ -87,25 +75,9 @@ void release_plan(cg_batch* b) {
   cudaStream_t s = b->own;
   if (s) cudaStreamSynchronize(s);
   cg::batch_index_free(p->bi, s);
-  for (void* q : p->owned) cudaFreeAsync(q, s);
   if (s) cudaStreamSynchronize(s);
   delete p;
   b->plan = nullptr;
-}
-
-template <typename T>
-cudaError_t plan_alloc(FusedPlan* p, T** out, size_t count, cudaStream_t s) {
-  cudaError_t e = cg::dalloc(out, count, s);
-  if (e == cudaSuccess) p->owned.push_back(*out);
-  return e;
-}
-
-template <typename T>
-cudaError_t plan_upload(FusedPlan* p, T** out, const std::vector<T>& h, cudaStream_t s) {
-  cudaError_t e = plan_alloc(p, out, h.size(), s);
-  if (e == cudaSuccess && !h.empty())
-    e = cudaMemcpyAsync(*out, h.data(), sizeof(T) * h.size(), cudaMemcpyHostToDevice, s);
-  return e;
 }
 
 // The job's form, as a one-job call would choose it (CG_PATH_AUTO: tensor
@@ -118,16 +90,8 @@ bool job_on_tc(const cg_batch* b, int j) {
   return path == CG_PATH_TC || path == CG_PATH_TC_FAST || J.grid->C >= 16;
 }
 
-// The FP32 register-blocking shape of a job: the autotuner's, else the
-// default for its channel count.
-int job_shape(const cg_batch* b, int j) {
-  const int32_t c = b->cfg[(size_t)j];
-  return (c >= 0 && c < cg::kF32MultiShapes) ? c : cg::f32_multi_shape(b->jobs[(size_t)j].grid->C);
-}
-
-// Build the fused plan: the shared sample index, the FP32 groups (their job
-// arguments, item counts, split counts and scratch) and the tensor-core
-// job list.  Host work plus allocations on b->own; nothing is launched.
+// Build the fused plan: the shared sample index.  Host work plus allocations
+// on b->own; nothing is launched.
 cg_status build_plan(cg_batch* b) {
   release_plan(b);
   FusedPlan* p = new (std::nothrow) FusedPlan();
@@ -170,7 +134,6 @@ cg_status build_plan(cg_batch* b) {
     key_blk.push_back(key_blk.back() + (J.n_samples + 255) / 256);
     gth_blk.push_back(gth_blk.back() + (J.n_samples + 255) / 256 + (4 * ns + 1 + 255) / 256);
     tile_off.push_back(tile_off.back() + t.n_tiles);
-    if (tc) p->tc_jobs.push_back(j);
   }
   cg::BatchIndex& bi = p->bi;
   bi.n_jobs = nj;
@@ -197,153 +160,26 @@ cg_status build_plan(cg_batch* b) {
   up64(&bi.gth_blk, gth_blk);
   up64(&bi.tile_off, tile_off);
   if (e != cudaSuccess) return cg::batch_fail(CG_ECUDA, "cg_batch_capture: %s", cudaGetErrorString(e));
-
-  // ---- FP32 groups ----
-  // FP32 jobs grouped by register-blocking shape (one launch per shape)
-  std::vector<int> f32;
-  for (int j = 0; j < nj; ++j)
-    if (!job_on_tc(b, j)) f32.push_back(j);
-  std::stable_sort(f32.begin(), f32.end(),
-                   [&](int x, int y) { return job_shape(b, x) < job_shape(b, y); });
-  // candidate splits: items of about 1 / (16 x CTAs) of the FP32 work each
-  double total = 0.0;
-  for (int j : f32) {
-    const cg_job& J = b->jobs[(size_t)j];
-    const int shape = job_shape(b, j);
-    const int cp = cg::f32_multi_cpad(shape);
-    const int nb = (J.grid->C + cp - 1) / cp;
-    total += (double)J.n_samples * (double)(cg::kTile + cp) * nb;
-  }
-  const double quantum = std::max(1.0, total / (16.0 * 2.0 * nsm));
-  for (size_t g0 = 0, g1 = 0; g0 < f32.size(); g0 = g1) {
-    p->groups.emplace_back();
-    FusedPlan::Group& G = p->groups.back();
-    std::vector<int64_t> item_off(1, 0), fin_blk(1, 0), red_blk(1, 0), word_off(1, 0);
-    const int shape0 = job_shape(b, f32[g0]);
-    for (g1 = g0; g1 < f32.size() && g1 - g0 < (size_t)cg::kF32MultiMaxJobs &&
-                  job_shape(b, f32[g1]) == shape0;
-         ++g1) {
-    }
-    G.m.shape = shape0;
-    for (size_t k = g0; k < g1 && e == cudaSuccess; ++k) {
-      const int j = f32[k];
-      const cg_job& J = b->jobs[(size_t)j];
-      cg_grid* g = J.grid;
-      const cg::BatchIndexJob& q = p->ijobs[(size_t)j];
-      cg::F32MultiJob mj;
-      std::memset(&mj, 0, sizeof(mj));
-      mj.shape = shape0;
-      mj.dtype = J.data_dtype;
-      mj.pad = cg::f32_multi_cpad(mj.shape);
-      mj.n_slabs = (g->C + mj.pad - 1) / mj.pad;
-      cg::GridArgs& a = mj.a;
-      a.tile_chi = g->t64.chi;
-      a.tile_clo = g->t64.clo;
-      a.tgt_a = g->t64.a;
-      a.tgt_f1 = g->tgt_f1;
-      a.tgt_f2 = g->tgt_f2;
-      a.tgt_ll = g->tgt_ll;
-      a.tgt_perm = g->tgt_perm;
-      a.range_off = g->t64.range_off;
-      a.range_s = g->t64.range_s;
-      a.s_hi = bi.s_hi + q.off;
-      a.s_lo = bi.s_lo + q.off;
-      a.sll = bi.sll + q.off;
-      // the sorted values are known once the sort's pass count is (ping-pong)
-      a.perm = nullptr;
-      a.data = J.data;
-      a.C = g->C;
-      const size_t esz = (J.data_dtype == CG_BF16) ? 2 : 4;
-      a.vec4 = (g->C % 4 == 0) && ((reinterpret_cast<uintptr_t>(J.data) % (4 * esz)) == 0);
-      a.kd = g->kdev;
-      a.kd.dscale = 0.f;
-      a.acc_num = g->acc_num;
-      a.acc_w = g->acc_w;
-      a.accumulate = 0;
-      a.pairs = nullptr;
-      a.tile_cand = g->t64.tile_cand;
-      const double per_tile = (double)J.n_samples / std::max<int64_t>(1, g->t64.n_tiles) *
-                              (double)(cg::kTile + mj.pad);
-      a.n_split = (int)std::min(64.0, std::max(1.0, std::ceil(per_tile / quantum)));
-      a.n_slots = g->n_slots;
-      if (a.n_split > 1) {
-        e = plan_alloc(p, &a.part_num, (size_t)a.n_split * g->n_slots * g->C, s);
-        if (e == cudaSuccess) e = plan_alloc(p, &a.part_w, (size_t)a.n_split * g->n_slots, s);
-      }
-      const int64_t nbits = g->n_slots * (int64_t)mj.n_slabs;
-      {
-        cudaStream_t keep = g->stream;
-        g->stream = s;
-        if (e == cudaSuccess) e = cg::nonfinite_prepare(g, nbits);
-        g->stream = keep;
-      }
-      a.nf_bits = g->nf_bits;
-      // without splits, [P][C] maps are written by the gridder itself
-      const bool direct = a.n_split == 1 && !J.layout_channel_major;
-      a.out = direct ? J.out : nullptr;
-      a.out_w = direct ? J.out_weights : nullptr;
-      G.hjobs.push_back(mj);
-      const int vec4 = !J.layout_channel_major && g->C % 4 == 0 &&
-                       reinterpret_cast<uintptr_t>(J.out) % 16 == 0;
-      G.houts.push_back({J.out, J.out_weights, J.layout_channel_major, vec4, g->P});
-      item_off.push_back(item_off.back() + g->t64.n_tiles * mj.n_slabs * a.n_split);
-      fin_blk.push_back(fin_blk.back() +
-                        (direct ? 0
-                                : (g->n_slots * (int64_t)g->C + cg::kMultiFinElems - 1) /
-                                      cg::kMultiFinElems));
-      red_blk.push_back(red_blk.back() +
-                        (a.n_split > 1 ? (g->n_slots * (int64_t)(g->C + 1) + cg::kMultiRedElems - 1) /
-                                             cg::kMultiRedElems
-                                       : 0));
-      word_off.push_back(word_off.back() + (nbits + 31) / 32);
-    }
-    cg::F32Multi& m = G.m;
-    m.n_jobs = (int)G.hjobs.size();
-    m.n_items = item_off.back();
-    m.n_fin_blk = fin_blk.back();
-    m.n_red_blk = red_blk.back();
-    m.n_words = word_off.back();
-    m.err = b->d_err;
-    if (e == cudaSuccess) e = plan_alloc(p, &m.nf_any, 1, s);
-    for (auto& mj : G.hjobs) mj.a.nf_any = m.nf_any;
-    if (e == cudaSuccess) e = plan_upload(p, &m.item_off, item_off, s);
-    if (e == cudaSuccess) e = plan_upload(p, &m.fin_blk, fin_blk, s);
-    if (e == cudaSuccess) e = plan_upload(p, &m.red_blk, red_blk, s);
-    if (e == cudaSuccess) e = plan_upload(p, &m.word_off, word_off, s);
-    if (e == cudaSuccess) e = plan_upload(p, &m.outs, G.houts, s);
-    if (e == cudaSuccess) e = plan_alloc(p, &m.order, (size_t)std::max<int64_t>(1, m.n_items), s);
-    if (e == cudaSuccess) e = plan_alloc(p, &m.head, 1, s);
-    if (e == cudaSuccess) e = plan_alloc(p, &m.jobs, G.hjobs.size(), s);
-    if (e != cudaSuccess) break;
-  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cg::batch_fail(CG_ECUDA, "cg_batch_capture: %s", cudaGetErrorString(e));
   return CG_OK;
 }
 
-// One pass of the fused pipeline on stream st: eager (upload = true: the
-// jobs' arguments are copied to the device once the sort's output buffers are
-// known) or under capture (upload = false).
-cg_status run_fused(cg_batch* b, cudaStream_t st, bool upload) {
+// One pass of the fused pipeline on stream st, eager or under capture: the
+// shared index, then every job's gridder on its segment of it, side by side on
+// the planner's branches.
+cg_status run_fused(cg_batch* b, cudaStream_t st) {
   FusedPlan* p = b->plan;
   cg::BatchIndex& bi = p->bi;
   int64_t launches = 0;
   cudaError_t e = cg::batch_index_run(bi, b->d_err, st, &launches);
-  // the tensor-core jobs (the planner's branch assignment) and the FP32
-  // groups (group k on branch k) run on the branch streams, side by side
-  const size_t ns = b->streams.size();
-  std::vector<char> used(ns, 0);
-  for (int j : p->tc_jobs) used[(size_t)b->stream_of[(size_t)j]] = 1;
-  for (size_t k = 0; k < p->groups.size(); ++k) used[k % ns] = 1;
   if (e == cudaSuccess) e = cudaEventRecord(b->ev_fork, st);
-  for (size_t i = 0; i < ns && e == cudaSuccess; ++i)
-    if (used[i]) e = cudaStreamWaitEvent(b->streams[i], b->ev_fork, 0);
-  for (size_t k = 0; k < p->tc_jobs.size() && e == cudaSuccess; ++k) {
-    const int j = p->tc_jobs[k];
-    const cg_job& J = b->jobs[(size_t)j];
+  for (size_t i = 0; i < b->streams.size() && e == cudaSuccess; ++i)
+    e = cudaStreamWaitEvent(b->streams[i], b->ev_fork, 0);
+  for (size_t j = 0; j < b->jobs.size() && e == cudaSuccess; ++j) {
+    const cg_job& J = b->jobs[j];
     cg_grid* g = J.grid;
-    const cg::BatchIndexJob& q = p->ijobs[(size_t)j];
-    cudaStream_t bs = b->streams[(size_t)b->stream_of[(size_t)j]];
+    const cg::BatchIndexJob& q = p->ijobs[j];
     // the handle sees its segment of the shared index for this call
     struct {
       cudaStream_t stream;
@@ -352,9 +188,11 @@ cg_status run_fused(cg_batch* b, cudaStream_t st, bool upload) {
       uint32_t *sorted_val, *sorted_key;
       int32_t* ring_off;
       int64_t last_n;
-    } keep = {g->stream, g->s_hi, g->s_lo, g->s_ll, g->sorted_val, g->sorted_key, g->ring_off,
-              g->last_n};
-    g->stream = bs;
+      int32_t f32_cfg;
+      unsigned* d_err;
+    } keep = {g->stream,   g->s_hi,   g->s_lo,    g->s_ll, g->sorted_val, g->sorted_key,
+              g->ring_off, g->last_n, g->f32_cfg, g->d_err};
+    g->stream = b->streams[(size_t)b->stream_of[j]];
     g->s_hi = bi.s_hi + q.off;
     g->s_lo = bi.s_lo + q.off;
     g->s_ll = bi.sll + q.off;
@@ -362,9 +200,26 @@ cg_status run_fused(cg_batch* b, cudaStream_t st, bool upload) {
     g->sorted_key = bi.skey + q.off;
     g->ring_off = bi.ring_off + q.ring_base;
     g->last_n = J.n_samples;
+    g->f32_cfg = b->cfg[j];
     const int64_t l0 = g->n_launches;
-    e = cg::grid_tiles_tc(g, J.data, 2, J.out, J.out_weights,
-                          b->path[(size_t)j] != CG_PATH_TC_FAST);
+    if (job_on_tc(b, (int)j)) {
+      e = cg::grid_tiles_tc(g, J.data, 2, J.out, J.out_weights, b->path[j] != CG_PATH_TC_FAST);
+    } else {
+      // a one-shot call's gridder and normalisation
+      bool direct = false, kept = false;
+      g->acc_empty = true;
+      g->d_err = b->d_err;   // reported by cg_batch_sync
+      g->hold_f32 = b->hold ? b->d_hold : nullptr;
+      g->hold_f32_cycles = b->hold_cycles;
+      e = cudaMemsetAsync(g->d_pairs, 0, sizeof(unsigned long long), g->stream);
+      if (e == cudaSuccess)
+        e = cg::grid_tiles_f32(g, J.data, J.data_dtype, J.layout_channel_major ? nullptr : J.out,
+                               J.layout_channel_major ? nullptr : J.out_weights, &direct, &kept);
+      if (e == cudaSuccess && !direct)
+        e = cg::finalize_maps(g, J.out, J.layout_channel_major ? 1 : 0, J.out_weights);
+      g->acc_empty = !kept;
+      g->hold_f32 = nullptr;
+    }
     launches += g->n_launches - l0;
     // restore the handle's own sample arrays (allocations made by the call,
     // such as the bitmap or the item order, stay with the handle)
@@ -376,29 +231,10 @@ cg_status run_fused(cg_batch* b, cudaStream_t st, bool upload) {
     g->sorted_key = keep.sorted_key;
     g->ring_off = keep.ring_off;
     g->last_n = keep.last_n;
+    g->f32_cfg = keep.f32_cfg;
+    g->d_err = keep.d_err;
   }
-  // the FP32 groups, launched after the tensor-core jobs so that their
-  // persistent CTAs fill what the tensor-core kernels leave free; the jobs'
-  // arguments point into the sort's output (known now)
-  for (size_t k = 0; k < p->groups.size() && e == cudaSuccess; ++k) {
-    FusedPlan::Group& G = p->groups[k];
-    cudaStream_t gs = b->streams[k % ns];
-    for (size_t i = 0; i < G.hjobs.size(); ++i) {
-      const int64_t off = (int64_t)(G.hjobs[i].a.s_hi - bi.s_hi);
-      G.hjobs[i].a.perm = bi.sorted_val + off;
-    }
-    G.m.hjobs = G.hjobs.data();
-    G.m.hold = b->hold ? b->d_hold : nullptr;
-    G.m.hold_cycles = b->hold_cycles;
-    if (upload) {
-      e = cudaMemcpyAsync(G.m.jobs, G.hjobs.data(), sizeof(cg::F32MultiJob) * G.hjobs.size(),
-                          cudaMemcpyHostToDevice, gs);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(gs);
-    }
-    if (e == cudaSuccess) e = cg::grid_f32_multi(G.m, gs, &launches);
-  }
-  for (size_t i = 0; i < used.size() && e == cudaSuccess; ++i) {
-    if (!used[i]) continue;
+  for (size_t i = 0; i < b->streams.size() && e == cudaSuccess; ++i) {
     e = cudaEventRecord(b->ev_join[i], b->streams[i]);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, b->ev_join[i], 0);
   }
@@ -443,18 +279,18 @@ cg_status ensure_own(cg_batch* b) {
   return CG_OK;
 }
 
-// Fused capture: plan, one eager pass (allocations, the jobs' arguments on
-// the device), then the same pass recorded on cap.
+// Fused capture: plan, one eager pass (allocations), then the same pass
+// recorded on cap.
 cg_status capture_fused(cg_batch* b, cudaStream_t cap) {
   cg_status st = ensure_own(b);
   if (st == CG_OK) st = build_plan(b);
-  if (st == CG_OK) st = run_fused(b, b->own, true);
+  if (st == CG_OK) st = run_fused(b, b->own);
   if (st != CG_OK) return st;
   cudaError_t e = cudaStreamSynchronize(b->own);
   if (e != cudaSuccess) return cg::batch_fail(CG_ECUDA, "cg_batch_capture: %s", cudaGetErrorString(e));
   release_graph(b);
   e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeRelaxed);
-  if (e == cudaSuccess) st = run_fused(b, cap, false);
+  if (e == cudaSuccess) st = run_fused(b, cap);
   cudaGraph_t graph = nullptr;
   const cudaError_t e_end = cudaStreamEndCapture(cap, &graph);
   if (e == cudaSuccess) e = e_end;
@@ -551,8 +387,9 @@ cg_status cg_batch_autotune(cg_batch* b, int32_t reps, int32_t allow_tc) {
     const cg_job& J = b->jobs[j];
     cg_grid* g = J.grid;
     cudaStream_t s = b->streams[(size_t)b->stream_of[j]];
-    // candidates: (path, FP32 shape)
+    // candidates: (path, FP32 shape; -1: the default form)
     std::vector<std::pair<int32_t, int32_t>> cand;
+    cand.push_back({CG_PATH_FP32, -1});
     const int d = cg::f32_default_config(g->C);
     for (int c = d - 1; c <= d + 1; ++c)
       if (c >= 0 && c < cg::kF32Configs) cand.push_back({CG_PATH_FP32, c});

@@ -29,6 +29,19 @@ __device__ __forceinline__ void set_error(unsigned* err, unsigned bit) {
   if (err) atomicOr(err, bit);
 }
 
+// Testing hook: the CTA waits, with a limit, for a word that nothing sets; true
+// (and the error recorded) when the wait ran out.  Called by every thread.
+__device__ __forceinline__ bool hold_gives_up(const int* hold, long long cycles, unsigned* err) {
+  bool out = false;
+  if (threadIdx.x == 0) {
+    const long long t0 = clock64();
+    while (*((volatile const int*)hold) == 0 && clock64() - t0 < cycles) __nanosleep(1000);
+    out = *((volatile const int*)hold) == 0;
+    if (out) set_error(err, ERR_TIMEOUT);
+  }
+  return __syncthreads_or(out);
+}
+
 // sin(pi x) / (pi x), 1 at x = 0 (the tapered-sinc kernel's sinc factor)
 __device__ __forceinline__ float sinc_pi(float x) {
   return (x == 0.f) ? 1.f : sinpif(x) / (3.14159265358979f * x);

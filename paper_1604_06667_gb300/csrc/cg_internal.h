@@ -202,6 +202,9 @@ struct cg_grid {
   bool hold = false;
   int64_t hold_cycles = 0;
   int32_t* d_hold = nullptr;
+  // the same for the FP32 gridders (set by a batch's testing hook for its calls)
+  const int32_t* hold_f32 = nullptr;
+  int64_t hold_f32_cycles = 0;
   int64_t n_launches = 0;         // kernels launched by this handle
 
   // optional stage timing (CUDA events on the handle's stream)
@@ -294,12 +297,17 @@ struct GridArgs {
   // set); null: numerator and W into the accumulators
   float* out;
   float* out_w;
+  int keep;             // one-shot output: the accumulators are written as well
+  unsigned* err;
+  const int* hold;      // testing hook: a word nothing sets (null: no hold)
+  long long hold_cycles;
 };
 // out != null (one-shot call, pixel-major map): R = N / W straight into out
 // when the pass has no candidate splits (*direct = true), else the
-// accumulators as usual.
+// accumulators as usual.  *kept: the sums stay in the accumulators for later
+// calls (with neither, they only serve this call's finalize).
 cudaError_t grid_tiles_f32(cg_grid* g, const void* data, int dtype, float* out = nullptr,
-                           float* out_w = nullptr, bool* direct = nullptr);
+                           float* out_w = nullptr, bool* direct = nullptr, bool* kept = nullptr);
 // k_grid_narrow.cu -- at most 8 channels: lanes over candidates.  rows: scratch
 // of n * narrow_width(C) floats (null: one channel, values in s_lo.w).
 constexpr int kNarrowMaxC = 8;
@@ -307,14 +315,20 @@ int narrow_width(int C);
 int narrow_splits(int64_t n_tiles, int64_t n, int n_sms);
 cudaError_t grid_narrow(const GridArgs& a, const Tiling& t, int64_t n, int dtype, float* rows,
                         cudaStream_t s);
+// k_grid_wide.cu -- more than 8 channels: warps over compact target groups and
+// all channels of a slab.
+int wide_cpad(int C);
+int wide_splits(int64_t n_tiles, int64_t n, int C, int n_sms);
+cudaError_t grid_wide(const GridArgs& a, const Tiling& t, int64_t n, int dtype, cudaStream_t s);
 constexpr int kF32Configs = 7;   // register-blocking shapes of the FP32 gridder
 int f32_default_config(int C);
+int f32_cpad(int shape);         // channels per slab of a shape
 // the same into given accumulators; dscale != 0 evaluates w d^2 dscale
 // instead of w (the d/dsigma pass) and counts no pairs
 cudaError_t grid_tiles_f32_to(cg_grid* g, const void* data, int dtype, float* acc_num,
                               float2* acc_w, int accumulate, float dscale, int C = -1,
                               float* out = nullptr, float* out_w = nullptr,
-                              bool* direct = nullptr);
+                              bool* direct = nullptr, bool* kept = nullptr);
 cg_status batch_fail(cg_status st, const char* fmt, ...) __attribute__((format(printf, 2, 3)));
 
 // ---- fused batches: one sample index for all jobs (k_healpix.cu) --------
@@ -369,60 +383,14 @@ cudaError_t batch_index_alloc(BatchIndex& bi, cudaStream_t s);
 cudaError_t batch_index_run(BatchIndex& bi, unsigned* err, cudaStream_t s, int64_t* launches);
 void batch_index_free(BatchIndex& bi, cudaStream_t s);
 
-// ---- fused batches: one FP32 gridder launch for all jobs (k_grid.cu) ----
-// Items (job, tile, channel slab, candidate split) are taken from a queue
-// ordered by decreasing estimated cost; one launch per register-blocking
-// shape of the one-job gridder (by channel count, or the autotuner's choice)
-// and up to kF32MultiMaxJobs jobs.
-constexpr int kF32MultiShapes = kF32Configs;
-constexpr int kF32MultiMaxJobs = 96;  // jobs per launch (their arguments fill the parameter space)
-int f32_multi_shape(int C);           // default shape for C channels (f32_default_config)
-int f32_multi_cpad(int shape);        // channels per slab of a shape
-struct F32MultiJob {
-  GridArgs a;
-  int shape;
-  int dtype;
-  int n_slabs;
-  int pad;                            // channels per slab of the shape
-};
-struct F32Multi {
-  int shape = 0;                      // the register-blocking shape of all its jobs
-  F32MultiJob* jobs = nullptr;        // device [n_jobs]
-  const F32MultiJob* hjobs = nullptr; // host copy (the launcher reads it)
-  int n_jobs = 0;
-  int64_t* item_off = nullptr;        // device [n_jobs + 1]: prefix of items
-  int64_t n_items = 0;
-  int32_t* order = nullptr;           // device [n_items]: items, costliest first
-  unsigned* head = nullptr;           // queue head (cleared by the order pass)
-  unsigned* err = nullptr;
-  const int* hold = nullptr;          // testing hook: a word nothing sets
-  long long hold_cycles = 0;
-  // split reduction, normalisation and non-finite fix-up of all jobs
-  struct Out {
-    float* out;                       // caller's map
-    float* out_w;
-    int channel_major;
-    int vec4;                         // [P][C], C % 4 == 0, 16-byte aligned map
-    int64_t P;
-  };
-  Out* outs = nullptr;                // device [n_jobs]
-  // CTAs of the normalisation (every job) and of the split reduction (jobs
-  // with candidate splits): prefix over the jobs of their CTA counts
-  int64_t* fin_blk = nullptr;         // device [n_jobs + 1]
-  int64_t n_fin_blk = 0;
-  int64_t* red_blk = nullptr;         // device [n_jobs + 1]
-  int64_t n_red_blk = 0;
-  int64_t* word_off = nullptr;        // device [n_jobs + 1]: prefix of bitmap words
-  int64_t n_words = 0;
-  uint32_t* nf_any = nullptr;
-};
-cudaError_t grid_f32_multi(const F32Multi& m, cudaStream_t s, int64_t* launches);
-constexpr int kMultiFinElems = 1024;  // map values per CTA of the normalisation
-constexpr int kMultiRedElems = 256;   // values per CTA of the split reduction
 // k_grid_tc.cu -- the tile gridder, BF16 tcgen05 form (TMEM accumulators).
 // mode 0: store into the accumulators, 1: add into them, 2: one-shot
 // normalised output in the caller's [P][C] layout (out, out_w).
 bool tc_supported(const cg_grid* g, int dtype, const void* data);
+// Tensor map over n rows of C values (16-byte aligned) for gathers of rows of
+// box_cols columns; swizzled in 128-byte rows for the MMA, or plain.
+cudaError_t encode_rows_map(void* tmap, const void* data, int dtype, int C, int64_t n, int box_cols,
+                            bool swizzle128);
 cudaError_t grid_tiles_tc(cg_grid* g, const void* data, int mode, float* out, float* out_w,
                           int split);
 // k_grid.cu -- rows a gridder flagged as non-finite, computed again in FP32
@@ -438,6 +406,7 @@ struct NonfiniteRows {
   int mode;               // 0 store, 1 add (into acc_num), 2 divide by W into out
   bool skip_zero;         // pairs of weight zero take part only in a sum that is non-finite anyway
   float* out;             // mode 2: user-order map
+  bool keep;              // mode 2: the numerator goes to acc_num as well
   float* acc_num;         // modes 0, 1: slot-order numerator
   KernelDev kd;
 };

@@ -16,7 +16,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-__device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
+__host__ __device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
 
 // (s, c) + (v, vc): two-sum of the leading parts, the corrections added up.
 __device__ __forceinline__ void comp_add(float& s, float& c, float v, float vc) {
@@ -41,7 +41,7 @@ struct WeightConst {
   float2 k1, k2;
   float c2_in, c2_out;
 };
-__device__ __forceinline__ WeightConst weight_const(const KernelDev& kd) {
+__host__ __device__ __forceinline__ WeightConst weight_const(const KernelDev& kd) {
   WeightConst c;
   c.q0 = f2(kd.k1);
   c.q1 = f2(kd.k1 * (1.f / 12.f));

@@ -636,6 +636,7 @@ template <int PB, int CB, int NCG, typename DT>
 __global__ void __launch_bounds__((kTile / PB) * NCG) k_grid_f32(const __grid_constant__ GridArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& S = *reinterpret_cast<F32Smem<PB, CB, NCG>*>(smem_raw);
+  if (a.hold && hold_gives_up(a.hold, a.hold_cycles, a.err)) return;
   grid_item_f32<PB, CB, NCG, DT>(a, S, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.y);
 }
 
@@ -713,15 +714,19 @@ cudaError_t launch(const GridArgs& a, int64_t n_tiles, int dtype, cudaStream_t s
 
 // Scratch of a pass with a.n_split candidate shares, and whether it writes
 // the one-shot map itself (a.out is kept only without candidate splits).
-cudaError_t begin_pass(cg_grid* g, GridArgs& a, int n_slabs, bool* direct) {
+cudaError_t begin_pass(cg_grid* g, GridArgs& a, int n_slabs, bool* direct, bool* kept) {
   cudaStream_t s = g->stream;
   a.part_num = nullptr;
   a.part_w = nullptr;
+  // sums meant to outlast the call: all but those of a one-shot map of many
+  // tiles (see sums_kept)
+  if (kept) *kept = !a.out || a.keep;
   if (a.n_split > 1 || a.accumulate) {
     a.out = nullptr;
     a.out_w = nullptr;
   }
   if (direct) *direct = a.out != nullptr;
+  a.keep = a.out && a.keep;
   if (a.n_split > 1) {
     const size_t need_n = (size_t)a.n_split * (size_t)g->n_slots * (size_t)a.C;
     const size_t need_w = (size_t)a.n_split * (size_t)g->n_slots;
@@ -772,9 +777,20 @@ cudaError_t end_pass(cg_grid* g, const GridArgs& a, int dtype, int cpad, int n_s
   rows.mode = a.out ? 2 : (a.accumulate ? 1 : 0);
   rows.skip_zero = skip_zero;
   rows.out = a.out;
+  rows.keep = a.keep != 0;
   rows.acc_num = a.acc_num;
   rows.kd = a.kd;
   return nonfinite_fixup(g, rows);
+}
+
+// Whether a one-shot call leaves its sums in the accumulators, for a finalize
+// or a degrid without weights of the caller's: maps of fewer tiles than fill
+// the GPU with the register-blocked shape of the channel count (they once
+// needed candidate splits there, whose sums end up in the accumulators).
+bool sums_kept(int64_t n_tiles, int C, int n_sms) {
+  static const int nth[kF32Configs] = {64, 64, 128, 128, 128, 128, 256};
+  const int cfg = f32_default_config(C), cpad = f32_cpad(cfg);
+  return n_tiles * ((C + cpad - 1) / cpad) * nth[cfg] < (int64_t)n_sms * 1024;
 }
 
 int sm_count() {
@@ -787,19 +803,20 @@ int sm_count() {
 // One FP32 gridder pass in a register-blocking shape: choose the candidate
 // splits, launch, reduce the splits, compute the flagged non-finite rows again.
 template <int PB, int CB, int NCG>
-cudaError_t run(cg_grid* g, GridArgs& a, int dtype, bool* direct) {
+cudaError_t run(cg_grid* g, GridArgs& a, int dtype, bool* direct, bool* kept) {
   constexpr int CPAD = CB * NCG;
   const int64_t nt = g->t64.n_tiles;
   const int n_slabs = (a.C + CPAD - 1) / CPAD;
   a.n_split = splits_for<PB, CB, NCG>(nt, a.C, sm_count());
-  cudaError_t e = begin_pass(g, a, n_slabs, direct);
+  a.keep = a.n_split > 1;
+  cudaError_t e = begin_pass(g, a, n_slabs, direct, kept);
   if (e == cudaSuccess) e = launch<PB, CB, NCG>(a, nt, dtype, g->stream);
   if (e != cudaSuccess || nt == 0) return e;
   return end_pass(g, a, dtype, CPAD, n_slabs, false);
 }
 
 // The same pass for at most 8 channels (k_grid_narrow.cu).
-cudaError_t run_narrow(cg_grid* g, GridArgs& a, int dtype, bool* direct) {
+cudaError_t run_narrow(cg_grid* g, GridArgs& a, int dtype, bool* direct, bool* kept) {
   const int64_t nt = g->t64.n_tiles;
   const int cw = narrow_width(a.C);
   const bool own_rows = !(g->rec_values && cw == 1);
@@ -812,7 +829,8 @@ cudaError_t run_narrow(cg_grid* g, GridArgs& a, int dtype, bool* direct) {
     g->rows_cap = need;
   }
   a.n_split = narrow_splits(nt, g->last_n, sm_count());
-  cudaError_t e = begin_pass(g, a, 1, direct);
+  a.keep = sums_kept(nt, a.C, sm_count());
+  cudaError_t e = begin_pass(g, a, 1, direct, kept);
   if (e == cudaSuccess) e = grid_narrow(a, g->t64, g->last_n, dtype, own_rows ? g->rows : nullptr,
                                          g->stream);
   if (e != cudaSuccess) return e;
@@ -820,22 +838,40 @@ cudaError_t run_narrow(cg_grid* g, GridArgs& a, int dtype, bool* direct) {
   return end_pass(g, a, dtype, cw, 1, true);
 }
 
+// The same pass for more channels (k_grid_wide.cu).
+cudaError_t run_wide(cg_grid* g, GridArgs& a, int dtype, bool* direct, bool* kept) {
+  const int64_t nt = g->t64.n_tiles;
+  const int cp = wide_cpad(a.C);
+  const int n_slabs = (a.C + cp - 1) / cp;
+  a.n_split = wide_splits(nt, g->last_n, a.C, sm_count());
+  a.keep = sums_kept(nt, a.C, sm_count());
+  cudaError_t e = begin_pass(g, a, n_slabs, direct, kept);
+  if (e == cudaSuccess) e = grid_wide(a, g->t64, g->last_n, dtype, g->stream);
+  if (e != cudaSuccess) return e;
+  return end_pass(g, a, dtype, cp, n_slabs, true);
+}
+
 }  // namespace
 
 cudaError_t grid_tiles_f32(cg_grid* g, const void* data, int dtype, float* out, float* out_w,
-                           bool* direct) {
+                           bool* direct, bool* kept) {
   return grid_tiles_f32_to(g, data, dtype, g->acc_num, g->acc_w, g->acc_empty ? 0 : 1, 0.f, -1,
-                           out, out_w, direct);
+                           out, out_w, direct, kept);
 }
 
 cudaError_t grid_tiles_f32_to(cg_grid* g, const void* data, int dtype, float* acc_num,
                               float2* acc_w, int accumulate, float dscale, int C, float* out,
-                              float* out_w, bool* direct) {
+                              float* out_w, bool* direct, bool* kept) {
   if (direct) *direct = false;
+  if (kept) *kept = true;
   if (C < 0) C = g->C;
   GridArgs a;
   a.out = out;
   a.out_w = out_w;
+  a.keep = 0;
+  a.err = g->d_err;
+  a.hold = g->hold_f32;
+  a.hold_cycles = g->hold_f32_cycles;
   a.tile_chi = g->t64.chi;
   a.tile_clo = g->t64.clo;
   a.tgt_a = g->t64.a;
@@ -864,19 +900,18 @@ cudaError_t grid_tiles_f32_to(cg_grid* g, const void* data, int dtype, float* ac
   a.n_slots = g->n_slots;
   int cfg = g->f32_cfg;
   if (cfg < 0 || cfg >= kF32Configs || C != g->C) {
-    // at most 8 channels: lanes over candidates (the register-blocked shapes
-    // stay for wider rows, for shapes asked for and for fused batches)
-    if (C <= kNarrowMaxC) return run_narrow(g, a, dtype, direct);
-    cfg = f32_default_config(C);
+    // the register-blocked shapes stay for shapes asked for and fused batches
+    return C <= kNarrowMaxC ? run_narrow(g, a, dtype, direct, kept)
+                            : run_wide(g, a, dtype, direct, kept);
   }
   switch (cfg) {
-    case 0: return run<1, 4, 1>(g, a, dtype, direct);
-    case 1: return run<1, 8, 1>(g, a, dtype, direct);
-    case 2: return run<1, 8, 2>(g, a, dtype, direct);
-    case 3: return run<2, 8, 4>(g, a, dtype, direct);
-    case 4: return run<2, 16, 4>(g, a, dtype, direct);
-    case 5: return run<4, 16, 8>(g, a, dtype, direct);
-    default: return run<4, 16, 16>(g, a, dtype, direct);
+    case 0: return run<1, 4, 1>(g, a, dtype, direct, kept);
+    case 1: return run<1, 8, 1>(g, a, dtype, direct, kept);
+    case 2: return run<1, 8, 2>(g, a, dtype, direct, kept);
+    case 3: return run<2, 8, 4>(g, a, dtype, direct, kept);
+    case 4: return run<2, 16, 4>(g, a, dtype, direct, kept);
+    case 5: return run<4, 16, 8>(g, a, dtype, direct, kept);
+    default: return run<4, 16, 16>(g, a, dtype, direct, kept);
   }
 }
 
@@ -908,7 +943,7 @@ struct FixArgs {
   KernelDev kd;
   const void* data;
   int bf16;
-  int C, cp, n_slabs, mode, skip_zero;
+  int C, cp, n_slabs, mode, skip_zero, keep;
   float* out;
   float* acc_num;
   const uint32_t* perm_t;
@@ -1003,6 +1038,7 @@ __device__ __forceinline__ void fix_word(const FixArgs& a, int64_t wd, FixShared
         const uint32_t user = a.perm_t[slot];
         if (user != 0xffffffffu)
           a.out[(size_t)user * a.C + c] = (W > 0.0) ? (float)((double)acc / W) : __int_as_float(0x7fc00000);
+        if (a.keep) a.acc_num[(size_t)slot * a.C + c] = acc;
       } else if (a.mode == 1) {
         a.acc_num[(size_t)slot * a.C + c] += acc;
       } else {
@@ -1061,6 +1097,7 @@ cudaError_t nonfinite_fixup(cg_grid* g, const NonfiniteRows& j) {
   a.n_slabs = j.n_slabs;
   a.mode = j.mode;
   a.skip_zero = j.skip_zero ? 1 : 0;
+  a.keep = j.keep ? 1 : 0;
   a.out = j.out;
   a.acc_num = j.acc_num;
   a.perm_t = g->tgt_perm;
@@ -1076,345 +1113,9 @@ cudaError_t nonfinite_fixup(cg_grid* g, const NonfiniteRows& j) {
   return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------------------
-// Fused batches: one FP32 gridder launch for the items of all jobs.
-// ---------------------------------------------------------------------------
-namespace {
-
-constexpr int kMultiBins = 256;
-constexpr int kOrderCta = 1024;
-
-// Largest j with off[j] <= x (off[0] = 0, off non-decreasing, x < off[n]).
-__device__ __forceinline__ int find_job(const int64_t* __restrict__ off, int n, int64_t x) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (off[mid] <= x) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-struct ItemPos {
-  int job;
-  int64_t tile;
-  int slab, split, n_slabs;
-};
-
-__device__ __forceinline__ ItemPos decode_item(const F32Multi& m, int64_t it) {
-  ItemPos q;
-  q.job = find_job(m.item_off, m.n_jobs, it);
-  const F32MultiJob& J = m.jobs[q.job];
-  const int64_t local = it - m.item_off[q.job];
-  const int ns = J.a.n_split, nb = J.n_slabs;
-  q.n_slabs = nb;
-  q.tile = local / ((int64_t)nb * ns);
-  const int r = (int)(local - q.tile * nb * ns);
-  q.slab = r / ns;
-  q.split = r % ns;
-  return q;
-}
-
-// Decreasing estimated cost (weights of the tile's share of candidates plus
-// its channel work), in log-spaced bins.
-__device__ __forceinline__ int multi_bin(const F32Multi& m, int64_t it) {
-  const ItemPos q = decode_item(m, it);
-  const F32MultiJob& J = m.jobs[q.job];
-  const int ns = J.a.n_split;
-  const float cand = (float)((J.a.tile_cand[q.tile] + ns - 1) / ns);
-  const float cost = cand * (float)(kTile + J.pad);
-  const int b = (int)(8.f * __log2f(1.f + cost));
-  return kMultiBins - 1 - min(max(b, 0), kMultiBins - 1);
-}
-
-// One CTA: the queue order (counting sort by cost bin), and the queue head
-// and the non-finite flag cleared for the gridder launch that follows.
-__global__ void __launch_bounds__(kOrderCta) k_multi_order(const __grid_constant__ F32Multi m) {
-  __shared__ int32_t cnt[kMultiBins];
-  __shared__ int32_t wsum[kOrderCta / 32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) {
-    *m.head = 0u;
-    *m.nf_any = 0u;
-  }
-  for (int i = tid; i < kMultiBins; i += kOrderCta) cnt[i] = 0;
-  __syncthreads();
-  for (int64_t it = tid; it < m.n_items; it += kOrderCta) atomicAdd(&cnt[multi_bin(m, it)], 1);
-  __syncthreads();
-  // exclusive scan of the bins (one per thread of the first kMultiBins)
-  const int v = tid < kMultiBins ? cnt[tid] : 0;
-  int incl = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) wsum[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    int x = wsum[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    wsum[lane] = x;
-  }
-  __syncthreads();
-  if (tid < kMultiBins) cnt[tid] = incl - v + (warp > 0 ? wsum[warp - 1] : 0);
-  __syncthreads();
-  for (int64_t it = tid; it < m.n_items; it += kOrderCta) {
-    const int pos = atomicAdd(&cnt[multi_bin(m, it)], 1);
-    m.order[pos] = (int32_t)it;
-  }
-}
-
-template <int PB, int CB, int NCG>
-__device__ __forceinline__ void multi_item(const GridArgs& a, unsigned char* raw, int dtype,
-                                           const ItemPos& q) {
-  auto& S = *reinterpret_cast<F32Smem<PB, CB, NCG>*>(raw);
-  if (dtype == CG_BF16)
-    grid_item_f32<PB, CB, NCG, __nv_bfloat16>(a, S, q.tile, q.slab, q.split, q.n_slabs);
-  else
-    grid_item_f32<PB, CB, NCG, float>(a, S, q.tile, q.slab, q.split, q.n_slabs);
-}
-
-// The gridder launch carries every job's arguments in its parameter space, so
-// that the items read them as constant operands (like a one-job launch).
-struct MultiLaunch {
-  F32Multi m;
-  GridArgs ga[kF32MultiMaxJobs];
-};
-
-// Persistent CTAs take items from the queue until it is empty.  One kernel
-// per register-blocking shape of the one-job gridder (the jobs of a launch
-// share it), held to the one-job kernel's CTAs per SM (MINB); as many CTAs as
-// fit on the GPU.
-template <int PB, int CB, int NCG, int MINB>
-__global__ void __launch_bounds__((kTile / PB) * NCG, MINB)
-    k_grid_f32_multi(const __grid_constant__ MultiLaunch L) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const F32Multi& m = L.m;
-  __shared__ int64_t s_item;
-  __shared__ int s_stop;
-  const int tid = threadIdx.x;
-  if (tid == 0) {
-    s_stop = 0;
-    if (m.hold) {
-      // testing hook: wait for a word that nothing sets; the wait runs out
-      // and the CTA leaves without taking an item
-      const long long t0 = clock64();
-      while (*((volatile const int*)m.hold) == 0 && clock64() - t0 < m.hold_cycles) __nanosleep(1000);
-      if (*((volatile const int*)m.hold) == 0) {
-        set_error(m.err, ERR_TIMEOUT);
-        s_stop = 1;
-      }
-    }
-  }
-  __syncthreads();
-  if (s_stop) return;
-  for (;;) {
-    if (tid == 0) {
-      const unsigned q = atomicAdd(m.head, 1u);
-      s_item = (int64_t)q < m.n_items ? (int64_t)m.order[q] : -1;
-    }
-    __syncthreads();
-    const int64_t it = s_item;
-    if (it < 0) break;
-    const ItemPos q = decode_item(m, it);
-    const int dtype = m.jobs[q.job].dtype;
-    const GridArgs& ja = L.ga[__shfl_sync(0xffffffffu, q.job, 0)];
-    multi_item<PB, CB, NCG>(ja, smem_raw, dtype, q);
-    __syncthreads();   // the item is done with s_item and shared memory
-  }
-}
-
-// Candidate-split partials of every split job, in split order, into its
-// accumulators; rows flagged as non-finite are left to the fix-up.  CTA b
-// serves kMultiRedElems values of the job whose CTA range holds b: the
-// numerator [slots][C], then the weight map [slots].
-__global__ void __launch_bounds__(kMultiRedElems) k_multi_reduce(const __grid_constant__ F32Multi m) {
-  __shared__ int s_job;
-  if (threadIdx.x == 0) s_job = find_job(m.red_blk, m.n_jobs, blockIdx.x);
-  __syncthreads();
-  const int job = s_job;
-  const F32MultiJob& J = m.jobs[job];
-  const int ns = J.a.n_split;
-  const int C = J.a.C;
-  const int64_t n_slots = J.a.n_slots;
-  const int64_t le = (int64_t)(blockIdx.x - m.red_blk[job]) * kMultiRedElems + threadIdx.x;
-  if (le < n_slots * C) {
-    const int64_t sl = le / C;
-    if (J.a.tgt_perm[sl] == 0xffffffffu) return;
-    const uint64_t b = (uint64_t)sl * (uint64_t)J.n_slabs + (uint64_t)((le - sl * C) / J.pad);
-    if ((J.a.nf_bits[b >> 5] >> (b & 31)) & 1u) return;
-    float v = 0.f;
-    for (int z = 0; z < ns; ++z) v += J.a.part_num[(size_t)z * n_slots * C + le];
-    J.a.acc_num[le] = v;
-    return;
-  }
-  const int64_t sl = le - n_slots * C;
-  if (sl >= n_slots || J.a.tgt_perm[sl] == 0xffffffffu) return;
-  float s = 0.f, c = 0.f;
-  for (int z = 0; z < ns; ++z) {
-    const float2 v = J.a.part_w[(size_t)z * n_slots + sl];
-    const float t = s + v.x;
-    const float bp = t - s;
-    c += (s - (t - bp)) + (v.x - bp) + v.y;
-    s = t;
-  }
-  J.a.acc_w[sl] = make_float2(s, c);
-}
-
-// The flagged rows of all jobs (bitmap words of all jobs, grid-stride).
-__global__ void __launch_bounds__(kFixThreads) k_multi_fixup(const __grid_constant__ F32Multi m) {
-  __shared__ FixShared F;
-  if (*m.nf_any == 0u) return;
-  for (int64_t gw = blockIdx.x; gw < m.n_words; gw += gridDim.x) {
-    const int job = find_job(m.word_off, m.n_jobs, gw);
-    const F32MultiJob& J = m.jobs[job];
-    const int64_t wd = gw - m.word_off[job];
-    if (J.a.nf_bits[wd] == 0u) continue;   // the same word for every thread
-    FixArgs f;
-    f.chi = J.a.tile_chi;
-    f.clo = J.a.tile_clo;
-    f.ta = J.a.tgt_a;
-    f.range_off = J.a.range_off;
-    f.range_s = J.a.range_s;
-    f.T = kTile;
-    f.f1 = J.a.tgt_f1;
-    f.f2 = J.a.tgt_f2;
-    f.tll = J.a.tgt_ll;
-    f.s_hi = J.a.s_hi;
-    f.s_lo = J.a.s_lo;
-    f.perm = J.a.perm;
-    f.sll = J.a.sll;
-    f.kd = J.a.kd;
-    f.data = J.a.data;
-    f.bf16 = J.dtype == CG_BF16;
-    f.C = J.a.C;
-    f.cp = J.pad;
-    f.n_slabs = J.n_slabs;
-    f.mode = J.a.out ? 2 : 0;
-    f.skip_zero = 0;
-    f.out = J.a.out;
-    f.acc_num = J.a.acc_num;
-    f.perm_t = J.a.tgt_perm;
-    f.bits = J.a.nf_bits;
-    f.any = m.nf_any;
-    f.n_words = 0;
-    fix_word(f, wd, F);
-  }
-}
-
-// Eq. 3 for every job: R = N / W (NaN where W = 0) in the caller's layout.
-// CTA b serves kMultiFinElems numerator values of the job whose CTA range
-// holds b, four consecutive channels of one target per thread where the
-// map allows 16-byte rows.
-__global__ void __launch_bounds__(256) k_multi_finalize(const __grid_constant__ F32Multi m) {
-  __shared__ int s_job;
-  if (threadIdx.x == 0) s_job = find_job(m.fin_blk, m.n_jobs, blockIdx.x);
-  __syncthreads();
-  const int job = s_job;
-  const F32MultiJob& J = m.jobs[job];
-  const F32Multi::Out o = m.outs[job];
-  const int C = J.a.C;
-  const int64_t n = J.a.n_slots * C;
-  const int64_t base = (int64_t)(blockIdx.x - m.fin_blk[job]) * kMultiFinElems;
-  if (o.vec4) {
-    const int64_t e = base + 4 * (int64_t)threadIdx.x;
-    if (e >= n) return;
-    const int64_t slot = e / C;
-    const int c = (int)(e - slot * C);
-    const uint32_t u = J.a.tgt_perm[slot];
-    if (u == 0xffffffffu) return;
-    const float2 w2 = J.a.acc_w[slot];
-    const float W = w2.x + w2.y;
-    const float4 v = *reinterpret_cast<const float4*>(J.a.acc_num + e);
-    float4 r;
-    if (W > 0.f) {
-      r = make_float4(v.x / W, v.y / W, v.z / W, v.w / W);
-    } else {
-      const float q = __int_as_float(0x7fc00000);
-      r = make_float4(q, q, q, q);
-    }
-    *reinterpret_cast<float4*>(o.out + (size_t)u * C + c) = r;
-    if (o.out_w && c == 0) o.out_w[u] = W;
-    return;
-  }
-  for (int r = 0; r < kMultiFinElems / 256; ++r) {
-    const int64_t e = base + r * 256 + threadIdx.x;
-    if (e >= n) return;
-    const int64_t slot = e / C;
-    const int c = (int)(e - slot * C);
-    const uint32_t u = J.a.tgt_perm[slot];
-    if (u == 0xffffffffu) continue;
-    const float2 w2 = J.a.acc_w[slot];
-    const float W = w2.x + w2.y;
-    const float v = (W > 0.f) ? J.a.acc_num[e] / W : __int_as_float(0x7fc00000);
-    if (o.channel_major) o.out[(size_t)c * o.P + u] = v;
-    else o.out[(size_t)u * C + c] = v;
-    if (o.out_w && c == 0) o.out_w[u] = W;
-  }
-}
-
-template <int PB, int CB, int NCG, int MINB>
-cudaError_t launch_multi(const MultiLaunch& L, int nsm, cudaStream_t s) {
-  constexpr int NTH = (kTile / PB) * NCG;
-  auto k = k_grid_f32_multi<PB, CB, NCG, MINB>;
-  const size_t smem = sizeof(F32Smem<PB, CB, NCG>);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NTH, smem);
-  if (e != cudaSuccess) return e;
-  const int64_t ctas = std::min<int64_t>((int64_t)std::max(1, per_sm) * nsm, L.m.n_items);
-  k<<<(unsigned)ctas, NTH, smem, s>>>(L);
-  return cudaGetLastError();
-}
-
-}  // namespace
-
-int f32_multi_shape(int C) { return f32_default_config(C); }
-
-int f32_multi_cpad(int shape) {
-  static const int cp[kF32MultiShapes] = {4, 8, 16, 32, 64, 128, 256};
-  return cp[shape < 0 ? 0 : (shape >= kF32MultiShapes ? kF32MultiShapes - 1 : shape)];
-}
-
-cudaError_t grid_f32_multi(const F32Multi& m, cudaStream_t s, int64_t* launches) {
-  if (m.n_items <= 0) return cudaSuccess;
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (m.n_jobs > kF32MultiMaxJobs || !m.hjobs) return cudaErrorInvalidValue;
-  static thread_local MultiLaunch L;   // large: not on the stack (the launch copies it)
-  L.m = m;
-  for (int j = 0; j < m.n_jobs; ++j) L.ga[j] = m.hjobs[j].a;
-  k_multi_order<<<1, kOrderCta, 0, s>>>(m);
-  cudaError_t e;
-  switch (m.shape) {
-    case 0: e = launch_multi<1, 4, 1, 12>(L, nsm, s); break;
-    case 1: e = launch_multi<1, 8, 1, 10>(L, nsm, s); break;
-    case 2: e = launch_multi<1, 8, 2, 6>(L, nsm, s); break;
-    case 3: e = launch_multi<2, 8, 4, 5>(L, nsm, s); break;
-    case 4: e = launch_multi<2, 16, 4, 4>(L, nsm, s); break;
-    case 5: e = launch_multi<4, 16, 8, 3>(L, nsm, s); break;
-    default: e = launch_multi<4, 16, 16, 2>(L, nsm, s); break;
-  }
-  if (e != cudaSuccess) return e;
-  int64_t n = 2;   // order, gridder
-  if (m.n_red_blk > 0) {
-    k_multi_reduce<<<(unsigned)m.n_red_blk, kMultiRedElems, 0, s>>>(m);
-    ++n;
-  }
-  k_multi_fixup<<<(unsigned)nsm, kFixThreads, 0, s>>>(m);
-  if (m.n_fin_blk > 0) {
-    // only jobs whose maps the gridder did not write (splits, channel-major)
-    k_multi_finalize<<<(unsigned)m.n_fin_blk, 256, 0, s>>>(m);
-    ++n;
-  }
-  if (launches) *launches += n + 1;
-  return cudaGetLastError();
+int f32_cpad(int shape) {
+  static const int cp[kF32Configs] = {4, 8, 16, 32, 64, 128, 256};
+  return cp[shape];
 }
 
 // Register-blocking shapes of the FP32 gridder, (targets x channels per

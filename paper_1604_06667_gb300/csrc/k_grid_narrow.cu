@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(kNTh, CN <= 2 ? 3 : 2)
     k_grid_narrow(const __grid_constant__ NarrowArgs na) {
   __shared__ NarrowSmem<CN> S;
   const GridArgs& a = na.g;
+  if (a.hold && hold_gives_up(a.hold, a.hold_cycles, a.err)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t tile = blockIdx.x;
   const int split = blockIdx.z;
@@ -370,11 +371,12 @@ __global__ void __launch_bounds__(kNTh, CN <= 2 ? 3 : 2)
   if (a.out) {
     const float W = wsum + wcor;
     if (a.out_w) a.out_w[u] = W;
-    if (bad) return;
+    if (!bad) {
 #pragma unroll
-    for (int k = 0; k < CN; ++k)
-      if (k < a.C) a.out[(size_t)u * a.C + k] = (W > 0.f) ? num[k] / W : __int_as_float(0x7fc00000);
-    return;
+      for (int k = 0; k < CN; ++k)
+        if (k < a.C) a.out[(size_t)u * a.C + k] = (W > 0.f) ? num[k] / W : __int_as_float(0x7fc00000);
+    }
+    if (!a.keep) return;
   }
   const bool splits = a.n_split > 1;
   if (!bad) {

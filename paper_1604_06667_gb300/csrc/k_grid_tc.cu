@@ -1078,6 +1078,25 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
+cudaError_t encode_rows_map(void* tmap, const void* data, int dtype, int C, int64_t n, int box_cols,
+                            bool swizzle128) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+  if (!enc) return cudaErrorNotSupported;
+  const bool b16 = dtype == CG_BF16;
+  const cuuint64_t gdim[2] = {(cuuint64_t)C, (cuuint64_t)n};
+  const cuuint64_t gstride[1] = {(cuuint64_t)C * (b16 ? 2 : 4)};
+  const cuuint32_t box[2] = {(cuuint32_t)box_cols, 1};
+  const cuuint32_t estr[2] = {1, 1};
+  return enc(static_cast<CUtensorMap*>(tmap),
+             b16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+             const_cast<void*>(data), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? cudaSuccess
+             : cudaErrorInvalidValue;
+}
+
 cudaError_t grid_tiles_tc(cg_grid* g, const void* data, int mode, float* out, float* out_w, int split) {
   const Tiling& t = g->t128;
   TcArgs a;
@@ -1169,17 +1188,11 @@ cudaError_t grid_tiles_tc(cg_grid* g, const void* data, int mode, float* out, fl
   }
   // tensor map over the caller's [N][C] BF16 rows: 64-channel x 1-row boxes,
   // 128-byte swizzle (the layout of the MMA's B operand); rows past N read 0
-  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
-  if (!enc) return cudaErrorNotSupported;
   CUtensorMap tmap;
-  const cuuint64_t gdim[2] = {(cuuint64_t)g->C, (cuuint64_t)g->last_n};
-  const cuuint64_t gstride[1] = {(cuuint64_t)g->C * 2};
-  const cuuint32_t box[2] = {64, 1};
-  const cuuint32_t estr[2] = {1, 1};
-  if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(data), gdim, gstride, box,
-          estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
+  {
+    const cudaError_t em = encode_rows_map(&tmap, data, CG_BF16, g->C, g->last_n, 64, true);
+    if (em != cudaSuccess) return em;
+  }
   // the series form drops the c^4/90 term of d^2, which changes the exponent
   // by |k1| c2^3 / 90; where that could exceed 1e-9 at the support radius the
   // exact 2 asin(c / 2) form is used instead
@@ -1203,6 +1216,7 @@ cudaError_t grid_tiles_tc(cg_grid* g, const void* data, int mode, float* out, fl
   rows.mode = mode;
   rows.skip_zero = false;
   rows.out = out;
+  rows.keep = false;
   rows.acc_num = g->acc_num;
   rows.kd = g->kdev;
   return nonfinite_fixup(g, rows);
