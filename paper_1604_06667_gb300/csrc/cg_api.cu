@@ -121,7 +121,9 @@ void free_all(cg_grid* g) {
   dfree(g->tix_hi, s);
   dfree(g->tix_lo, s);
   dfree(g->tix_ring_off, s);
-  dfree(g->tix_invw, s);
+  dfree(g->tix_rows, s);
+  g->tix_rows_cap = 0;
+  dfree(g->tix_dirty, s);
   if (g->tix_sw.keys_alt) cudaFreeAsync(g->tix_sw.keys_alt, s);
   g->tix_sw.keys_alt = nullptr;
   dfree(g->tix_sw.vals_alt, s);

@@ -102,24 +102,62 @@ __host__ __device__ __forceinline__ void ring_span(int ns, float tlo, float thi,
   ihi = ihi > 4 * ns - 1 ? 4 * ns - 1 : ihi;
 }
 
+struct RingGeo {
+  int count, first;
+  float phase, dphi;
+};
+__host__ __device__ __forceinline__ RingGeo ring_geo(int ns, int i) {
+  RingGeo r;
+  r.phase = 0.5f;
+  if (i < ns) {
+    r.count = 4 * i;
+    r.first = 2 * i * (i - 1);
+  } else if (i <= 3 * ns) {
+    r.count = 4 * ns;
+    r.first = 2 * ns * (ns - 1) + (i - ns) * 4 * ns;
+    r.phase = (((i - ns) & 1) == 0) ? 0.5f : 0.f;
+  } else {
+    const int k = 4 * ns - i;
+    r.count = 4 * k;
+    r.first = 12 * ns * ns - 2 * k * (k + 1);
+  }
+  r.dphi = 2.f * kPiF / (float)r.count;
+  return r;
+}
+
+// Pixels of ring i whose centres lie in the longitude interval [lo, hi] (full:
+// all): up to 2 ranges into out.
+__host__ __device__ __forceinline__ int ring_pixels(const RingGeo& g, int i, float lo, float hi, bool full,
+                                                    Range* out) {
+  int jlo = 0, jhi = g.count - 1;
+  if (!full) {
+    // interval ends in pixels: good to ~1e-2 of a pixel at nside 8192, and
+    // the half pixel in the discs' half-widths reaches to the pixel centres
+    jlo = (int)ceilf(lo / g.dphi - g.phase - 0.02f);
+    jhi = (int)floorf(hi / g.dphi - g.phase + 0.02f);
+    if (jhi < jlo) return 0;
+    if (jhi - jlo + 1 >= g.count) full = true;
+  }
+  if (full) {
+    out[0] = Range{g.first, g.first + g.count - 1, i, 0};
+    return 1;
+  }
+  int a = jlo % g.count, b = jhi % g.count;
+  if (a < 0) a += g.count;
+  if (b < 0) b += g.count;
+  if (a <= b) {
+    out[0] = Range{g.first + a, g.first + b, i, 0};
+    return 1;
+  }
+  out[0] = Range{g.first, g.first + b, i, 0};
+  out[1] = Range{g.first + a, g.first + g.count - 1, i, 0};
+  return 2;
+}
+
 // Pixel ranges of ring i met by the union of nd discs (the hull of their
 // pixel intervals on the ring, a superset); writes up to 2 into out.
 __host__ __device__ inline int ring_ranges(int ns, int i, const Disc* discs, int nd, Range* out) {
-  int count, first;
-  float phase = 0.5f;
-  if (i < ns) {
-    count = 4 * i;
-    first = 2 * i * (i - 1);
-  } else if (i <= 3 * ns) {
-    count = 4 * ns;
-    first = 2 * ns * (ns - 1) + (i - ns) * 4 * ns;
-    phase = (((i - ns) & 1) == 0) ? 0.5f : 0.f;
-  } else {
-    const int k = 4 * ns - i;
-    count = 4 * k;
-    first = 12 * ns * ns - 2 * k * (k + 1);
-  }
-  const float dphi = 2.f * kPiF / (float)count;
+  const RingGeo g = ring_geo(ns, i);
   const float ta = ring_colat(ns, i - 1), tb = ring_colat(ns, i + 1);
   bool any = false, full = false;
   float lo = 0.f, hi = 0.f;   // hull of [pc - W, pc + W], unwrapped near the first disc
@@ -127,7 +165,7 @@ __host__ __device__ inline int ring_ranges(int ns, int i, const Disc* discs, int
     if (discs[q].R < 0.f) continue;   // empty group
     const float hw = disc_halfwidth(discs[q], ta, tb);
     if (hw < 0.f) continue;
-    const float W = hw + 0.5f * dphi + 2e-6f;
+    const float W = hw + 0.5f * g.dphi + 2e-6f;
     if (W >= kPiF) { full = true; break; }
     float c = discs[q].pc;
     if (any) {  // move c to within pi of the hull's centre
@@ -144,29 +182,7 @@ __host__ __device__ inline int ring_ranges(int ns, int i, const Disc* discs, int
     }
   }
   if (!any && !full) return 0;
-  int jlo = 0, jhi = count - 1;
-  if (!full) {
-    // interval ends in pixels: good to ~1e-2 of a pixel at nside 8192, and
-    // the half pixel in W reaches to the pixel centres
-    jlo = (int)ceilf(lo / dphi - phase - 0.02f);
-    jhi = (int)floorf(hi / dphi - phase + 0.02f);
-    if (jhi < jlo) return 0;
-    if (jhi - jlo + 1 >= count) full = true;
-  }
-  if (full) {
-    out[0] = Range{first, first + count - 1, i, 0};
-    return 1;
-  }
-  int a = jlo % count, b = jhi % count;
-  if (a < 0) a += count;
-  if (b < 0) b += count;
-  if (a <= b) {
-    out[0] = Range{first + a, first + b, i, 0};
-    return 1;
-  }
-  out[0] = Range{first, first + b, i, 0};
-  out[1] = Range{first + a, first + count - 1, i, 0};
-  return 2;
+  return ring_pixels(g, i, lo, hi, full, out);
 }
 
 __device__ __forceinline__ bool valid_coord(double lon, double lat) {
@@ -329,6 +345,18 @@ __device__ __forceinline__ int32_t lower_bound_u32(const uint32_t* __restrict__ 
     if (a[mid] < v) lo = mid + 1; else hi = mid;
   }
   return lo;
+}
+
+// Ring number (1 .. 4 ns - 1) of RING pixel p; integer arithmetic with an FP32
+// square-root estimate corrected exactly (nside <= 8192).
+__device__ __forceinline__ int ring_of_pix(int ns, int p) {
+  const int npix = 12 * ns * ns, ncap = 2 * ns * (ns - 1);
+  if (p >= ncap && p < npix - ncap) return ns + (p - ncap) / (4 * ns);
+  const int q = p < ncap ? p : npix - 1 - p;
+  int k = (int)(0.5f * (1.f + sqrtf(1.f + 2.f * (float)q)));
+  while (k > 1 && 2 * k * (k - 1) > q) --k;
+  while (2 * (k + 1) * k <= q) ++k;
+  return p < ncap ? k : 4 * ns - k;
 }
 
 // First pixel of ring i = 0 .. 4 ns (ring 0 is empty, ring 4 ns past the end).

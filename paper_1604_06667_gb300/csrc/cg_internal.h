@@ -42,6 +42,13 @@ struct KernelDev {        // kernel constants used by the gridder
   float inv_a;            // CG_TSINC: 1 / a (rad^-1); k1 then holds the taper -log2(e)/b^2
 };
 
+// Exponents' coefficients of the weights (cg_pair.cuh), both lanes of a packed pair.
+struct WeightConst {
+  float2 q0, q1, q2;      // k1, k1 / 12, k1 / 90: exponent as a series in c^2
+  float2 k1, k2;
+  float c2_in, c2_out;
+};
+
 struct Tiling {           // geometry of one tiling of the targets
   int T = 0;
   int64_t n_tiles = 0;
@@ -160,7 +167,9 @@ struct cg_grid {
   float4* tix_hi = nullptr;       // [n_slots] sorted order
   float4* tix_lo = nullptr;
   int32_t* tix_ring_off = nullptr;  // [4 nside + 1]
-  float* tix_invw = nullptr;      // [n_slots] 1 / W of the operator being transposed
+  float* tix_rows = nullptr;      // map rows in the index's order, times 1 / W
+  size_t tix_rows_cap = 0;
+  uint32_t* tix_dirty = nullptr;  // set when a map holds non-finite values
   cg::SortWork tix_sw;
   // scratch accumulators of cg_grid_dsigma (w' = dw/dsigma pass)
   float* ds_num = nullptr;        // [slots][C]
@@ -422,6 +431,39 @@ cudaError_t target_index_build(cg_grid* g);
 // one weight per sample and channel (k_variants.cu)
 cudaError_t pcw_pack(cg_grid* g, const void* data, int dtype, const float* omega, int64_t n);
 cudaError_t pcw_finalize(cg_grid* g, float* out, int channel_major, float* out_w);
+
+// k_adjoint.cu -- adjoint and interpolation of circular kernels
+struct AdjointArgs {
+  int ns;
+  // samples of the last add, sorted
+  const uint32_t* skey;
+  const uint32_t* sval;
+  const int32_t* ring_off;
+  const float4* s_hi;
+  const float4* s_lo;
+  const double2* sll;       // input order FP64 lon/lat
+  int64_t n;
+  // target index, sorted
+  const uint32_t* t_key;
+  const uint32_t* t_slot;
+  const float4* t_hi;
+  const float4* t_lo;
+  const int32_t* t_ring_off;
+  const double2* tll;       // per slot
+  const uint32_t* perm;
+  KernelDev kd;
+  WeightConst kc;           // set by grid_adjoint
+  float* rows;              // scratch [targets][cpad]
+  int cpad;                 // adjoint_cpad(C)
+  int C;
+  float* out;               // [N][C]
+  int interp;
+  float* vsum;              // [N] or null (interpolation)
+  uint32_t* dirty;          // set when the map holds non-finite values
+};
+int adjoint_cpad(int C);
+cudaError_t grid_adjoint(AdjointArgs a, const float* y, const float* wmap, const float2* acc_w,
+                         int64_t n_targets, cudaStream_t s);
 
 cudaError_t grid_degrid(cg_grid* g, const float* y, const float* wmap, float* out,
                         bool interp = false, float* vsum = nullptr);

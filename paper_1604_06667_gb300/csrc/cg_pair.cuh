@@ -18,6 +18,24 @@ __device__ __forceinline__ float ex2_approx(float x) {
 
 __host__ __device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
 
+// Factor of a target's map row in the adjoint: 1 / W_p (0 where W_p <= 0 or not
+// finite) from a user-order weight map or the slot-order accumulator;
+// interpolation: 1.
+__device__ __forceinline__ float target_factor(uint32_t slot, uint32_t user,
+                                               const float* __restrict__ wmap,
+                                               const float2* __restrict__ acc_w, int interp) {
+  if (user == 0xffffffffu) return 0.f;
+  if (interp) return 1.f;
+  float W;
+  if (wmap) {
+    W = wmap[user];
+  } else {
+    const float2 a = acc_w[slot];
+    W = a.x + a.y;
+  }
+  return (W > 0.f && isfinite(W)) ? 1.f / W : 0.f;
+}
+
 // (s, c) + (v, vc): two-sum of the leading parts, the corrections added up.
 __device__ __forceinline__ void comp_add(float& s, float& c, float v, float vc) {
   const float t = s + v;
@@ -35,12 +53,6 @@ inline int weight_form(const KernelDev& kd) {
   return kd.type == CG_GAUSS1D ? kWGauss1 : kWGauss2;
 }
 
-// Exponents' coefficients (uniform per launch).
-struct WeightConst {
-  float2 q0, q1, q2;      // k1, k1 / 12, k1 / 90: exponent as a series in c^2
-  float2 k1, k2;
-  float c2_in, c2_out;
-};
 __host__ __device__ __forceinline__ WeightConst weight_const(const KernelDev& kd) {
   WeightConst c;
   c.q0 = f2(kd.k1);

@@ -9,6 +9,8 @@
 //            ring offsets and double-float unit vectors in sorted order (the
 //            sample index of k_healpix.cu, built for the targets once per
 //            cg_set_kernel);
+//   circular kernels: k_adjoint.cu; the general kernel below serves the
+//            elliptical kernel and maps with non-finite values:
 //   samples  one warp per 32 consecutive sorted samples of the last add (a
 //            compact strip of one HEALPix ring); its bounding disc, widened by
 //            the support, is queried ring by ring (the per-ring intervals of
@@ -27,6 +29,7 @@
 #include "cg_cut.cuh"
 #include "cg_healpix.cuh"
 #include "cg_internal.h"
+#include "cg_pair.cuh"
 #include "cg_trig.cuh"
 
 namespace cg {
@@ -56,39 +59,6 @@ __global__ void k_target_keys(int64_t ns, const double2* __restrict__ tll,
   u_lo[i] = make_float4(x.lo, y.lo, sb.lo, 0.f);
 }
 
-// 1 / W per slot from a user-order weight map, or from the handle's
-// double-float accumulator (slot order); 0 where W <= 0 or not finite.
-// Normalised interpolation: every valid target slot gets the factor 1.
-__global__ void k_interp_invw(const uint32_t* __restrict__ perm, int64_t n_slots,
-                              float* __restrict__ invw) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n_slots) invw[i] = (perm[i] != 0xffffffffu) ? 1.f : 0.f;
-}
-
-__global__ void k_degrid_invw(const float* __restrict__ wmap, const float2* __restrict__ acc_w,
-                              const uint32_t* __restrict__ perm, int64_t n_slots,
-                              float* __restrict__ invw) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_slots) return;
-  const uint32_t u = perm[i];
-  float W = 0.f;
-  if (u != 0xffffffffu) {
-    if (wmap) {
-      W = wmap[u];
-    } else {
-      const float2 a = acc_w[i];
-      W = a.x + a.y;
-    }
-  }
-  invw[i] = (W > 0.f && isfinite(W)) ? 1.f / W : 0.f;
-}
-
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 struct DegridArgs {
   int64_t ns;
   // samples of the last add, sorted
@@ -109,7 +79,8 @@ struct DegridArgs {
   const float4* f2;
   const double2* tll;
   const uint32_t* perm;
-  const float* invw;
+  const float* wmap;        // W_p in user order, or null: acc_w
+  const float2* acc_w;
   // operator
   KernelDev kd;
   // map and output
@@ -121,12 +92,14 @@ struct DegridArgs {
   // out = sum w y / sum w (NaN where no target is within r), vsum = sum w
   int interp;
   float* vsum;              // [N] or null
+  const uint32_t* dirty;    // null: always run; else only if the word is set
 };
 
 // One warp per 32 consecutive sorted samples; CB channels per pass (grid.y
 // covers the channel blocks).
 template <int CB, int KT, bool BIG>
 __global__ void __launch_bounds__(256) k_degrid(DegridArgs a) {
+  if (a.dirty && *a.dirty == 0u) return;
   const int lane = threadIdx.x & 31;
   const int64_t wt = (int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int64_t s = wt * 32 + lane;
@@ -211,7 +184,8 @@ __global__ void __launch_bounds__(256) k_degrid(DegridArgs a) {
           const int t1 = __shfl_sync(0xffffffffu, iv[q].y, j);
           for (int t = t0; t < t1; ++t) {
             const uint32_t slot = a.t_slot[t];
-            const float iw = a.invw[slot];
+            const uint32_t user = a.perm[slot];
+            const float iw = target_factor(slot, user, a.wmap, a.acc_w, a.interp);
             if (iw == 0.f) continue;        // W_p = 0: the row of G is zero
             const float4 th = a.t_hi[t], tl = a.t_lo[t];
             const float dx = df_diff(h.x, l.x, th.x, tl.x);
@@ -248,10 +222,11 @@ __global__ void __launch_bounds__(256) k_degrid(DegridArgs a) {
             }
             vs += coef;
             if (!__any_sync(0xffffffffu, coef != 0.f)) continue;
-            const float* yr = a.y + (size_t)a.perm[slot] * a.C + c_base;
+            // (a pair that does not take part leaves non-finite values alone)
+            const float* yr = a.y + (size_t)user * a.C + c_base;
 #pragma unroll
             for (int c = 0; c < CB; ++c)
-              if (c_base + c < a.C) x[c] = fmaf(coef, __ldg(yr + c), x[c]);
+              if (c_base + c < a.C && coef != 0.f) x[c] = fmaf(coef, __ldg(yr + c), x[c]);
           }
         }
       }
@@ -358,7 +333,7 @@ cudaError_t target_index_build(cg_grid* g) {
     if ((e = dalloc(&g->tix_ulo, (size_t)m, s)) != cudaSuccess) return e;
     if ((e = dalloc(&g->tix_hi, (size_t)m, s)) != cudaSuccess) return e;
     if ((e = dalloc(&g->tix_lo, (size_t)m, s)) != cudaSuccess) return e;
-    if ((e = dalloc(&g->tix_invw, (size_t)m, s)) != cudaSuccess) return e;
+    if ((e = dalloc(&g->tix_dirty, 1, s)) != cudaSuccess) return e;
   }
   if ((e = dalloc(&g->tix_ring_off, (size_t)(4 * g->nside + 1), s)) != cudaSuccess) return e;
   k_target_keys<<<ceil_div(m, 256), 256, 0, s>>>(g->nside, g->tgt_ll, g->tgt_perm, m, g->tix_key,
@@ -384,12 +359,6 @@ cudaError_t grid_degrid(cg_grid* g, const float* y, const float* wmap, float* ou
   cudaStream_t s = g->stream;
   cudaError_t e = target_index_build(g);
   if (e != cudaSuccess) return e;
-  if (interp)
-    k_interp_invw<<<ceil_div(g->n_slots, 256), 256, 0, s>>>(g->tgt_perm, g->n_slots, g->tix_invw);
-  else
-    k_degrid_invw<<<ceil_div(g->n_slots, 256), 256, 0, s>>>(wmap, g->acc_w, g->tgt_perm,
-                                                            g->n_slots, g->tix_invw);
-  g->n_launches += 1;
   DegridArgs a;
   a.ns = g->nside;
   a.skey = g->sorted_key;
@@ -407,7 +376,8 @@ cudaError_t grid_degrid(cg_grid* g, const float* y, const float* wmap, float* ou
   a.f2 = g->tgt_f2;
   a.tll = g->tgt_ll;
   a.perm = g->tgt_perm;
-  a.invw = g->tix_invw;
+  a.wmap = wmap;
+  a.acc_w = g->acc_w;
   a.kd = g->kdev;
   a.y = y;
   a.out = out;
@@ -415,7 +385,47 @@ cudaError_t grid_degrid(cg_grid* g, const float* y, const float* wmap, float* ou
   a.err = g->d_err;
   a.interp = interp ? 1 : 0;
   a.vsum = vsum;
+  a.dirty = nullptr;
   if (a.n == 0) return cudaGetLastError();
+  if (g->kernel_type != CG_GAUSS2D) {
+    // circular kernels: the tiled gather; the general kernel below then only
+    // runs where the map holds non-finite values
+    AdjointArgs t;
+    t.ns = g->nside;
+    t.skey = a.skey;
+    t.sval = a.sval;
+    t.ring_off = g->ring_off;
+    t.s_hi = a.s_hi;
+    t.s_lo = a.s_lo;
+    t.sll = a.sll;
+    t.n = a.n;
+    t.t_key = a.t_key;
+    t.t_slot = a.t_slot;
+    t.t_hi = a.t_hi;
+    t.t_lo = a.t_lo;
+    t.t_ring_off = a.t_ring_off;
+    t.tll = a.tll;
+    t.perm = a.perm;
+    t.kd = a.kd;
+    t.C = g->C;
+    t.cpad = adjoint_cpad(g->C);
+    t.out = out;
+    t.interp = a.interp;
+    t.vsum = vsum;
+    t.dirty = g->tix_dirty;
+    const size_t need = (size_t)g->n_slots * (size_t)t.cpad;
+    if (g->tix_rows_cap < need) {
+      dfree(g->tix_rows, s);
+      g->tix_rows_cap = 0;
+      if ((e = dalloc(&g->tix_rows, need, s)) != cudaSuccess) return e;
+      g->tix_rows_cap = need;
+    }
+    t.rows = g->tix_rows;
+    if ((e = cudaMemsetAsync(g->tix_dirty, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
+    if ((e = grid_adjoint(t, y, wmap, g->acc_w, g->n_slots, s)) != cudaSuccess) return e;
+    g->n_launches += 2;
+    a.dirty = g->tix_dirty;
+  }
   g->n_launches += 1;
   const bool big = g->kdev.big_support != 0;
   if (g->C <= 8) return launch_degrid<8>(a, big, s);
