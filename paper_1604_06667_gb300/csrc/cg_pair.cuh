@@ -44,6 +44,25 @@ __device__ __forceinline__ void comp_add(float& s, float& c, float v, float vc) 
   s = t;
 }
 
+// Kahan sums of two lanes: s += w with the correction nc (the negative of what
+// is still to subtract); the differences as fma with -1, since packed operands
+// take no sign.
+__device__ __forceinline__ void kahan2(float2& s, float2& nc, float2 w) {
+  const float2 m1 = make_float2(-1.f, -1.f);
+  const float2 y = __fadd2_rn(w, nc);
+  const float2 t = __fadd2_rn(s, y);
+  const float2 e = __ffma2_rn(s, m1, t);
+  nc = __ffma2_rn(e, m1, y);
+  s = t;
+}
+
+// Distance of two squared chords from the centre of the guard band, the smaller
+// with what came before.
+__device__ __forceinline__ float band_near(const WeightConst& k, float2 c2, float before) {
+  const float2 x = __fadd2_rn(c2, k.nmid);
+  return fminf(fminf(fabsf(x.x), fabsf(x.y)), before);
+}
+
 // Forms of the weight evaluation: the Gaussians with the series for d^2 (c^2
 // small, see KernelDev::big_support), and everything else (large supports,
 // the tapered sinc, the width derivative) chosen at run time.
@@ -60,8 +79,12 @@ __host__ __device__ __forceinline__ WeightConst weight_const(const KernelDev& kd
   c.q2 = f2(kd.k1 * (1.f / 90.f));
   c.k1 = f2(kd.k1);
   c.k2 = f2(kd.k2);
-  c.c2_in = kd.c2_in;
   c.c2_out = kd.c2_out;
+  // (a little wide: the sum and difference round; who falls in here is decided
+  // against c2_in and c2_out themselves)
+  const float mid = 0.5f * (kd.c2_in + kd.c2_out);
+  c.nmid = f2(-mid);
+  c.hw = 0.5f * (kd.c2_out - kd.c2_in) * 1.02f;
   return c;
 }
 

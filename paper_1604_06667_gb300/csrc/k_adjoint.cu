@@ -195,7 +195,7 @@ template <int FORM, int NG>
 __device__ __forceinline__ void pair_weights(const AdjointArgs& a, const AdjWarp<NG>& S, float4 h, float4 l,
                                              int t, int part, float2 (&w)[NG / 2]) {
   const WeightConst& kc = a.kc;
-  bool band = false;
+  float near = INFINITY;
 #pragma unroll
   for (int j = 0; j < NG / 2; ++j) {
     const float4 u0 = lds4(&S.pair[j][0]), u1 = lds4(&S.pair[j][2]), u2 = lds4(&S.pair[j][4]);
@@ -209,11 +209,11 @@ __device__ __forceinline__ void pair_weights(const AdjointArgs& a, const AdjWarp
     const float2 v = weight2<FORM>(kc, a.kd, c2, dx, dy, dz, Axes2{});
     const bool i0 = c2.x <= kc.c2_out, i1 = c2.y <= kc.c2_out;
     w[j] = make_float2(i0 ? v.x : 0.f, i1 ? v.y : 0.f);
-    band |= (i0 && c2.x >= kc.c2_in) || (i1 && c2.y >= kc.c2_in);
+    near = band_near(kc, c2, near);
   }
   uint32_t kill = part >= 0 ? ~(1u << part) : 0u;
-  if (band)
-    kill |= adjoint_band(NG, S.s_hi, S.s_lo, S.s_idx, h, l, a.tll[a.t_slot[t]], a.sll, kc.c2_in, kc.c2_out,
+  if (near <= kc.hw)
+    kill |= adjoint_band(NG, S.s_hi, S.s_lo, S.s_idx, h, l, a.tll[a.t_slot[t]], a.sll, a.kd.c2_in, a.kd.c2_out,
                          a.kd.c2r_hi, a.kd.c2r_lo, a.kd.c2r_tol, a.kd.r_rad);
   if (kill) {
 #pragma unroll

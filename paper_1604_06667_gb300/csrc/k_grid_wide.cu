@@ -22,9 +22,9 @@
 // per 8 to 16 targets keeps 50-65 % of the executed FMAs inside the support.
 //
 // Measured on GB300 against the register-blocked form (k_grid.cu), per call:
-// 1e6 samples x 256 channels onto 512 x 512 targets 6.55 -> 4.16 ms, 1e7 x 32
-// on the sphere, elliptical, onto 4096 x 2048 20.0 -> 11.2 ms, 2.5e5 x 256 onto
-// 256 x 256 2.12 -> 1.37 ms, eight scans of 25,000 x 37 2.70 -> 2.06 ms.  Of
+// 1e6 samples x 256 channels onto 512 x 512 targets 6.55 -> 4.10 ms, 1e7 x 32
+// on the sphere, elliptical, onto 4096 x 2048 20.0 -> 11.1 ms, 2.5e5 x 256 onto
+// 256 x 256 2.12 -> 1.35 ms, eight scans of 25,000 x 37 2.70 -> 2.03 ms.  Of
 // the cube's 4.0 ms of gridder 2.5 are channel sums (FMA pipe ~90 % while they
 // run), 1.4 staging, lists and weights.  What it took: no spilled sums (with
 // two CTAs per SM the stages leave no L1 for them: a ninth, producing warp and
@@ -368,12 +368,12 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
       const float2 c2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
       const float2 v = __fmul2_rn(weight2<FORM>(kc, a.kd, c2, dx, dy, dz, A), make_float2(zo.z, zo.w));
       bool i0 = c2.x <= kc.c2_out, i1 = c2.y <= kc.c2_out;
-      if ((i0 && c2.x >= kc.c2_in) || (i1 && c2.y >= kc.c2_in)) {
+      if (band_near(kc, c2, INFINITY) <= kc.hw) {
         // guard band: the cut is decided from the coordinates
         const double2 tll = a.tgt_ll[my_slot];
-        if (i0 && c2.x >= kc.c2_in)
+        if (i0 && c2.x >= a.kd.c2_in)
           i0 = pair_inside(tll, a.sll[S.idx[rs][S.row[warp][k]]], a.kd.c2r_hi, a.kd.c2r_lo, a.kd.c2r_tol, a.kd.r_rad);
-        if (i1 && c2.y >= kc.c2_in)
+        if (i1 && c2.y >= a.kd.c2_in)
           i1 = pair_inside(tll, a.sll[S.idx[rs][S.row[warp][k + 1]]], a.kd.c2r_hi, a.kd.c2r_lo, a.kd.c2r_tol,
                            a.kd.r_rad);
       }
@@ -381,15 +381,16 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
       npair += (i0 ? 1u : 0u) + (i1 ? 1u : 0u);
       S.w[warp][k][lane & (G - 1)] = w0;
       S.w[warp][k + 1][lane & (G - 1)] = w1;
-      // Kahan sum of the target's weights
+      // Kahan sum of the target's weights (one: the packed pair of sums that the
+      // narrow form keeps costs this one 4 % at 256 channels)
       {
-        const float y = w0 - wc, t = ws + y;
-        wc = (t - ws) - y;
+        const float y = w0 + wc, t = ws + y;
+        wc = y - (t - ws);
         ws = t;
       }
       {
-        const float y = w1 - wc, t = ws + y;
-        wc = (t - ws) - y;
+        const float y = w1 + wc, t = ws + y;
+        wc = y - (t - ws);
         ws = t;
       }
     }
@@ -430,7 +431,7 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
   }
 
   // ---- W: lane l holds a part of target l % G's sum ----
-  float wsum = ws, wcor = -wc;
+  float wsum = ws, wcor = wc;
 #pragma unroll
   for (int o = 16; o >= G; o >>= 1) {
     const float s2 = __shfl_xor_sync(0xffffffffu, wsum, o), c2 = __shfl_xor_sync(0xffffffffu, wcor, o);
