@@ -4,9 +4,13 @@
 // lines (Sect. 3.5, WcsGrid / SlGrid).  Here targets are always a list of
 // directions.  To give each CTA a compact group of targets (its "tile"), the
 // targets are split by a k-d tree over their unit vectors: every node is
-// sorted along its widest axis and cut at a multiple of the leaf size, so all
-// leaves hold exactly that many targets (except the last) and each leaf is a
-// compact box.  The tree is cut to 128-target leaves, then each leaf into
+// sorted along the wider of its axes and cut at a multiple of the leaf size, so
+// all leaves hold exactly that many targets (except the last) and each leaf is a
+// compact box.  The axes are east, north and outward at one of the node's
+// targets: along x, y and z the cuts of a field away from those axes are oblique
+// and its leaves lozenges, which reach further.  1e6 samples x 256 channels onto
+// 512 x 512 targets at latitude 30: 6.19 -> 5.85 million candidates, in BF16
+// 1.072 -> 0.984 ms per call, in FP32 4.10 -> 3.78; 2.5e5 x 128 1.35 -> 1.26 ms.  The tree is cut to 128-target leaves, then each leaf into
 // 64 + 64, 32 + 32 and on down to groups of 4, so a 128-tile is two 64-tiles,
 // four 32-target quarters and thirty-two 4-target groups, all compact
 // (consecutive slots).  A position's node at any level follows from its index
@@ -111,70 +115,124 @@ __device__ __forceinline__ Node node_at(uint32_t s, uint32_t P, int level) {
   return q;
 }
 
-// Bounding boxes of the nodes of a level: box[6 n] = min x, y, z, then the
-// complements of max x, y, z (order-preserving integers, so one fill of ones
-// and one atomic minimum serve both).  A warp covers 256 positions and
-// reduces before its atomics (nodes start at multiples of 128): with one
-// atomic per target and side the first levels serialised on a few addresses
-// (13 ms for 786,432 targets).
+// Axes of a node: east, north and outward at the target in its middle (in the
+// order reached so far) where its targets agree on them, else x, y and z.  They
+// agree where the node spans at most 20 degrees and the meridians turn by less
+// than 15 degrees across it; parts of one node cut along directions that differ
+// more become triangles (whole sky, 4096 x 2048 targets, 32 channels: 11.1 ms
+// with the rule, 16.6 with local axes at all levels).
+struct Frame {
+  float3 c, e, n, r;
+};
+
+__device__ __forceinline__ Frame world_frame() {
+  return {make_float3(0.f, 0.f, 0.f), make_float3(1.f, 0.f, 0.f), make_float3(0.f, 1.f, 0.f),
+          make_float3(0.f, 0.f, 1.f)};
+}
+
+// The local axes at a target; reach receives the largest extent of a node along
+// x, y or z for which they are used.
+__device__ __forceinline__ Frame local_frame(const float4 c, float& reach) {
+  const float h2 = c.x * c.x + c.y * c.y;
+  if (!(h2 > 1e-6f)) {
+    reach = -1.f;
+    return world_frame();
+  }
+  const float i = rsqrtf(h2);
+  reach = fminf(0.35f, 0.26f * h2 * i / fmaxf(fabsf(c.z), 1e-6f));
+  return {make_float3(c.x, c.y, c.z), make_float3(-c.y * i, c.x * i, 0.f),
+          make_float3(-c.z * c.x * i, -c.z * c.y * i, h2 * i), make_float3(c.x, c.y, c.z)};
+}
+
+__device__ __forceinline__ float3 in_frame(const Frame& f, const float4 v) {
+  const float x = v.x - f.c.x, y = v.y - f.c.y, z = v.z - f.c.z;
+  return make_float3(x * f.e.x + y * f.e.y + z * f.e.z, x * f.n.x + y * f.n.y + z * f.n.z,
+                     x * f.r.x + y * f.r.y + z * f.r.z);
+}
+
+// Extent of a box (order-preserving minima, complements of maxima).
+__device__ __forceinline__ float3 box_extent(const uint32_t* b) {
+  return make_float3(from_orderable(~b[3]) - from_orderable(b[0]),
+                     from_orderable(~b[4]) - from_orderable(b[1]),
+                     from_orderable(~b[5]) - from_orderable(b[2]));
+}
+
+// Bounding boxes of the nodes of a level along x, y, z and along their local
+// axes: box[12 n] = the minima, then the complements of the maxima
+// (order-preserving integers, so one fill of ones and one atomic minimum serve
+// both), and the same again.  A warp covers 256 positions and reduces before its
+// atomics (nodes start at multiples of 128): with one atomic per target and side
+// the first levels serialised on a few addresses (13 ms for 786,432 targets).
 __global__ void __launch_bounds__(256) k_kd_box(const float4* __restrict__ pos,
                                                 const uint32_t* __restrict__ ord, uint32_t P,
                                                 int level, uint32_t* __restrict__ box) {
   const int lane = threadIdx.x & 31;
   const uint32_t s0 = (blockIdx.x * 8u + (threadIdx.x >> 5)) * 256u;
-  uint32_t b[6], cur = 0xffffffffu;
+  uint32_t b[12], cur = 0xffffffffu;
+  Frame f{};
 #pragma unroll
-  for (int k = 0; k < 6; ++k) b[k] = 0xffffffffu;
+  for (int k = 0; k < 12; ++k) b[k] = 0xffffffffu;
   auto flush = [&]() {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < 12; ++k) {
       const uint32_t m = __reduce_min_sync(0xffffffffu, b[k]);
-      if (lane == 0) atomicMin(&box[6 * cur + k], m);
+      if (lane == 0) atomicMin(&box[12 * cur + k], m);
       b[k] = 0xffffffffu;
     }
   };
   for (int r = 0; r < 8; ++r) {
     const uint32_t sw = s0 + 32u * r;   // uniform over the warp
     if (sw >= P) break;
-    const uint32_t id = node_at(sw, P, level).id;
-    if (id != cur && cur != 0xffffffffu) flush();
-    cur = id;
+    const Node q = node_at(sw, P, level);
+    if (q.id != cur) {
+      if (cur != 0xffffffffu) flush();
+      cur = q.id;
+      float reach;
+      f = local_frame(pos[ord[q.start + q.cnt / 2]], reach);
+    }
     const uint32_t s = sw + lane;
     if (s < P) {
-      const float4 v = pos[ord[s]];
-      const uint32_t x = orderable(v.x), y = orderable(v.y), z = orderable(v.z);
-      b[0] = min(b[0], x);
-      b[1] = min(b[1], y);
-      b[2] = min(b[2], z);
-      b[3] = min(b[3], ~x);
-      b[4] = min(b[4], ~y);
-      b[5] = min(b[5], ~z);
+      const float4 w = pos[ord[s]];
+      const float3 v = in_frame(f, w);
+      const float c[6] = {w.x, w.y, w.z, v.x, v.y, v.z};
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const uint32_t x = orderable(c[k]);
+        const int at = k < 3 ? k : k + 3;
+        b[at] = min(b[at], x);
+        b[at + 3] = min(b[at + 3], ~x);
+      }
     }
   }
   if (cur != 0xffffffffu) flush();
 }
 
 // Sort key: (node, 16-bit coordinate within the node's box along its widest
-// axis).
+// axis).  ord may be val: every position is rewritten with what it holds.
 __global__ void __launch_bounds__(256) k_kd_keys(const float4* __restrict__ pos,
                                                  const uint32_t* ord, uint32_t P, int level,
                                                  const uint32_t* __restrict__ box,
                                                  uint32_t* __restrict__ key, uint32_t* val) {
   const uint32_t s = blockIdx.x * 256u + threadIdx.x;
   if (s >= P) return;
-  const uint32_t id = node_at(s, P, level).id;
-  float lo[3], ext[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    lo[k] = from_orderable(box[6 * id + k]);
-    ext[k] = from_orderable(~box[6 * id + 3 + k]) - lo[k];
+  const Node nd = node_at(s, P, level);
+  const uint32_t* b = box + 12 * (size_t)nd.id;
+  float reach;
+  Frame f = local_frame(pos[ord[nd.start + nd.cnt / 2]], reach);
+  float3 ext = box_extent(b);
+  if (fmaxf(ext.x, fmaxf(ext.y, ext.z)) <= reach) {
+    b += 6;
+    ext = box_extent(b);
+  } else {
+    f = world_frame();
   }
   const uint32_t o = ord[s];
-  const float4 v = pos[o];
-  const int ax = (ext[0] >= ext[1] && ext[0] >= ext[2]) ? 0 : (ext[1] >= ext[2] ? 1 : 2);
-  const float c = ax == 0 ? v.x - lo[0] : (ax == 1 ? v.y - lo[1] : v.z - lo[2]);
-  const float q = ext[ax] > 0.f ? c / ext[ax] * 65535.f : 0.f;
-  key[s] = (id << 16) | min((uint32_t)q, 65535u);
+  const float3 v = in_frame(f, pos[o]);
+  const int ax = (ext.x >= ext.y && ext.x >= ext.z) ? 0 : (ext.y >= ext.z ? 1 : 2);
+  const float c = (ax == 0 ? v.x : (ax == 1 ? v.y : v.z)) - from_orderable(b[ax]);
+  const float ex = ax == 0 ? ext.x : (ax == 1 ? ext.y : ext.z);
+  const float q = ex > 0.f ? c / ex * 65535.f : 0.f;
+  key[s] = (nd.id << 16) | min((uint32_t)q, 65535u);
   val[s] = o;
 }
 
@@ -217,8 +275,44 @@ __global__ void __launch_bounds__(kNodeThreads) k_kd_node(const float4* __restri
     const uint32_t i = tid + k * kNodeThreads;
     seg[k] = Node{0u, 0u, n};
     if (i < np) S.key[i] = i < n ? (uint64_t)i : ~0ull;
-    if (i < n) {
-      const float4 v = pos[ord[nd.start + i]];
+  }
+  // the node's axes
+  if (tid < 6) S.box[0][tid] = 0xffffffffu;
+  __syncthreads();
+  float4 w[kPer];
+  {
+    uint32_t b[6];
+#pragma unroll
+    for (int d = 0; d < 6; ++d) b[d] = 0xffffffffu;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t i = tid + k * kNodeThreads;
+      if (i >= n) continue;
+      w[k] = pos[ord[nd.start + i]];
+      const float c[3] = {w[k].x, w[k].y, w[k].z};
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        b[d] = min(b[d], orderable(c[d]));
+        b[d + 3] = min(b[d + 3], ~orderable(c[d]));
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+      const uint32_t m = __reduce_min_sync(0xffffffffu, b[d]);
+      if (lane == 0 && m != 0xffffffffu) atomicMin(&S.box[0][d], m);
+    }
+  }
+  __syncthreads();
+  if (n > 0u) {
+    float reach;
+    Frame f = local_frame(pos[ord[nd.start + n / 2]], reach);
+    const float3 ext = box_extent(S.box[0]);
+    if (!(fmaxf(ext.x, fmaxf(ext.y, ext.z)) <= reach)) f = world_frame();
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t i = tid + k * kNodeThreads;
+      if (i >= n) continue;
+      const float3 v = in_frame(f, w[k]);
       S.pos[0][i] = v.x;
       S.pos[1][i] = v.y;
       S.pos[2][i] = v.z;
@@ -482,7 +576,7 @@ cudaError_t targets_build(cg_grid* g, const double* lon, const double* lat) {
   if (e == cudaSuccess) e = dalloc(&ord, (size_t)P, s);
   if (e == cudaSuccess) e = dalloc(&val, (size_t)P, s);
   if (e == cudaSuccess && top > 0) e = dalloc(&key, (size_t)P, s);
-  if (e == cudaSuccess && top > 0) e = dalloc(&box, (size_t)6 << (top - 1), s);
+  if (e == cudaSuccess && top > 0) e = dalloc(&box, (size_t)12 << (top - 1), s);
   const unsigned nb = ceil_div(P, 256);
   if (e == cudaSuccess) {
     k_target_init<<<nb, 256, 0, s>>>(lon, lat, P, u_hi, u_lo, ord, g->d_err);
@@ -490,7 +584,7 @@ cudaError_t targets_build(cg_grid* g, const double* lon, const double* lat) {
   }
   uint32_t* cur = ord;   // the targets in the order reached so far
   for (int l = 0; l < top && e == cudaSuccess; ++l) {
-    e = cudaMemsetAsync(box, 0xff, sizeof(uint32_t) * ((size_t)6 << l), s);
+    e = cudaMemsetAsync(box, 0xff, sizeof(uint32_t) * ((size_t)12 << l), s);
     if (e != cudaSuccess) break;
     k_kd_box<<<ceil_div(P, 2048), 256, 0, s>>>(u_hi, cur, (uint32_t)P, l, box);
     k_kd_keys<<<nb, 256, 0, s>>>(u_hi, cur, (uint32_t)P, l, box, key, val);
