@@ -553,16 +553,21 @@ int wide_cpad(int C) {
   return w256 <= w128 ? 256 : 128;
 }
 
-// Candidate shares per tile: only where the tiles and slabs do not fill the
-// chip once, and of at least eight stages each.
+// Candidate shares per tile: where the tiles and slabs do not fill the chip
+// once, shares of at least eight stages each; and where many samples fall on
+// few targets, shares of about a thousand candidates, because a long chain of
+// FP32 additions loses digits (6,000 additions: 1.1e-6 of the map, against
+// 4e-7 for the 800 of an ordinary cube) and a share's sums cost 8 bytes of
+// traffic per thousand multiply-adds.  These partial sums take at most 256 MB.
 int wide_splits(int64_t n_tiles, int64_t n, int C, int n_sms) {
   const int cp = wide_cpad(C);
   const int64_t ctas = n_tiles * ((C + cp - 1) / cp);
   const int64_t fill = (int64_t)n_sms * (cp >= 128 ? 2 : 4);
-  if (4 * ctas >= 3 * fill) return 1;
-  const int64_t want = (2 * fill + ctas - 1) / ctas;
-  const int64_t most = 2 * n / n_tiles / (8 * 32);
-  return (int)std::max<int64_t>(1, std::min<int64_t>(64, std::min(want, most)));
+  const int64_t cand = 2 * n / n_tiles;   // of a tile, or more where the reach is long
+  const int64_t room = ((int64_t)64 << 20) / (n_tiles * kTile * C);
+  int64_t s = std::min(cand / 1024, room);
+  if (4 * ctas < 3 * fill) s = std::max(s, std::min((2 * fill + ctas - 1) / ctas, cand / (8 * 32)));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(64, s));
 }
 
 cudaError_t grid_wide(const GridArgs& a, const Tiling& t, int64_t n, int dtype, cudaStream_t s) {
