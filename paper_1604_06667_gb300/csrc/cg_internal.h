@@ -235,6 +235,7 @@ namespace cg {
 cudaError_t radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int key_bits,
                            SortWork& w, cudaStream_t s, uint32_t** out_keys,
                            uint32_t** out_vals);
+int radix_sort_u32_launches(int64_t n, int key_bits);
 cudaError_t radix_sort_u32_scratch(uint32_t* keys, uint32_t* vals, int64_t n, int key_bits,
                                    uint32_t* keys_alt, uint32_t* vals_alt, uint32_t* hist,
                                    uint32_t* totals, cudaStream_t s, uint32_t** out_keys,

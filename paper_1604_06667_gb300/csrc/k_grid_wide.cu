@@ -24,7 +24,7 @@
 // Measured on GB300 against the register-blocked form (k_grid.cu), per call:
 // 1e6 samples x 256 channels onto 512 x 512 targets 6.55 -> 3.78 ms, 1e7 x 32
 // on the sphere, elliptical, onto 4096 x 2048 20.0 -> 10.9 ms, 2.5e5 x 256 onto
-// 256 x 256 2.12 -> 1.26 ms, eight scans of 25,000 x 37 2.70 -> 1.93 ms.  Of
+// 256 x 256 2.12 -> 1.26 ms, eight scans of 25,000 x 37 2.70 -> 1.73 ms.  Of
 // the cube's 4.0 ms of gridder 2.5 are channel sums (FMA pipe ~90 % while they
 // run), 1.4 staging, lists and weights.  What it took: no spilled sums (with
 // two CTAs per SM the stages leave no L1 for them: a ninth, producing warp and

@@ -250,38 +250,39 @@ __device__ __forceinline__ uint64_t os_word(uint32_t epoch, uint64_t kind, uint3
   return ((uint64_t)epoch << 34) | (kind << 32) | v;
 }
 
-// One pass.  Warp w of the tile ranks the keys [512 w, 512 w + 512) of the
-// tile, 32 consecutive keys per round: equal digits of a round are grouped by
+// One pass.  Warp w of the tile ranks the keys [32 ITEMS w, + 32 ITEMS)
+// of the tile, 32 consecutive keys per round: equal digits of a round are grouped by
 // a warp match, the warp's running count per digit lives in its own row of
 // shared counters, so ranking needs no block barrier.  Then one block step
 // turns the per-warp counts into per-warp digit offsets and the tile's digit
 // counts, the look-back finds the tile's offsets, and every key is written
 // to  tile offset + offset of its warp + its rank within the warp  -- the
 // position of the key among equal digits follows its input position (stable).
+template <int ITEMS>
 __global__ void __launch_bounds__(kThreads) k_os_pass_warp(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
     uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, int64_t n, int shift,
     const uint32_t* __restrict__ ghist, uint64_t* status, uint32_t* ticket, uint32_t epoch,
     unsigned* err) {
-  constexpr int kPerWarp = kOsTile / kWarps;       // 512 keys per warp
+  constexpr int kTile = kThreads * ITEMS, kPerWarp = kTile / kWarps;
   __shared__ uint32_t s_b;
   __shared__ uint32_t blk_off[kRadix];
   __shared__ uint32_t wcnt[kWarps][kRadix];
   __shared__ uint32_t warp_sums[kWarps];
   __shared__ uint32_t t_start[kRadix];      // the tile's keys before digit d
-  __shared__ uint32_t s_key[kOsTile];       // the tile in sorted order
-  __shared__ uint32_t s_val[kOsTile];
+  __shared__ uint32_t s_key[kTile];       // the tile in sorted order
+  __shared__ uint32_t s_val[kTile];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (tid == 0) s_b = atomicAdd(ticket, 1u);
 #pragma unroll
   for (int w2 = 0; w2 < kWarps; ++w2) wcnt[w2][tid] = 0;
   __syncthreads();
   const int64_t b = s_b;
-  const int64_t wbase = b * kOsTile + (int64_t)wid * kPerWarp;
+  const int64_t wbase = b * kTile + (int64_t)wid * kPerWarp;
   const uint32_t lt_mask = (1u << lane) - 1u;
-  uint32_t k_it[kOsItems], v_it[kOsItems], r_it[kOsItems];
+  uint32_t k_it[ITEMS], v_it[ITEMS], r_it[ITEMS];
 #pragma unroll
-  for (int it = 0; it < kOsItems; ++it) {
+  for (int it = 0; it < ITEMS; ++it) {
     const int64_t i = wbase + it * 32 + lane;
     k_it[it] = 0;
     v_it[it] = 0;
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(kThreads) k_os_pass_warp(
   // ranks within the warp, round by round
   uint32_t* wc = wcnt[wid];
 #pragma unroll
-  for (int it = 0; it < kOsItems; ++it) {
+  for (int it = 0; it < ITEMS; ++it) {
     const bool valid = wbase + it * 32 + lane < n;
     const unsigned d = valid ? ((k_it[it] >> shift) & 0xffu) : (unsigned)kRadix;
     const uint32_t peers = __match_any_sync(0xffffffffu, d);
@@ -313,17 +314,17 @@ __global__ void __launch_bounds__(kThreads) k_os_pass_warp(
     wcnt[w2][tid] = c;
     c += x;
   }
+  // publish the count before anything else: the tiles behind wait for it
+  volatile uint64_t* st = status;
+  st[(size_t)b * kRadix + tid] = os_word(epoch, b == 0 ? kInc : kAgg, c);
   // global exclusive offset of digit tid, and the tile's own
   uint32_t tot;
   const uint32_t g_excl = block_exclusive_scan(ghist[tid], warp_sums, tot);
   t_start[tid] = block_exclusive_scan(c, warp_sums, tot);
-  // publish the count, look back for the prefix, publish the prefix
-  volatile uint64_t* st = status;
+  // look back for the prefix, publish the prefix
   if (b == 0) {
-    st[(size_t)tid] = os_word(epoch, kInc, c);
     blk_off[tid] = g_excl;
   } else {
-    st[(size_t)b * kRadix + tid] = os_word(epoch, kAgg, c);
     // look back 8 predecessors per step (independent loads), summing in order
     // until an inclusive prefix; a predecessor not yet published is re-read
     uint32_t prefix = 0;
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(kThreads) k_os_pass_warp(
   // the tile in sorted order in shared memory, then written out in runs per
   // digit (consecutive threads, consecutive positions)
 #pragma unroll
-  for (int it = 0; it < kOsItems; ++it) {
+  for (int it = 0; it < ITEMS; ++it) {
     if (wbase + it * 32 + lane < n) {
       const unsigned d = (k_it[it] >> shift) & 0xffu;
       const uint32_t lp = t_start[d] + wc[d] + r_it[it];
@@ -372,8 +373,8 @@ __global__ void __launch_bounds__(kThreads) k_os_pass_warp(
     }
   }
   __syncthreads();
-  const int64_t tbase = b * kOsTile;
-  const int n_tile = (int)((n - tbase) < kOsTile ? (n - tbase) : kOsTile);
+  const int64_t tbase = b * kTile;
+  const int n_tile = (int)((n - tbase) < kTile ? (n - tbase) : kTile);
   for (int lp = tid; lp < n_tile; lp += kThreads) {
     const uint32_t k = s_key[lp];
     const uint32_t d = (k >> shift) & 0xffu;
@@ -517,7 +518,160 @@ __global__ void __launch_bounds__(kThreads, 4) k_os_pass_block(
   }
 }
 
+// ---------------------------------------------------------------------------
+// Up to kClusterMax keys: all passes in one launch, by one cluster of eight
+// CTAs that keeps keys and values in shared memory.  Every CTA holds an equal
+// part of the array; a pass ranks the part as k_os_pass_warp does (warp w ranks
+// 32 x rounds consecutive keys), the CTAs exchange their digit counts through
+// distributed shared memory, and every key goes straight to its place in the
+// shared memory of the CTA that holds it next.
+//
+// Bound by latency: two cluster barriers and some ten block barriers per pass.
+// The one-sweep passes are so too, but pay a launch, tickets, look-back and
+// round trips to memory for each digit: a map of 2e4 samples 95 -> 69 us, 1000
+// samples 73 -> 45, 40,000 106 -> 90, and no gain at 65,536, so parts go up to
+// 6 x 1024 keys; eight scans of 25,000 samples 1.95 -> 1.73 ms.
+// ---------------------------------------------------------------------------
+constexpr int kClCtas = 8, kClThreads = 1024, kClWarps = kClThreads / 32;
+
+template <int ITEMS>
+struct ClusterSmem {
+  static constexpr int kTile = kClThreads * ITEMS;
+  uint32_t key[2][kTile], val[2][kTile];
+  alignas(16) uint16_t wcnt[kClWarps][kRadix];   // keys of a warp, then before it, per digit
+  uint32_t cnt[kRadix];                          // keys of the CTA per digit
+  uint32_t base[kRadix];                         // place of its first key with the digit
+  uint32_t warp_sums[kWarps];
+};
+
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_load(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+template <int ITEMS>
+__global__ void __cluster_dims__(kClCtas, 1, 1) __launch_bounds__(kClThreads, 1)
+    k_cluster_sort(uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, uint32_t n, int npass) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  ClusterSmem<ITEMS>& S = *reinterpret_cast<ClusterSmem<ITEMS>*>(raw);
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, wid = tid >> 5;
+  const uint32_t rank = blockIdx.x;                             // one cluster
+  const uint32_t part = ((n + kClCtas - 1) / kClCtas + 31u) & ~31u;
+  const uint32_t first = rank * part;
+  const uint32_t mine = first < n ? min(part, n - first) : 0u;
+  const uint32_t rounds = (part + kClThreads - 1) / kClThreads;   // <= ITEMS
+  const uint32_t w0 = wid * rounds * 32u + lane;
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  for (uint32_t i = tid; i < mine; i += kClThreads) {
+    S.key[0][i] = keys[first + i];
+    S.val[0][i] = vals[first + i];
+  }
+  // no CTA writes to another that has not started yet
+  cluster_barrier();
+  uint32_t d_it[ITEMS], r_it[ITEMS];
+  for (int p = 0; p < npass; ++p) {
+    const int cur = p & 1;
+    *reinterpret_cast<uint4*>(&S.wcnt[0][0] + 8 * tid) = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    uint16_t* wc = S.wcnt[wid];
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+      d_it[it] = kRadix;   // invalid lanes form their own group
+      r_it[it] = 0u;
+      if (it >= (int)rounds) continue;
+      const uint32_t i = w0 + it * 32u;
+      const bool valid = i < mine;
+      if (valid) d_it[it] = (S.key[cur][i] >> (8 * p)) & 0xffu;
+      const uint32_t peers = __match_any_sync(0xffffffffu, d_it[it]);
+      const uint32_t before = __popc(peers & lt_mask);
+      const uint32_t c0 = valid ? wc[d_it[it]] : 0u;
+      r_it[it] = c0 + before;
+      __syncwarp();
+      if (valid && before == 0u) wc[d_it[it]] = (uint16_t)(c0 + __popc(peers));
+      __syncwarp();
+    }
+    __syncthreads();
+    if (tid < kRadix) {
+      uint32_t c = 0;
+#pragma unroll
+      for (int w = 0; w < kClWarps; ++w) {
+        const uint32_t x = S.wcnt[w][tid];
+        S.wcnt[w][tid] = (uint16_t)c;
+        c += x;
+      }
+      S.cnt[tid] = c;
+    }
+    cluster_barrier();   // every CTA's counts
+    uint32_t before = 0, incl = 0;
+    if (tid < kRadix) {
+      uint32_t total = 0;
+#pragma unroll
+      for (uint32_t q = 0; q < kClCtas; ++q) {
+        const uint32_t v = cluster_load(cluster_addr(&S.cnt[tid], q));
+        if (q < rank) before += v;
+        total += v;
+      }
+      before -= total;   // exclusive: the inclusive sum below holds the digit itself
+      incl = total;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)lane >= o) incl += y;
+      }
+      if (lane == 31u) S.warp_sums[wid] = incl;
+    }
+    __syncthreads();
+    if (tid < kRadix) {
+      for (uint32_t w = 0; w < wid; ++w) incl += S.warp_sums[w];
+      S.base[tid] = incl + before;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+      if (d_it[it] >= (uint32_t)kRadix) continue;
+      const uint32_t i = w0 + it * 32u;
+      const uint32_t pos = S.base[d_it[it]] + wc[d_it[it]] + r_it[it];
+      const uint32_t to = pos / part, at = pos - to * part;
+      cluster_store(cluster_addr(&S.key[cur ^ 1][at], to), S.key[cur][i]);
+      cluster_store(cluster_addr(&S.val[cur ^ 1][at], to), S.val[cur][i]);
+    }
+    cluster_barrier();   // every key is in its place
+  }
+  for (uint32_t i = tid; i < mine; i += kClThreads) {
+    keys[first + i] = S.key[npass & 1][i];
+    vals[first + i] = S.val[npass & 1][i];
+  }
+}
+
+constexpr int64_t kClusterMax = (int64_t)kClCtas * kClThreads * 6;
+
+template <int ITEMS>
+cudaError_t cluster_sort(uint32_t* keys, uint32_t* vals, int64_t n, int npass, cudaStream_t s) {
+  const int smem = (int)sizeof(ClusterSmem<ITEMS>);
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_cluster_sort<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  k_cluster_sort<ITEMS><<<kClCtas, kClThreads, smem, s>>>(keys, vals, (uint32_t)n, npass);
+  return cudaGetLastError();
+}
+
 }  // namespace
+
+int radix_sort_u32_launches(int64_t n, int key_bits) {
+  return n <= 0 ? 0 : (n <= kClusterMax ? 1 : 1 + (key_bits + 7) / 8);
+}
 
 cudaError_t radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int key_bits,
                            SortWork& w, cudaStream_t s, uint32_t** out_keys,
@@ -526,7 +680,21 @@ cudaError_t radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int key_bi
   *out_vals = vals;
   if (n <= 0) return cudaSuccess;
   const int npass = (key_bits + 7) / 8;
-  const int nblk = (int)ceil_div(n, kOsTile);
+  if (n <= kClusterMax)
+    return n <= (int64_t)kClCtas * kClThreads * 4 ? cluster_sort<4>(keys, vals, n, npass, s)
+                                                  : cluster_sort<6>(keys, vals, n, npass, s);
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  // Warp-ranked passes are faster while the tiles run as one wave (their
+  // look-back waits overlap the ranking), with half as many rounds of ranking
+  // as soon as the half tiles are one wave (a map of 2e5 samples 150 -> 139 us,
+  // 6e4 111 -> 99, 7e5 240 -> 234, 1e6 291 -> 296); with many waves of tiles
+  // the block-ranked pass keeps more tiles in flight (measured on GB300: 1e6
+  // keys 0.081 vs 0.098 ms, 1e8 keys 8.4 vs 7.6 ms for the sort).
+  const bool warp_ranked = ceil_div(n, kOsTile) <= 2 * nsm;
+  const bool few = ceil_div(n, kThreads * 8) <= 2 * nsm;
+  const int nblk = (int)ceil_div(n, few ? kThreads * 8 : kOsTile);
   cudaError_t e = ensure_work<uint32_t>(w, n, (int)ceil_div(n, kTileKeys), s);
   if (e != cudaSuccess) return e;
   if (w.cap_status < (size_t)nblk * kRadix) {
@@ -551,19 +719,15 @@ cudaError_t radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int key_bi
   k_os_hist<<<hblk, kThreads, 0, s>>>(keys, n, npass, ghist);
   uint32_t *kin = keys, *kout = static_cast<uint32_t*>(w.keys_alt);
   uint32_t *vin = vals, *vout = w.vals_alt;
-  // Warp-ranked passes are faster while the tiles run as one wave (their
-  // look-back waits overlap the ranking); with many waves of tiles the
-  // block-ranked pass keeps more tiles in flight (measured on GB300: 1e6
-  // keys 0.081 vs 0.098 ms, 1e8 keys 8.4 vs 7.6 ms for the sort).
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const bool warp_ranked = nblk <= 2 * nsm;
   for (int p = 0; p < npass; ++p) {
     w.epoch = (w.epoch + 1) & 0x3fffffffu;
     if (w.epoch == 0) w.epoch = 1;
-    if (warp_ranked)
-      k_os_pass_warp<<<nblk, kThreads, 0, s>>>(kin, vin, kout, vout, n, 8 * p,
+    if (few)
+      k_os_pass_warp<8><<<nblk, kThreads, 0, s>>>(kin, vin, kout, vout, n, 8 * p,
+                                                  ghist + p * kRadix, w.status, tickets + p,
+                                                  w.epoch, w.err);
+    else if (warp_ranked)
+      k_os_pass_warp<kOsItems><<<nblk, kThreads, 0, s>>>(kin, vin, kout, vout, n, 8 * p,
                                                ghist + p * kRadix, w.status, tickets + p,
                                                w.epoch, w.err);
     else

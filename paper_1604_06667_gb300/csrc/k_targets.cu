@@ -591,7 +591,7 @@ cudaError_t targets_build(cg_grid* g, const double* lon, const double* lat) {
     uint32_t* sk = nullptr;
     const int bits = 16 + l;
     e = radix_sort_u32(key, val, P, bits, w, s, &sk, &cur);
-    g->n_launches += 3 + (bits + 7) / 8;
+    g->n_launches += 2 + radix_sort_u32_launches(P, bits);
   }
   if (e == cudaSuccess) {
     // (`ord` is free unless nothing has been sorted: then val takes the result)
