@@ -47,6 +47,7 @@ struct WeightConst {
   float2 q0, q1, q2;      // k1, k1 / 12, k1 / 90: exponent as a series in c^2
   float2 k1, k2;
   float c2_out;           // squared chord beyond which a pair is outside
+  float2 ds;              // width derivative: its factor over k1
   float2 nmid;            // minus the centre of the guard band, and its half-width:
   float hw;               // |c2 - mid| <= hw finds every pair of the band
 };

@@ -64,11 +64,12 @@ __device__ __forceinline__ float band_near(const WeightConst& k, float2 c2, floa
 }
 
 // Forms of the weight evaluation: the Gaussians with the series for d^2 (c^2
-// small, see KernelDev::big_support), and everything else (large supports,
-// the tapered sinc, the width derivative) chosen at run time.
-enum { kWGauss1 = 0, kWGauss2 = 1, kWAny = 2 };
+// small, see KernelDev::big_support), the circular one's width derivative, and
+// everything else (large supports, the tapered sinc) chosen at run time.
+enum { kWGauss1 = 0, kWGauss2 = 1, kWAny = 2, kWGauss1Ds = 3 };
 inline int weight_form(const KernelDev& kd) {
-  if (kd.big_support || kd.dscale != 0.f || kd.type == CG_TSINC) return kWAny;
+  if (kd.big_support || kd.type == CG_TSINC) return kWAny;
+  if (kd.dscale != 0.f) return kd.type == CG_GAUSS1D ? kWGauss1Ds : kWAny;
   return kd.type == CG_GAUSS1D ? kWGauss1 : kWGauss2;
 }
 
@@ -79,6 +80,7 @@ __host__ __device__ __forceinline__ WeightConst weight_const(const KernelDev& kd
   c.q2 = f2(kd.k1 * (1.f / 90.f));
   c.k1 = f2(kd.k1);
   c.k2 = f2(kd.k2);
+  c.ds = f2(kd.dscale / kd.k1);
   c.c2_out = kd.c2_out;
   // (a little wide: the sum and difference round; who falls in here is decided
   // against c2_in and c2_out themselves)
@@ -129,6 +131,9 @@ __device__ __forceinline__ float2 weight2(const WeightConst& k, const KernelDev&
   if constexpr (FORM == kWGauss1) {
     const float2 e = __fmul2_rn(c2, __ffma2_rn(c2, __ffma2_rn(c2, k.q2, k.q1), k.q0));
     return make_float2(ex2_approx(e.x), ex2_approx(e.y));
+  } else if constexpr (FORM == kWGauss1Ds) {
+    const float2 e = __fmul2_rn(c2, __ffma2_rn(c2, __ffma2_rn(c2, k.q2, k.q1), k.q0));
+    return __fmul2_rn(__fmul2_rn(e, k.ds), make_float2(ex2_approx(e.x), ex2_approx(e.y)));
   } else if constexpr (FORM == kWGauss2) {
     const float2 ap = __ffma2_rn(dx, A.ax, __ffma2_rn(dy, A.ay, __fmul2_rn(dz, A.az)));
     const float2 bp = __ffma2_rn(dx, A.bx, __ffma2_rn(dy, A.by, __fmul2_rn(dz, A.bz)));

@@ -266,26 +266,40 @@ cudaError_t launch_degrid(const DegridArgs& a, bool big, cudaStream_t s) {
 constexpr int kDsBlock = 256;
 
 // dR[user][c] = (N' - R W') / W (NaN where W = 0) and the block's share of
-// sum g dR (FP64) -- one thread per (slot, channel).
+// sum g dR (FP64) -- one thread per (slot, channel).  Bound by FP64 operations
+// (1.6 per clock and SM), so the quotients of a slot, 1 / W and W' / W, are taken
+// once per slot and block.
 __global__ void __launch_bounds__(kDsBlock) k_dsigma_out(
     const float* __restrict__ n0, const float2* __restrict__ w0, const float* __restrict__ n1,
     const float2* __restrict__ w1, const uint32_t* __restrict__ perm, int64_t n_slots, int C,
     const float* __restrict__ grad, float* __restrict__ dR, double* __restrict__ part) {
   __shared__ double red[kDsBlock / 32];
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double acc = 0.0;
-  if (e < n_slots * C) {
-    const int64_t slot = e / C;
-    const int c = (int)(e % C);
-    const uint32_t u = perm[slot];
-    if (u != 0xffffffffu) {
+  __shared__ double inv[kDsBlock], ratio[kDsBlock];   // 1 / W (-1: no W), W' / W
+  const int64_t e0 = (int64_t)blockIdx.x * kDsBlock;
+  const int64_t slot0 = e0 / C;
+  const int64_t e = e0 + threadIdx.x;
+  {
+    const int64_t last = min(e0 + kDsBlock, n_slots * C) - 1;
+    const int64_t slot = slot0 + threadIdx.x;
+    if (slot <= last / C) {
       const float2 a0 = w0[slot], a1 = w1[slot];
       const double W = (double)a0.x + (double)a0.y;
       const double Wp = (double)a1.x + (double)a1.y;
+      inv[threadIdx.x] = W > 0.0 ? 1.0 / W : -1.0;
+      ratio[threadIdx.x] = W > 0.0 ? Wp / W : 0.0;
+    }
+  }
+  __syncthreads();
+  double acc = 0.0;
+  if (e < n_slots * C) {
+    const int64_t slot = e / C;
+    const int c = (int)(e - slot * C);
+    const uint32_t u = perm[slot];
+    if (u != 0xffffffffu) {
       double v = __int_as_float(0x7fc00000);
-      if (W > 0.0) {
-        const double R = (double)n0[slot * C + c] / W;
-        v = ((double)n1[slot * C + c] - R * Wp) / W;
+      const double iw = inv[slot - slot0];
+      if (iw >= 0.0) {
+        v = ((double)n1[e] - (double)n0[e] * ratio[slot - slot0]) * iw;
         if (grad) acc = (double)grad[(size_t)u * C + c] * v;
       }
       if (dR) dR[(size_t)u * C + c] = (float)v;

@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kNTh, CN <= 2 ? 3 : 2)
     A[0] = make_float2(p.x, q.x);
     A[1] = make_float2(p.y, q.y);
     A[2] = make_float2(p.z, q.z);
-    if (FORM != kWGauss1 && a.kd.type == CG_GAUSS2D) {
+    if (FORM != kWGauss1 && FORM != kWGauss1Ds && a.kd.type == CG_GAUSS2D) {
       const float4 f1a = a.tgt_f1[sa], f1b = a.tgt_f1[sa + 1];
       const float4 f2a = a.tgt_f2[sa], f2b = a.tgt_f2[sa + 1];
       A[4] = make_float2(f1a.x, f1b.x);
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kNTh, CN <= 2 ? 3 : 2)
           const float2 dz = __fadd2_rn(lds2(q6 + 16), nz);
           const float2 c2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
           Axes2 A{};
-          if (FORM != kWGauss1) {
+          if (FORM != kWGauss1 && FORM != kWGauss1Ds) {
             const float4 u0 = lds4(q6 + 32), u1 = lds4(q6 + 48), u2 = lds4(q6 + 64);
             A.ax = make_float2(u0.x, u0.y); A.ay = make_float2(u0.z, u0.w);
             A.az = make_float2(u1.x, u1.y); A.bx = make_float2(u1.z, u1.w);
@@ -432,6 +432,7 @@ cudaError_t launch_narrow(const NarrowArgs& na, int64_t n_tiles, int64_t n, int 
   switch (weight_form(na.g.kd)) {
     case kWGauss1: k_grid_narrow<CN, kWGauss1><<<grid, kNTh, 0, s>>>(na); break;
     case kWGauss2: k_grid_narrow<CN, kWGauss2><<<grid, kNTh, 0, s>>>(na); break;
+    case kWGauss1Ds: k_grid_narrow<CN, kWGauss1Ds><<<grid, kNTh, 0, s>>>(na); break;
     default: k_grid_narrow<CN, kWAny><<<grid, kNTh, 0, s>>>(na); break;
   }
   return cudaGetLastError();

@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
   const WeightConst& kc = wa.kc;
   const float4 at = a.tgt_a[my_slot];
   Axes2 A{};
-  if (FORM != kWGauss1 && a.kd.type == CG_GAUSS2D) {
+  if (FORM != kWGauss1 && FORM != kWGauss1Ds && a.kd.type == CG_GAUSS2D) {
     const float4 u = a.tgt_f1[my_slot], v = a.tgt_f2[my_slot];
     A.ax = f2(u.x); A.ay = f2(u.y); A.az = f2(u.z);
     A.bx = f2(v.x); A.by = f2(v.y); A.bz = f2(v.z);
@@ -525,6 +525,7 @@ cudaError_t launch_wide(const WideArgs& wa, const CUtensorMap& tmap, int64_t n_t
   switch (weight_form(wa.g.kd)) {
     case kWGauss1: return go(k_grid_wide<SH, kWGauss1, MINB>);
     case kWGauss2: return go(k_grid_wide<SH, kWGauss2, MINB>);
+    case kWGauss1Ds: return go(k_grid_wide<SH, kWGauss1Ds, MINB>);
     default: return go(k_grid_wide<SH, kWAny, MINB>);
   }
 }
