@@ -646,9 +646,13 @@ __global__ void k_split_reduce(const float* __restrict__ part_num,
                                const uint32_t* __restrict__ perm, int64_t n_slots, int C,
                                int n_split, int accumulate, float* __restrict__ acc_num,
                                float2* __restrict__ acc_w, const uint32_t* __restrict__ nf_bits,
-                               int cpad, int n_slabs) {
+                               int cpad, int n_slabs, const int32_t* __restrict__ tile_cand) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_slots * (C + 1)) return;
+  if (tile_cand) {   // the wide form: shares per tile; whole tiles are written already
+    n_split = wide_shares(tile_cand[(e < n_slots * C ? e / C : e - n_slots * C) / kTile], n_split);
+    if (n_split == 1) return;
+  }
   if (e < n_slots * C) {
     const int64_t sl = e / C;
     if (perm[sl] == 0xffffffffu) return;
@@ -757,13 +761,13 @@ cudaError_t begin_pass(cg_grid* g, GridArgs& a, int n_slabs, bool* direct, bool*
 // After the gridder: the splits' sum and the flagged non-finite rows
 // (bitmap rows of cpad channels).
 cudaError_t end_pass(cg_grid* g, const GridArgs& a, int dtype, int cpad, int n_slabs,
-                     bool skip_zero) {
+                     bool skip_zero, const int32_t* tile_cand = nullptr) {
   cudaError_t e;
   if (a.n_split > 1) {
     const int64_t m = g->n_slots * (int64_t)(a.C + 1);
     k_split_reduce<<<ceil_div(m, 256), 256, 0, g->stream>>>(
         a.part_num, a.part_w, a.tgt_perm, g->n_slots, a.C, a.n_split, a.accumulate, a.acc_num,
-        a.acc_w, a.nf_bits, cpad, n_slabs);
+        a.acc_w, a.nf_bits, cpad, n_slabs, tile_cand);
     g->n_launches += 1;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -843,12 +847,12 @@ cudaError_t run_wide(cg_grid* g, GridArgs& a, int dtype, bool* direct, bool* kep
   const int64_t nt = g->t64.n_tiles;
   const int cp = wide_cpad(a.C);
   const int n_slabs = (a.C + cp - 1) / cp;
-  a.n_split = wide_splits(nt, g->last_n, a.C, sm_count());
+  a.n_split = wide_splits(nt, g->last_n, a.C, sm_count(), !a.out && a.acc_num == g->acc_num);
   a.keep = sums_kept(nt, a.C, sm_count());
   cudaError_t e = begin_pass(g, a, n_slabs, direct, kept);
   if (e == cudaSuccess) e = grid_wide(a, g->t64, g->last_n, dtype, g->stream);
   if (e != cudaSuccess) return e;
-  return end_pass(g, a, dtype, cp, n_slabs, true);
+  return end_pass(g, a, dtype, cp, n_slabs, true, a.tile_cand);
 }
 
 }  // namespace
