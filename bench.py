@@ -405,7 +405,7 @@ def time_form(g, wl, form, lon, lat, data, out, out_w, args, world, local, peaks
         ach = 2.0 * upd / (t_grid / 1e3) / 1e12
         roof = {"bound": "alu", "achieved": ach, "peak": peak_tf, "unit": "TFLOP/s",
                 "frac": ach / peak_tf, "traffic": None,
-                "kernel": "k_grid_f32 (tile gridder, FP32 CUDA cores)",
+                "kernel": "k_grid_wide (tile gridder, FP32 CUDA cores)",
                 "peak_source": "152 SMs x 128 FP32 lanes x 2 flop x max SM clock"}
     else:
         hbm = peaks["hbm_gbs"]
@@ -524,8 +524,8 @@ def time_batched(args, dev, n_jobs=64):
     autotuner free to pick the tensor-core form, plain form = FP32 data on
     the FP32 CUDA-core path (autotuned shapes).  Each form is timed twice on
     the same jobs and choices: the per-job graph (one pipeline per job on 16
-    branches) and the fused graph (one sample index and one persistent FP32
-    gridder launch per register shape).  Inputs resident in HBM."""
+    branches) and the fused graph (one sample index for all jobs, the one-job
+    gridders on it).  Inputs resident in HBM."""
     import torch
     import workloads
     from paper_1604_06667_gb300 import Batch, Gridder
@@ -564,8 +564,7 @@ def time_batched(args, dev, n_jobs=64):
                      "updates_per_batch": upd, "pairs_per_batch": int(sum(pairs)),
                      "graph_kernels": b.info()["graph_kernels"],
                      "tc_jobs": sum(1 for c in ch if c["path"] == 2)}
-        # the fused pipeline on the same jobs and choices: one sample index,
-        # one persistent FP32 gridder launch, tensor-core jobs on their own
+        # the fused pipeline on the same jobs and choices: one sample index
         b.set_fused(True).capture()
         for _ in range(max(3, args.warmup)):
             b.run()

@@ -1,4 +1,9 @@
-// k_grid.cu -- tile gridder, FP32 CUDA-core form (paper Eq. 1-2).
+// k_grid.cu -- tile gridder, FP32 CUDA-core form (paper Eq. 1-2): the passes
+// over the FP32 forms, and the register-blocked form.
+//
+// A pass runs k_grid_narrow.cu (at most 8 channels) or k_grid_wide.cu unless a
+// register-blocked shape was named (cg_set_f32_shape, or the autotuner's
+// choice); the kernels below serve those shapes.
 //
 // One CTA owns one tile of kTile targets, so no two CTAs ever write the same
 // output cell: the race-free ownership of target pixels of the paper's lookup
