@@ -1,0 +1,34 @@
+// cg_index.h -- index arithmetic of the kernels that a host compiler can check
+// as well (plain C++; under nvcc the functions serve both sides).
+#pragma once
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define CG_HD __host__ __device__ __forceinline__
+#else
+#define CG_HD inline
+#endif
+
+namespace cg {
+
+constexpr uint32_t kEmptySlot = 0xffffffffu;   // tgt_perm of a slot without a target
+
+// Shares that a tile of `total` candidates is worked on in, of at most n_split
+// (the wide FP32 form; shares of fewer than eight stages cost more than they
+// give).
+CG_HD int wide_shares(int total, int n_split) {
+  const int s = total / 256;
+  return s < 1 ? 1 : (s < n_split ? s : n_split);
+}
+
+// Partial sums of a slot: the shares of its tile, 0 for an empty slot.  Slots
+// come in whole 128-target tiles, candidate counts in 64-target tiles that hold
+// at least one target, so an empty slot's tile may lie past the last count: it
+// is not looked up.  tile_cand null: every tile has n_split shares.
+template <class Perm, class Cand>
+CG_HD int slot_shares(Perm perm, Cand tile_cand, int64_t slot, int tile, int n_split) {
+  if (perm[slot] == kEmptySlot) return 0;
+  return tile_cand ? wide_shares(tile_cand[slot / tile], n_split) : n_split;
+}
+
+}  // namespace cg

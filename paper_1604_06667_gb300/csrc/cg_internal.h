@@ -7,6 +7,8 @@
 
 #include <vector>
 
+#include "cg_index.h"
+
 // the public C ABI is the only thing the shared library exports
 #pragma GCC visibility push(default)
 #include "../../include/cygrid_gb300.h"
@@ -331,13 +333,6 @@ cudaError_t grid_narrow(const GridArgs& a, const Tiling& t, int64_t n, int dtype
 // k_grid_wide.cu -- more than 8 channels: warps over compact target groups and
 // all channels of a slab.
 int wide_cpad(int C);
-// Shares that a tile of `total` candidates is worked on in, of at most n_split
-// (the wide form; shares of fewer than eight stages cost more than they give).
-__host__ __device__ inline int wide_shares(int total, int n_split) {
-  const int s = total / 256;
-  return s < 1 ? 1 : (s < n_split ? s : n_split);
-}
-
 int wide_splits(int64_t n_tiles, int64_t n, int C, int n_sms, bool uneven);
 cudaError_t grid_wide(const GridArgs& a, const Tiling& t, int64_t n, int dtype, cudaStream_t s);
 constexpr int kF32Configs = 7;   // register-blocking shapes of the FP32 gridder

@@ -654,13 +654,11 @@ __global__ void k_split_reduce(const float* __restrict__ part_num,
                                int cpad, int n_slabs, const int32_t* __restrict__ tile_cand) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_slots * (C + 1)) return;
-  if (tile_cand) {   // the wide form: shares per tile; whole tiles are written already
-    n_split = wide_shares(tile_cand[(e < n_slots * C ? e / C : e - n_slots * C) / kTile], n_split);
-    if (n_split == 1) return;
-  }
+  // (the wide form: shares per tile; tiles of one share are written already)
+  const int64_t sl = e < n_slots * C ? e / C : e - n_slots * C;
+  n_split = slot_shares(perm, tile_cand, sl, kTile, n_split);
+  if (n_split == 0 || (tile_cand && n_split == 1)) return;
   if (e < n_slots * C) {
-    const int64_t sl = e / C;
-    if (perm[sl] == 0xffffffffu) return;
     // a row some split flagged as non-finite is the fix-up pass's to write
     const uint64_t b = (uint64_t)sl * (uint64_t)n_slabs + (uint64_t)((e - sl * C) / cpad);
     if ((nf_bits[b >> 5] >> (b & 31)) & 1u) return;
@@ -669,8 +667,6 @@ __global__ void k_split_reduce(const float* __restrict__ part_num,
     acc_num[e] = accumulate ? acc_num[e] + v : v;
     return;
   }
-  const int64_t sl = e - n_slots * C;
-  if (perm[sl] == 0xffffffffu) return;
   float s = 0.f, c = 0.f;
   for (int z = 0; z < n_split; ++z) {
     const float2 v = part_w[(size_t)z * n_slots + sl];

@@ -1,0 +1,60 @@
+"""Index arithmetic of the kernels, checked on the host: the same header
+(csrc/cg_index.h) compiled as plain C++ against tables that refuse an index out
+of range."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1604_06667_gb300", "csrc")
+
+PRELUDE = r"""
+#include <cstdint>
+#include <cstdio>
+#include <cstdlib>
+#include <vector>
+#include "cg_index.h"
+#define CHECK(x) do { if (!(x)) { std::printf("line %d: %s\n", __LINE__, #x); std::exit(1); } } while (0)
+template <class T>
+struct Table {                       // an array that refuses an index out of range
+  std::vector<T> v;
+  explicit operator bool() const { return true; }
+  const T& operator[](int64_t i) const {
+    if (i < 0 || i >= (int64_t)v.size()) { std::printf("index %lld of %zu\n", (long long)i, v.size()); std::exit(1); }
+    return v[(size_t)i];
+  }
+};
+"""
+
+
+def _run(tmp_path, body):
+    cxx = shutil.which("g++") or pytest.skip("no host compiler")
+    src, exe = str(tmp_path / "t.cpp"), str(tmp_path / "t")
+    with open(src, "w") as f:
+        f.write(PRELUDE + body)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-I", CSRC, src, "-o", exe], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
+
+
+def test_shares_of_empty_slots(tmp_path):
+    """Slots of a last 128-target tile whose second half is empty have no
+    candidate count of their own."""
+    _run(tmp_path, r"""
+int main() {
+  for (int P : {1, 63, 64, 65, 128, 129, 192, 193, 40000, 40001}) {
+    const int slots = (P + 127) / 128 * 128;
+    Table<uint32_t> perm;
+    Table<int> cand;
+    for (int s = 0; s < slots; ++s) perm.v.push_back(s < P ? (uint32_t)s : cg::kEmptySlot);
+    for (int t = 0; t < (P + 63) / 64; ++t) cand.v.push_back(300 * (t % 5));
+    for (int s = 0; s < slots; ++s) {
+      const int n = cg::slot_shares(perm, cand, s, 64, 4);
+      CHECK(n == (s < P ? cg::wide_shares(cand[s / 64], 4) : 0));
+      CHECK(cg::slot_shares(perm, (const int*)nullptr, s, 64, 4) == (s < P ? 4 : 0));
+    }
+  }
+}
+""")
