@@ -31,4 +31,21 @@ CG_HD int slot_shares(Perm perm, Cand tile_cand, int64_t slot, int tile, int n_s
   return tile_cand ? wide_shares(tile_cand[slot / tile], n_split) : n_split;
 }
 
+// Targets' k-d tree: levels of nodes that are sorted over the whole array, until
+// a node of the `n_tiles` tiles of `tile` targets holds at most `cap` targets.
+CG_HD int kd_top_levels(int64_t n_tiles, int tile, int cap) {
+  int top = 0;
+  while (((n_tiles + ((int64_t)1 << top) - 1) >> top) * tile > cap) ++top;
+  return top;
+}
+
+// Such a level's 32-bit sort key: the node's number (`level` bits) above the
+// coordinate, which gives way from level 17 on (more than 2^29 targets).
+CG_HD int kd_coord_bits(int level) { return level > 16 ? 32 - level : 16; }
+CG_HD uint32_t kd_key(uint32_t node, int level, float t) {   // t: 0 .. 1 across the node
+  const int bits = kd_coord_bits(level);
+  const uint32_t most = (1u << bits) - 1u, q = (uint32_t)(t * (float)most);
+  return (node << bits) | (q < most ? q : most);
+}
+
 }  // namespace cg

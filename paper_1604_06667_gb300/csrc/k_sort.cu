@@ -680,6 +680,7 @@ cudaError_t radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int key_bi
   *out_vals = vals;
   if (n <= 0) return cudaSuccess;
   const int npass = (key_bits + 7) / 8;
+  if (npass > kMaxPasses) return cudaErrorInvalidValue;
   if (n <= kClusterMax)
     return n <= (int64_t)kClCtas * kClThreads * 4 ? cluster_sort<4>(keys, vals, n, npass, s)
                                                   : cluster_sort<6>(keys, vals, n, npass, s);

@@ -207,8 +207,8 @@ __global__ void __launch_bounds__(256) k_kd_box(const float4* __restrict__ pos,
   if (cur != 0xffffffffu) flush();
 }
 
-// Sort key: (node, 16-bit coordinate within the node's box along its widest
-// axis).  ord may be val: every position is rewritten with what it holds.
+// Sort key: (node, coordinate within the node's box along its widest axis).
+// ord may be val: every position is rewritten with what it holds.
 __global__ void __launch_bounds__(256) k_kd_keys(const float4* __restrict__ pos,
                                                  const uint32_t* ord, uint32_t P, int level,
                                                  const uint32_t* __restrict__ box,
@@ -231,8 +231,7 @@ __global__ void __launch_bounds__(256) k_kd_keys(const float4* __restrict__ pos,
   const int ax = (ext.x >= ext.y && ext.x >= ext.z) ? 0 : (ext.y >= ext.z ? 1 : 2);
   const float c = (ax == 0 ? v.x : (ax == 1 ? v.y : v.z)) - from_orderable(b[ax]);
   const float ex = ax == 0 ? ext.x : (ax == 1 ? ext.y : ext.z);
-  const float q = ex > 0.f ? c / ex * 65535.f : 0.f;
-  key[s] = (nd.id << 16) | min((uint32_t)q, 65535u);
+  key[s] = kd_key(nd.id, level, ex > 0.f ? c / ex : 0.f);
   val[s] = o;
 }
 
@@ -564,9 +563,9 @@ cudaError_t targets_build(cg_grid* g, const double* lon, const double* lat) {
 
   // levels to 128-target leaves; the first `top` of them over the whole array,
   // until a node has at most kNodeCap targets
-  int levels2 = 0, top = 0;
+  int levels2 = 0;
+  const int top = kd_top_levels(g->t128.n_tiles, kTile2, kNodeCap);
   while (((int64_t)1 << levels2) < g->t128.n_tiles) ++levels2;
-  while (((g->t128.n_tiles + ((int64_t)1 << top) - 1) >> top) * kTile2 > kNodeCap) ++top;
   float4 *u_hi = nullptr, *u_lo = nullptr;
   uint32_t *ord = nullptr, *key = nullptr, *val = nullptr, *box = nullptr;
   SortWork w;
@@ -589,7 +588,7 @@ cudaError_t targets_build(cg_grid* g, const double* lon, const double* lat) {
     k_kd_box<<<ceil_div(P, 2048), 256, 0, s>>>(u_hi, cur, (uint32_t)P, l, box);
     k_kd_keys<<<nb, 256, 0, s>>>(u_hi, cur, (uint32_t)P, l, box, key, val);
     uint32_t* sk = nullptr;
-    const int bits = 16 + l;
+    const int bits = kd_coord_bits(l) + l;
     e = radix_sort_u32(key, val, P, bits, w, s, &sk, &cur);
     g->n_launches += 2 + radix_sort_u32_launches(P, bits);
   }

@@ -58,3 +58,29 @@ int main() {
   }
 }
 """)
+
+
+def test_kd_keys_fit_32_bits(tmp_path):
+    """Up to 2^31 - 1 targets the node's number and the coordinate share 32 bits,
+    the node above the coordinate."""
+    _run(tmp_path, r"""
+int main() {
+  for (int64_t P : {(int64_t)4096, (int64_t)4097, ((int64_t)1 << 28) + 1, (int64_t)1 << 29, ((int64_t)1 << 29) + 1,
+                    (int64_t)805306368, ((int64_t)1 << 30) + 1, ((int64_t)1 << 31) - 1}) {
+    const int64_t tiles = (P + 127) / 128;
+    const int top = cg::kd_top_levels(tiles, 128, 4096);
+    CHECK(((tiles + ((int64_t)1 << top) - 1) >> top) * 128 <= 4096);
+    for (int l = 0; l < top; ++l) {
+      const int bits = cg::kd_coord_bits(l);
+      CHECK(bits >= 8 && bits <= 16 && l + bits <= 32);
+      const uint32_t last = (uint32_t)(((uint64_t)1 << l) - 1);      // the level's last node
+      for (uint32_t node : {0u, last / 2, last}) {
+        const uint64_t lo = cg::kd_key(node, l, 0.f), hi = cg::kd_key(node, l, 1.f);
+        CHECK(lo == (uint64_t)node << bits && hi == lo + (1u << bits) - 1);
+        CHECK(cg::kd_key(node, l, 0.25f) < cg::kd_key(node, l, 0.75f));
+        CHECK((hi >> (l + bits)) == 0);
+      }
+    }
+  }
+}
+""")
