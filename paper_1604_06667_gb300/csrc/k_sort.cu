@@ -716,6 +716,13 @@ cudaError_t radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int key_bi
   uint32_t* tickets = w.os_meta + kMaxPasses * kRadix;
   e = cudaMemsetAsync(w.os_meta, 0, sizeof(uint32_t) * (kMaxPasses * kRadix + kMaxPasses), s);
   if (e != cudaSuccess) return e;
+  // A captured sort replays its epochs.  Several passes write over one another's
+  // words, so a pass of the replay finds another pass's epoch; a single pass
+  // would find its own of the replay before and take old prefixes for new ones.
+  if (npass == 1) {
+    e = cudaMemsetAsync(w.status, 0, sizeof(uint64_t) * (size_t)nblk * kRadix, s);
+    if (e != cudaSuccess) return e;
+  }
   const int hblk = (int)std::min<int64_t>(ceil_div(n, kThreads * 8), 1024);
   k_os_hist<<<hblk, kThreads, 0, s>>>(keys, n, npass, ghist);
   uint32_t *kin = keys, *kout = static_cast<uint32_t*>(w.keys_alt);
