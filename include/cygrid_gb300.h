@@ -461,10 +461,11 @@ cg_status cg_batch_set_fused(cg_batch* b, int32_t fused);
 cg_status cg_batch_sync(cg_batch* b);
 
 /* Testing hook (no paper counterpart): with enable != 0 the fused FP32
- * gridder's CTAs first wait, for at most wait_cycles SM clock cycles (0: two
- * million), for a device word that nothing sets, then record ERR_TIMEOUT and
- * leave without computing, so that cg_batch_sync reports CG_ETIMEOUT without a
- * GPU fault.  Invalidates a captured graph. */
+ * gridder's CTAs (above 8 channels: one warp of each, so that the waits of its
+ * other warps run out) first wait, for about wait_cycles SM clock cycles (0:
+ * two million), for a device word that nothing sets, then record ERR_TIMEOUT
+ * and leave without results, so that cg_batch_sync reports CG_ETIMEOUT without
+ * a GPU fault.  Invalidates a captured graph. */
 cg_status cg_batch_debug_hold(cg_batch* b, int32_t enable, int64_t wait_cycles);
 
 /* Release the graph, branch streams and events (not the jobs' handles). */

@@ -56,6 +56,7 @@ struct WideArgs {
   int n_rows;               // samples (rows of the data tensor)
   int n_slabs;
   int vec_out;              // the map's rows take 16-byte stores
+  long long wait_cycles;    // limit of the waits (SM clock)
   WeightConst kc;
 };
 
@@ -99,24 +100,23 @@ __device__ __forceinline__ void mbar_arrive_tx(uint64_t* b, uint32_t bytes) {
                : "memory");
 }
 
-// Bounded wait for the phase of the given parity (~1 s of SM clock): false on
-// time-out or once another warp has given up.
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
+// Bounded wait of a warp for the phase of the given parity: false when the wait
+// ran out or another warp has given up.  The lanes decide together, so that they
+// stay together for the votes and barriers that follow.
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, long long limit) {
   const uint32_t a = su32(b);
-  const long long t0 = clock64();
+  long long t0 = 0;
   for (uint32_t it = 0;; ++it) {
     uint32_t done;
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
-        "selp.u32 %0, 1, 0, p;\n}"
+        "vote.sync.all.pred p, p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}"
         : "=r"(done)
         : "r"(a), "r"(parity), "r"(20000u)
         : "memory");
     if (done) return true;
-    if ((it & 3u) == 3u) {
-      if (*abort_flag) return false;
-      if (clock64() - t0 > 2000000000LL) return false;
-    }
+    if (it == 0) t0 = clock64();
+    if ((it & 3u) == 3u && __any_sync(0xffffffffu, *abort_flag || clock64() - t0 > limit)) return false;
   }
 }
 
@@ -130,7 +130,6 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
   extern __shared__ __align__(128) unsigned char raw[];
   typename SH::Smem& S = *reinterpret_cast<typename SH::Smem*>(raw);
   const GridArgs& a = wa.g;
-  if (a.hold && hold_gives_up(a.hold, a.hold_cycles, a.err)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t tile = blockIdx.x;
   const int slab = blockIdx.y, split = blockIdx.z;
@@ -215,8 +214,8 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
   // ---- channel rows of chunk q (its records are there) ----
   auto stage_rows = [&](int q) -> bool {
     const int st = q % NS, rs = q % SH::RR;
-    if (!mbar_wait(&S.rfull[rs], (q / SH::RR) & 1, abort_flag)) return false;
-    if (q >= NS && !mbar_wait(&S.empty[st], ((q / NS) - 1) & 1, abort_flag)) return false;
+    if (!mbar_wait(&S.rfull[rs], (q / SH::RR) & 1, abort_flag, wa.wait_cycles)) return false;
+    if (q >= NS && !mbar_wait(&S.empty[st], ((q / NS) - 1) & 1, abort_flag, wa.wait_cycles)) return false;
     if (wa.rows_mode == kRowsTma) {
       // lane j gathers the rows of candidates 4 j .. 4 j + 3 (padding: past the
       // last row, zeros)
@@ -317,8 +316,16 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
   unsigned npair = 0;
 
   bool ok = true;
+  if (a.hold && warp == 0) {
+    // testing hook: this warp stages nothing until a word that nothing sets, so
+    // that the other warps' waits run out
+    const long long t0 = clock64();
+    while (*((volatile const int*)a.hold) == 0 && !*abort_flag && clock64() - t0 < 4 * a.hold_cycles)
+      __nanosleep(1000);
+    ok = __all_sync(0xffffffffu, *((volatile const int*)a.hold) != 0);
+  }
   int mine = -1;                  // the last chunk whose rows this warp staged
-  for (int q = warp; q < SH::RA && q < n_chunks; q += NW) stage_records(q);
+  for (int q = warp; ok && q < SH::RA && q < n_chunks; q += NW) stage_records(q);
   for (int q = 0; q < AHEAD && q < n_chunks && ok; ++q)
     if (q % NW == warp) {
       ok = stage_rows(q);
@@ -331,13 +338,13 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
       ok = stage_rows(q + AHEAD);
       if (ok) mine = q + AHEAD;
     }
-    if (!ok || !mbar_wait(&S.full[st], (q / NS) & 1, abort_flag)) {
+    if (!ok || !mbar_wait(&S.full[st], (q / NS) & 1, abort_flag, wa.wait_cycles)) {
       // gave up: own copies have to land before the CTA ends
       set_error(a.err, ERR_TIMEOUT);
       *abort_flag = 1;
       int no_abort = 0;
-      if (mine >= 0) mbar_wait(&S.full[mine % NS], (mine / NS) & 1, &no_abort);
-      break;
+      if (mine >= 0) mbar_wait(&S.full[mine % NS], (mine / NS) & 1, &no_abort, wa.wait_cycles);
+      return;   // without results: the call reports the time-out
     }
     // ---- list the candidates in reach of the warp's targets (a sample of
     // weight zero is listed too, for the pair count) ----
@@ -583,6 +590,7 @@ cudaError_t grid_wide(const GridArgs& a, const Tiling& t, int64_t n, int dtype, 
   wa.g = a;
   wa.range_c = t.range_c;
   wa.n_rows = (int)n;
+  wa.wait_cycles = a.hold ? a.hold_cycles : 2000000000LL;   // ~1 s
   wa.kc = weight_const(a.kd);
   const int cp = wide_cpad(a.C);
   wa.n_slabs = (a.C + cp - 1) / cp;
