@@ -174,7 +174,7 @@ struct cg_grid {
   int32_t* tix_ring_off = nullptr;  // [4 nside + 1]
   float* tix_rows = nullptr;      // map rows in the index's order, times 1 / W
   size_t tix_rows_cap = 0;
-  uint32_t* tix_dirty = nullptr;  // set when a map holds non-finite values
+  uint32_t* tix_dirty = nullptr;  // set when a map holds values that the general kernel has to take
   cg::SortWork tix_sw;
   // scratch accumulators of cg_grid_dsigma (w' = dw/dsigma pass)
   float* ds_num = nullptr;        // [slots][C]
@@ -465,7 +465,7 @@ struct AdjointArgs {
   float* out;               // [N][C]
   int interp;
   float* vsum;              // [N] or null (interpolation)
-  uint32_t* dirty;          // set when the map holds non-finite values
+  uint32_t* dirty;          // set when the general kernel has to take the map
 };
 int adjoint_cpad(int C);
 cudaError_t grid_adjoint(AdjointArgs a, const float* y, const float* wmap, const float2* acc_w,

@@ -475,10 +475,19 @@ __global__ void __launch_bounds__(kNTh, 2) k_adjoint_wide(const __grid_constant_
   }
 }
 
+// Whether v = x / W of a target leaves the range in which sums over v and then the
+// sample's weight give what sums over w omega / W x give: too large, as for a
+// small W (0 x inf would reach other samples of the strip), or small because of
+// a large W, so that products with w fall below the normal numbers.  (An ordinary
+// W leaves small map values alone, such as the tails of a model's sources.)
+__device__ __forceinline__ bool out_of_range(float v, float x, float iw) {
+  return !(fabsf(v) <= 0x1p100f) || (iw < 0x1p-20f && x != 0.f && fabsf(v) < 0x1p-100f);
+}
+
 // Rows of the map in the order of the sorted target index, times 1 / W_p (0
 // where W_p <= 0 or not finite) or as they are (interpolation), padded to cpad
-// channels.  Non-finite values become 0 and set *dirty: the general kernel
-// then computes the result again.
+// channels.  Non-finite or out-of-range values become 0 and set *dirty: the
+// general kernel then computes the result again.
 __global__ void __launch_bounds__(256) k_adjoint_rows(const float* __restrict__ y, int C, int cpad,
                                                       const uint32_t* __restrict__ t_slot,
                                                       const uint32_t* __restrict__ perm,
@@ -497,7 +506,7 @@ __global__ void __launch_bounds__(256) k_adjoint_rows(const float* __restrict__ 
     if (iw != 0.f) {
       const float x = y[(size_t)u * C + c];
       v = iw * x;
-      if (!isfinite(x)) {
+      if (interp ? !isfinite(x) : out_of_range(v, x, iw)) {
         v = 0.f;
         *dirty = 1u;
       }

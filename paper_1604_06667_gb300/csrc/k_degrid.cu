@@ -10,7 +10,7 @@
 //            sample index of k_healpix.cu, built for the targets once per
 //            cg_set_kernel);
 //   circular kernels: k_adjoint.cu; the general kernel below serves the
-//            elliptical kernel and maps with non-finite values:
+//            elliptical kernel and maps with non-finite or out-of-range values:
 //   samples  one warp per 32 consecutive sorted samples of the last add (a
 //            compact strip of one HEALPix ring); its bounding disc, widened by
 //            the support, is queried ring by ring (the per-ring intervals of
@@ -403,7 +403,7 @@ cudaError_t grid_degrid(cg_grid* g, const float* y, const float* wmap, float* ou
   if (a.n == 0) return cudaGetLastError();
   if (g->kernel_type != CG_GAUSS2D) {
     // circular kernels: the tiled gather; the general kernel below then only
-    // runs where the map holds non-finite values
+    // runs where the map holds non-finite or out-of-range values
     AdjointArgs t;
     t.ns = g->nside;
     t.skey = a.skey;
