@@ -21,6 +21,13 @@ CG_HD int wide_shares(int total, int n_split) {
   return s < 1 ? 1 : (s < n_split ? s : n_split);
 }
 
+// Chunks of kc candidates between two folds of the wide form's sums: a tile's
+// `total` candidates in n_fold parts, of at least two chunks.
+CG_HD int wide_fold_chunks(int total, int n_fold, int kc) {
+  const int64_t part = (int64_t)n_fold * kc, k = (total + part - 1) / part;
+  return k < 2 ? 2 : (int)k;
+}
+
 // Partial sums of a slot: the shares of its tile, 0 for an empty slot.  Slots
 // come in whole 128-target tiles, candidate counts in 64-target tiles that hold
 // at least one target, so an empty slot's tile may lie past the last count: it

@@ -301,6 +301,7 @@ struct GridArgs {
   // CTAs that write partial sums, summed by k_split_reduce in split order
   const int32_t* tile_cand;
   int n_split;
+  int n_fold;           // (wide form) parts of a tile's candidates that are summed apart
   int64_t n_slots;
   float* part_num;      // [n_split][slots][C]
   float2* part_w;       // [n_split][slots]

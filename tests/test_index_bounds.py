@@ -84,3 +84,19 @@ int main() {
   }
 }
 """)
+
+
+def test_folds_keep_chains_short(tmp_path):
+    """Parts of a tile's candidates that are summed apart: no longer than a share
+    of n_fold equal ones rounded up to chunks (or two chunks), for any total."""
+    _run(tmp_path, r"""
+int main() {
+  for (int total : {0, 1, 63, 64, 65, 200, 1000, 4097, 1 << 20, 2147483647})
+    for (int n : {2, 3, 29, 64}) {
+      const int64_t k = cg::wide_fold_chunks(total, n, 32);
+      CHECK(k >= 2);
+      CHECK(k * 32 * n >= total);
+      CHECK(k == 2 || (k - 1) * 32 * n < total);
+    }
+}
+""")
