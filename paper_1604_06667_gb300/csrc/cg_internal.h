@@ -329,7 +329,7 @@ cudaError_t grid_tiles_f32(cg_grid* g, const void* data, int dtype, float* out =
 constexpr int kNarrowMaxC = 8;
 int narrow_width(int C);
 int narrow_splits(int64_t n_tiles, int64_t n, int n_sms);
-cudaError_t grid_narrow(const GridArgs& a, const Tiling& t, int64_t n, int dtype, float* rows,
+cudaError_t grid_narrow(const GridArgs& a, const Tiling& t, int64_t n, int dtype, float* rows, int n_sms,
                         cudaStream_t s);
 // k_grid_wide.cu -- more than 8 channels: warps over compact target groups and
 // all channels of a slab.

@@ -842,7 +842,7 @@ cudaError_t run_narrow(cg_grid* g, GridArgs& a, int dtype, bool* direct, bool* k
   a.keep = sums_kept(nt, a.C, sm_count());
   cudaError_t e = begin_pass(g, a, 1, direct, kept);
   if (e == cudaSuccess) e = grid_narrow(a, g->t64, g->last_n, dtype, own_rows ? g->rows : nullptr,
-                                         g->stream);
+                                         sm_count(), g->stream);
   if (e != cudaSuccess) return e;
   g->n_launches += own_rows ? 1 : 0;   // the rows' gather
   return end_pass(g, a, dtype, cw, 1, true);

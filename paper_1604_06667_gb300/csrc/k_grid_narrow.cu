@@ -69,6 +69,7 @@ struct NarrowArgs {
   const int32_t* range_c;              // the tile's candidates before each range
   const float* rows;                   // [n][CN] channel values in sorted order (null: CN = 1
                                        // and the values came with the index, in s_lo.w)
+  bool sparse;                         // few candidates per tile (k_grid_sparse)
   WeightConst kc;
 };
 
@@ -100,6 +101,275 @@ __device__ __forceinline__ float2 lds2(uint32_t p) {
   return v;
 }
 
+// A candidate's channel values: row s of rows (null: one channel, in the record).
+template <int CN>
+__device__ __forceinline__ void load_row(const float* rows, int64_t s, float in_rec, float (&d)[CN]) {
+  const float* row = rows + (size_t)s * CN;
+  if constexpr (CN == 1) {
+    d[0] = rows ? row[0] : in_rec;
+  } else if constexpr (CN == 2) {
+    const float2 q = *reinterpret_cast<const float2*>(row);
+    d[0] = q.x; d[1] = q.y;
+  } else {
+#pragma unroll
+    for (int k = 0; k < CN; k += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(row + k);
+      d[k] = q.x; d[k + 1] = q.y; d[k + 2] = q.z; d[k + 3] = q.w;
+    }
+  }
+}
+
+// A group's targets 2 lane, 2 lane + 1 (lane < 4) as a packed pair: vectors and, for
+// the elliptical kernel, axis directions.
+template <int FORM>
+__device__ __forceinline__ void load_pair(const GridArgs& a, float2* A, int64_t sa) {
+  const float4 p = a.tgt_a[sa], q = a.tgt_a[sa + 1];
+  A[0] = make_float2(p.x, q.x);
+  A[1] = make_float2(p.y, q.y);
+  A[2] = make_float2(p.z, q.z);
+  if (FORM != kWGauss1 && FORM != kWGauss1Ds && a.kd.type == CG_GAUSS2D) {
+    const float4 f1a = a.tgt_f1[sa], f1b = a.tgt_f1[sa + 1];
+    const float4 f2a = a.tgt_f2[sa], f2b = a.tgt_f2[sa + 1];
+    A[4] = make_float2(f1a.x, f1b.x);
+    A[5] = make_float2(f1a.y, f1b.y);
+    A[6] = make_float2(f1a.z, f1b.z);
+    A[7] = make_float2(f2a.x, f2b.x);
+    A[8] = make_float2(f2a.y, f2b.y);
+    A[9] = make_float2(f2a.z, f2b.z);
+  }
+}
+
+// Disc of a group of 8 targets (p: target lane & 7; empty slots sit at (4, 4, 4)),
+// widened by the support: centre and squared reach (chords; -1: no target).
+__device__ __forceinline__ float4 group_reach(float4 p, float c2_out) {
+  const bool on = p.x < 3.f;
+  float sx = on ? p.x : 0.f, sy = on ? p.y : 0.f, sz = on ? p.z : 0.f, sn = on ? 1.f : 0.f;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    sx += __shfl_xor_sync(0xffffffffu, sx, o);
+    sy += __shfl_xor_sync(0xffffffffu, sy, o);
+    sz += __shfl_xor_sync(0xffffffffu, sz, o);
+    sn += __shfl_xor_sync(0xffffffffu, sn, o);
+  }
+  const float inv = sn > 0.f ? 1.f / sn : 0.f;
+  const float gx = sx * inv, gy = sy * inv, gz = sz * inv;
+  const float ex = p.x - gx, ey = p.y - gy, ez = p.z - gz;
+  float rad2 = on ? ex * ex + ey * ey + ez * ez : 0.f;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) rad2 = fmaxf(rad2, __shfl_xor_sync(0xffffffffu, rad2, o));
+  const float reach = sqrtf(rad2) + sqrtf(c2_out);
+  return make_float4(gx, gy, gz, sn > 0.f ? reach * reach * 1.0001f + 1e-12f : -1.f);
+}
+
+// A lane's sums over its candidates: 8 targets as 4 packed pairs.
+template <int CN>
+struct LaneSums {
+  float2 acc[CN][4], ws[4], wc[4];
+  unsigned npair;
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      ws[j] = wc[j] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < CN; ++c) acc[c][j] = make_float2(0.f, 0.f);
+    }
+    npair = 0;
+  }
+};
+
+// The warp's list of the first n candidates (32 at a time) in reach of its group;
+// their number.
+__device__ __forceinline__ int list_near(const float4* rec, int n, float4 g, uint16_t* list) {
+  const int lane = threadIdx.x & 31;
+  int cnt = 0;
+#pragma unroll 8
+  for (int b = 0; b < n; b += 32) {
+    const float4 p = rec[b + lane];
+    const float ex = p.x - g.x, ey = p.y - g.y, ez = p.z - g.z;
+    const bool in = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= g.w;
+    const uint32_t m = __ballot_sync(0xffffffffu, in);
+    if (in) list[cnt + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(b + lane);
+    cnt += __popc(m);
+  }
+  __syncwarp();
+  return cnt;
+}
+
+// Weights and sums of cnt listed candidates, 32 at a time; pair_s: the group's
+// packed pairs, tv and slot0: its targets.
+template <int CN, int FORM>
+__device__ __forceinline__ void add_listed(const NarrowArgs& na, LaneSums<CN>& L, const uint16_t* list, int cnt,
+                                           const float4* rec, const float* dat, const uint32_t* idx,
+                                           uint32_t pair_s, const float4* tv, int64_t slot0) {
+  const GridArgs& a = na.g;
+  const WeightConst& kc = na.kc;
+  const int lane = threadIdx.x & 31;
+  for (int b = 0; b < cnt; b += 32) {
+    float4 p = make_float4(-4.f, -4.f, -4.f, 0.f);
+    int ci = 0;
+    float d[CN];
+#pragma unroll
+    for (int k = 0; k < CN; ++k) d[k] = 0.f;
+    if (b + lane < cnt) {
+      ci = list[b + lane];
+      p = rec[ci];
+#pragma unroll
+      for (int k = 0; k < CN; ++k) d[k] = dat[ci * CN + k];
+    }
+    const float2 nx = f2(-p.x), ny = f2(-p.y), nz = f2(-p.z), om = f2(p.w);
+    float2 w[4];
+    float near = INFINITY;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      // read for every batch: held in registers they would be spilled
+      const uint32_t q6 = pair_s + j * (uint32_t)(10 * sizeof(float2));
+      const float4 xy = lds4(q6);
+      const float2 dx = __fadd2_rn(make_float2(xy.x, xy.y), nx);
+      const float2 dy = __fadd2_rn(make_float2(xy.z, xy.w), ny);
+      const float2 dz = __fadd2_rn(lds2(q6 + 16), nz);
+      const float2 c2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+      Axes2 A{};
+      if (FORM != kWGauss1 && FORM != kWGauss1Ds) {
+        const float4 u0 = lds4(q6 + 32), u1 = lds4(q6 + 48), u2 = lds4(q6 + 64);
+        A.ax = make_float2(u0.x, u0.y); A.ay = make_float2(u0.z, u0.w);
+        A.az = make_float2(u1.x, u1.y); A.bx = make_float2(u1.z, u1.w);
+        A.by = make_float2(u2.x, u2.y); A.bz = make_float2(u2.z, u2.w);
+      }
+      const float2 v = __fmul2_rn(weight2<FORM>(kc, a.kd, c2, dx, dy, dz, A), om);
+      const bool i0 = c2.x <= kc.c2_out, i1 = c2.y <= kc.c2_out;
+      // outside the support: -0.0 adds nothing to any finite sum
+      w[j] = make_float2(i0 ? v.x : -0.f, i1 ? v.y : -0.f);
+      L.npair += (i0 ? 1u : 0u) + (i1 ? 1u : 0u);
+      near = band_near(kc, c2, near);
+    }
+    if (near <= kc.hw) {
+      const uint32_t kill = narrow_band(tv, p, a.tgt_ll + slot0, a.sll[idx[ci]],
+                                        a.kd.c2_in, a.kd.c2_out, a.kd.c2r_hi, a.kd.c2r_lo,
+                                        a.kd.c2r_tol, a.kd.r_rad);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (kill & (1u << (2 * j))) { w[j].x = -0.f; --L.npair; }
+        if (kill & (2u << (2 * j))) { w[j].y = -0.f; --L.npair; }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      kahan2(L.ws[j], L.wc[j], w[j]);
+#pragma unroll
+      for (int k = 0; k < CN; ++k) L.acc[k][j] = __ffma2_rn(w[j], f2(d[k]), L.acc[k][j]);
+    }
+  }
+}
+
+// Sum over the lanes of 8 targets' values: every step halves the targets a lane
+// holds, keeping those of its lane bit; lanes 4 t .. 4 t + 3 end with target t.
+__device__ __forceinline__ float lanes_sum(const float2 (&v)[4]) {
+  const int lane = threadIdx.x & 31;
+  float x[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) x[t] = (t & 1) ? v[t >> 1].y : v[t >> 1].x;
+#pragma unroll
+  for (int o = 16, half = 4; half > 0; o >>= 1, half >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const float keep = up ? x[i + half] : x[i], send = up ? x[i] : x[i + half];
+      x[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  x[0] += __shfl_xor_sync(0xffffffffu, x[0], 2);
+  return x[0] + __shfl_xor_sync(0xffffffffu, x[0], 1);
+}
+// The same for compensated sums.
+__device__ __forceinline__ float2 lanes_comp(const float2 (&s)[4], const float2 (&c)[4]) {
+  const int lane = threadIdx.x & 31;
+  float x[8], y[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    x[t] = (t & 1) ? s[t >> 1].y : s[t >> 1].x;
+    y[t] = (t & 1) ? c[t >> 1].y : c[t >> 1].x;
+  }
+#pragma unroll
+  for (int o = 16, half = 4; half > 0; o >>= 1, half >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const float xs = up ? x[i] : x[i + half], ys = up ? y[i] : y[i + half];
+      const float xr = __shfl_xor_sync(0xffffffffu, xs, o), yr = __shfl_xor_sync(0xffffffffu, ys, o);
+      x[i] = up ? x[i + half] : x[i];
+      y[i] = up ? y[i + half] : y[i];
+      comp_add(x[i], y[i], xr, yr);
+    }
+  }
+#pragma unroll
+  for (int o = 2; o > 0; o >>= 1)
+    comp_add(x[0], y[0], __shfl_xor_sync(0xffffffffu, x[0], o), __shfl_xor_sync(0xffffffffu, y[0], o));
+  return make_float2(x[0], y[0]);
+}
+
+// A target's sums into the one-shot map, the accumulators or a share's partial
+// sums.
+template <int CN>
+__device__ __forceinline__ void write_target(const GridArgs& a, int64_t slot, float wsum, float wcor,
+                                             const float (&num)[CN], int split) {
+  const uint32_t u = a.tgt_perm[slot];
+  if (u == 0xffffffffu) return;
+  // A non-finite channel value of a candidate outside the support reaches the
+  // target through 0 x NaN: such rows are computed again by the fix-up pass
+  // with only the pairs inside the support.
+  float chk = 0.f;
+#pragma unroll
+  for (int k = 0; k < CN; ++k) chk += num[k];
+  const bool bad = !isfinite(chk);
+  if (bad) {
+    atomicOr(&a.nf_bits[slot >> 5], 1u << (slot & 31));
+    atomicOr(a.nf_any, 1u);
+  }
+  if (a.out) {
+    const float W = wsum + wcor;
+    if (a.out_w) a.out_w[u] = W;
+    if (!bad) {
+#pragma unroll
+      for (int k = 0; k < CN; ++k)
+        if (k < a.C) a.out[(size_t)u * a.C + k] = (W > 0.f) ? num[k] / W : __int_as_float(0x7fc00000);
+    }
+    if (!a.keep) return;
+  }
+  const bool splits = a.n_split > 1;
+  if (!bad) {
+    float* dst = splits ? a.part_num + ((size_t)split * a.n_slots + slot) * a.C
+                        : a.acc_num + (size_t)slot * a.C;
+    const bool add = a.accumulate && !splits;
+#pragma unroll
+    for (int k = 0; k < CN; ++k)
+      if (k < a.C) dst[k] = add ? dst[k] + num[k] : num[k];
+  }
+  if (splits) {
+    a.part_w[(size_t)split * a.n_slots + slot] = make_float2(wsum, wcor);
+    return;
+  }
+  float2 old = a.accumulate ? a.acc_w[slot] : make_float2(0.f, 0.f);
+  comp_add(old.x, old.y, wsum, wcor);
+  a.acc_w[slot] = old;
+}
+
+// Adds up the lanes' sums and writes the group's targets.
+template <int CN>
+__device__ __forceinline__ void write_group(const NarrowArgs& na, LaneSums<CN>& L, int64_t slot0, int split) {
+  const GridArgs& a = na.g;
+  const int lane = threadIdx.x & 31;
+  const float2 w = lanes_comp(L.ws, L.wc);
+  const float wsum = w.x, wcor = w.y;
+  float num[CN];
+#pragma unroll
+  for (int k = 0; k < CN; ++k) num[k] = lanes_sum(L.acc[k]);
+  unsigned npair = __reduce_add_sync(0xffffffffu, L.npair);
+  if (lane == 0 && npair && a.pairs) atomicAdd(a.pairs, (unsigned long long)npair);
+  if (lane & 3) return;
+  const int64_t slot = slot0 + (lane >> 2);
+  write_target<CN>(a, slot, wsum, wcor, num, split);
+}
+
 template <int CN, int FORM>
 __global__ void __launch_bounds__(kNTh, CN <= 2 ? 3 : 2)
     k_grid_narrow(const __grid_constant__ NarrowArgs na) {
@@ -111,62 +381,14 @@ __global__ void __launch_bounds__(kNTh, CN <= 2 ? 3 : 2)
   const int split = blockIdx.z;
   const int64_t slot0 = tile * kTile + warp * kNG;   // the warp's first target
   const float4 chi = a.tile_chi[tile], clo = a.tile_clo[tile];
-  const WeightConst& kc = na.kc;
-
   const uint32_t pair_s = (uint32_t)__cvta_generic_to_shared(&S.pair[warp][0][0]);
   // ---- the warp's targets: packed pairs in shared memory (read by all lanes
   // at once); centre and reach of the group (empty slots sit at (4, 4, 4)) ----
   if (tid < kTile) S.tv[tid] = a.tgt_a[tile * kTile + tid];
-  if (lane < 4) {
-    float2* A = S.pair[warp][lane];
-    const int64_t sa = slot0 + 2 * lane;
-    const float4 p = a.tgt_a[sa], q = a.tgt_a[sa + 1];
-    A[0] = make_float2(p.x, q.x);
-    A[1] = make_float2(p.y, q.y);
-    A[2] = make_float2(p.z, q.z);
-    if (FORM != kWGauss1 && FORM != kWGauss1Ds && a.kd.type == CG_GAUSS2D) {
-      const float4 f1a = a.tgt_f1[sa], f1b = a.tgt_f1[sa + 1];
-      const float4 f2a = a.tgt_f2[sa], f2b = a.tgt_f2[sa + 1];
-      A[4] = make_float2(f1a.x, f1b.x);
-      A[5] = make_float2(f1a.y, f1b.y);
-      A[6] = make_float2(f1a.z, f1b.z);
-      A[7] = make_float2(f2a.x, f2b.x);
-      A[8] = make_float2(f2a.y, f2b.y);
-      A[9] = make_float2(f2a.z, f2b.z);
-    }
-  }
-  float gx, gy, gz, reach2;
-  {
-    const float4 p = a.tgt_a[slot0 + (lane & 7)];   // four copies of the group
-    const bool on = p.x < 3.f;
-    float sx = on ? p.x : 0.f, sy = on ? p.y : 0.f, sz = on ? p.z : 0.f, sn = on ? 1.f : 0.f;
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-      sx += __shfl_xor_sync(0xffffffffu, sx, o);
-      sy += __shfl_xor_sync(0xffffffffu, sy, o);
-      sz += __shfl_xor_sync(0xffffffffu, sz, o);
-      sn += __shfl_xor_sync(0xffffffffu, sn, o);
-    }
-    const float inv = sn > 0.f ? 1.f / sn : 0.f;
-    gx = sx * inv;
-    gy = sy * inv;
-    gz = sz * inv;
-    const float ex = p.x - gx, ey = p.y - gy, ez = p.z - gz;
-    float rad2 = on ? ex * ex + ey * ey + ez * ez : 0.f;
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) rad2 = fmaxf(rad2, __shfl_xor_sync(0xffffffffu, rad2, o));
-    const float reach = sqrtf(rad2) + sqrtf(a.kd.c2_out);
-    reach2 = sn > 0.f ? reach * reach * 1.0001f + 1e-12f : -1.f;
-  }
-
-  float2 acc[CN][4], ws[4], wc[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    ws[j] = wc[j] = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int c = 0; c < CN; ++c) acc[c][j] = make_float2(0.f, 0.f);
-  }
-  unsigned npair = 0;
+  if (lane < 4) load_pair<FORM>(a, S.pair[warp][lane], slot0 + 2 * lane);
+  const float4 near = group_reach(a.tgt_a[slot0 + (lane & 7)], a.kd.c2_out);   // four copies of the group
+  LaneSums<CN> L;
+  L.clear();
 
   const int64_t r0 = a.range_off[tile], r1 = a.range_off[tile + 1];
   int c_lo = 0, c_hi = 0x7fffffff;
@@ -220,19 +442,7 @@ __global__ void __launch_bounds__(kNTh, CN <= 2 ? 3 : 2)
         c.h = a.s_hi[s];
         c.l = a.s_lo[s];
         c.idx = a.perm[s];
-        const float* row = na.rows + (size_t)s * CN;
-        if constexpr (CN == 1) {
-          c.d[0] = na.rows ? row[0] : c.l.w;
-        } else if constexpr (CN == 2) {
-          const float2 q = *reinterpret_cast<const float2*>(row);
-          c.d[0] = q.x; c.d[1] = q.y;
-        } else {
-#pragma unroll
-          for (int k = 0; k < CN; k += 4) {
-            const float4 q = *reinterpret_cast<const float4*>(row + k);
-            c.d[k] = q.x; c.d[k + 1] = q.y; c.d[k + 2] = q.z; c.d[k + 3] = q.w;
-          }
-        }
+        load_row<CN>(na.rows, s, c.l.w, c.d);
       }
       return c;
     };
@@ -255,144 +465,182 @@ __global__ void __launch_bounds__(kNTh, CN <= 2 ? 3 : 2)
         put(pre, st ^ 1);
         if (q + 2 < n_steps) pre = fetch(v_lo + (q + 2) * kNTh);
       }
-      // ---- list the candidates in reach of the warp's targets ----
-      int cnt = 0;
-#pragma unroll
-      for (int b = 0; b < kNTh / 32; ++b) {
-        const float4 p = S.rec[st][32 * b + lane];
-        const float ex = p.x - gx, ey = p.y - gy, ez = p.z - gz;
-        const bool in = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= reach2;
-        const uint32_t m = __ballot_sync(0xffffffffu, in);
-        if (in) S.list[warp][cnt + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(32 * b + lane);
-        cnt += __popc(m);
-      }
-      __syncwarp();
-      // ---- weights and sums, 32 listed candidates at a time ----
-      for (int b = 0; b < cnt; b += 32) {
-        float4 p = make_float4(-4.f, -4.f, -4.f, 0.f);
-        int ci = 0;
-        float d[CN];
-#pragma unroll
-        for (int k = 0; k < CN; ++k) d[k] = 0.f;
-        if (b + lane < cnt) {
-          ci = S.list[warp][b + lane];
-          p = S.rec[st][ci];
-#pragma unroll
-          for (int k = 0; k < CN; ++k) d[k] = S.dat[st][ci * CN + k];
-        }
-        const float2 nx = f2(-p.x), ny = f2(-p.y), nz = f2(-p.z), om = f2(p.w);
-        float2 w[4];
-        float near = INFINITY;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          // read for every batch: held in registers they would be spilled
-          const uint32_t q6 = pair_s + j * (uint32_t)sizeof(S.pair[0][0]);
-          const float4 xy = lds4(q6);
-          const float2 dx = __fadd2_rn(make_float2(xy.x, xy.y), nx);
-          const float2 dy = __fadd2_rn(make_float2(xy.z, xy.w), ny);
-          const float2 dz = __fadd2_rn(lds2(q6 + 16), nz);
-          const float2 c2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-          Axes2 A{};
-          if (FORM != kWGauss1 && FORM != kWGauss1Ds) {
-            const float4 u0 = lds4(q6 + 32), u1 = lds4(q6 + 48), u2 = lds4(q6 + 64);
-            A.ax = make_float2(u0.x, u0.y); A.ay = make_float2(u0.z, u0.w);
-            A.az = make_float2(u1.x, u1.y); A.bx = make_float2(u1.z, u1.w);
-            A.by = make_float2(u2.x, u2.y); A.bz = make_float2(u2.z, u2.w);
-          }
-          const float2 v = __fmul2_rn(weight2<FORM>(kc, a.kd, c2, dx, dy, dz, A), om);
-          const bool i0 = c2.x <= kc.c2_out, i1 = c2.y <= kc.c2_out;
-          // outside the support: -0.0 adds nothing to any finite sum
-          w[j] = make_float2(i0 ? v.x : -0.f, i1 ? v.y : -0.f);
-          npair += (i0 ? 1u : 0u) + (i1 ? 1u : 0u);
-          near = band_near(kc, c2, near);
-        }
-        if (near <= kc.hw) {
-          const uint32_t kill = narrow_band(S.tv + warp * kNG, p, a.tgt_ll + slot0, a.sll[S.idx[st][ci]],
-                                            a.kd.c2_in, a.kd.c2_out, a.kd.c2r_hi, a.kd.c2r_lo,
-                                            a.kd.c2r_tol, a.kd.r_rad);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (kill & (1u << (2 * j))) { w[j].x = -0.f; --npair; }
-            if (kill & (2u << (2 * j))) { w[j].y = -0.f; --npair; }
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          kahan2(ws[j], wc[j], w[j]);
-#pragma unroll
-          for (int k = 0; k < CN; ++k) acc[k][j] = __ffma2_rn(w[j], f2(d[k]), acc[k][j]);
-        }
-      }
+      const int cnt = list_near(S.rec[st], min(kNTh, v_hi - v_lo - q * kNTh), near, S.list[warp]);
+      add_listed<CN, FORM>(na, L, S.list[warp], cnt, S.rec[st], S.dat[st], S.idx[st], pair_s, S.tv + warp * kNG, slot0);
       __syncthreads();   // the stage may be rewritten; the next one is visible
     }
   }
 
-  // ---- the lanes' sums ----
-  float wsum = 0.f, wcor = 0.f, num[CN];
-#pragma unroll
-  for (int k = 0; k < CN; ++k) num[k] = 0.f;
-#pragma unroll
-  for (int t = 0; t < kNG; ++t) {
-    float s = (t & 1) ? ws[t >> 1].y : ws[t >> 1].x;
-    float c = (t & 1) ? wc[t >> 1].y : wc[t >> 1].x;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
-      comp_add(s, c, s2, c2);
+  write_group(na, L, slot0, split);
+}
+
+// The same for tiles of few candidates.  A tile is some five dependent loads and
+// little work, so what counts is how many run at a time: two warps per tile
+// (twelve tiles per SM against three).  Up to 64 candidates, lanes over targets:
+// no list, no sums over lanes.  More: four groups per warp, one after the other
+// on candidates that are staged once (above 128: again for every group).
+// Measured on GB300 per call, one channel, gauss1d, onto 2048 x 1024 targets of
+// the whole sky: 1e5 samples 559 -> 187 us (register-blocked form 280), 3e5 594 ->
+// 244 (413); 1e6 x 7 1290 -> 928 (927); 8,000 x 3 onto 500 x 500 129 -> 72 (72).
+constexpr int kSpTh = 64, kSpStep = 128, kSpRanges = 128;
+constexpr int kSpDirect = 64;   // tiles of so few candidates: a lane per target
+template <int CN>
+struct SparseSmem {
+  float4 rec[kSpStep];
+  alignas(16) float dat[kSpStep * CN];
+  uint32_t idx[kSpStep];
+  float4 tv[kTile];
+  alignas(16) float2 pair[kTile / kNG][4][10];
+  uint16_t list[kSpTh / 32][kSpStep];
+  int2 rg[kSpRanges];
+  int rg_c[kSpRanges];
+};
+
+template <int CN, int FORM>
+__global__ void __launch_bounds__(kSpTh, CN <= 2 ? 12 : 8) k_grid_sparse(const __grid_constant__ NarrowArgs na) {
+  __shared__ SparseSmem<CN> S;
+  const GridArgs& a = na.g;
+  if (a.hold && hold_gives_up(a.hold, a.hold_cycles, a.err)) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t tile = blockIdx.x;
+  const float4 chi = a.tile_chi[tile], clo = a.tile_clo[tile];
+  const int total = a.tile_cand[tile];
+  const int64_t r0 = a.range_off[tile];
+  const int nr = (int)(a.range_off[tile + 1] - r0);
+  const bool rg_in = nr <= kSpRanges;   // more are searched in global memory
+  if (rg_in)
+    for (int r = tid; r < nr; r += kSpTh) {
+      S.rg[r] = a.range_s[r0 + r];
+      S.rg_c[r] = na.range_c[r0 + r];
     }
-    if (lane == t) { wsum = s; wcor = c; }
+  S.tv[tid] = a.tgt_a[tile * kTile + tid];
+  if (lane < 16) {
+    const int p = 16 * warp + lane;   // pair of the tile
+    load_pair<FORM>(a, S.pair[p >> 2][p & 3], tile * kTile + 2 * p);
+  }
+  __syncthreads();
+
+  auto stage = [&](int v0) {
+    for (int i = tid; i < kSpStep; i += kSpTh) {
+      const int v = v0 + i;
+      // padding lies far from every target and from the empty slots
+      float4 rec = make_float4(-4.f, -4.f, -4.f, 0.f);
+      float d[CN];
 #pragma unroll
-    for (int k = 0; k < CN; ++k) {
-      float v = (t & 1) ? acc[k][t >> 1].y : acc[k][t >> 1].x;
+      for (int k = 0; k < CN; ++k) d[k] = 0.f;
+      if (v < total) {
+        int lo = 0, hi = nr - 1;   // last range with so many candidates before it
+        int64_t s;
+        if (rg_in) {
+          while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (S.rg_c[mid] <= v) lo = mid; else hi = mid - 1;
+          }
+          s = S.rg[lo].x + (v - S.rg_c[lo]);
+        } else {
+          while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (na.range_c[r0 + mid] <= v) lo = mid; else hi = mid - 1;
+          }
+          s = a.range_s[r0 + lo].x + (v - na.range_c[r0 + lo]);
+        }
+        const float4 h = a.s_hi[s], l = a.s_lo[s];
+        rec = make_float4(df_diff(h.x, l.x, chi.x, clo.x), df_diff(h.y, l.y, chi.y, clo.y),
+                          df_diff(h.z, l.z, chi.z, clo.z), h.w);
+        S.idx[i] = a.perm[s];
+        load_row<CN>(na.rows, s, l.w, d);
+      }
+      S.rec[i] = rec;
+      // a sample of weight zero does not take part, whatever its values
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == t) num[k] = v;
+      for (int k = 0; k < CN; ++k) S.dat[i * CN + k] = rec.w != 0.f ? d[k] : 0.f;
     }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) npair += __shfl_xor_sync(0xffffffffu, npair, o);
-  if (lane == 0 && npair && a.pairs) atomicAdd(a.pairs, (unsigned long long)npair);
-  if (lane >= kNG) return;
-  const int64_t slot = slot0 + lane;
-  const uint32_t u = a.tgt_perm[slot];
-  if (u == 0xffffffffu) return;
-  // A non-finite channel value of a candidate outside the support reaches the
-  // target through 0 x NaN: such rows are computed again by the fix-up pass
-  // with only the pairs inside the support.
-  float chk = 0.f;
-#pragma unroll
-  for (int k = 0; k < CN; ++k) chk += num[k];
-  const bool bad = !isfinite(chk);
-  if (bad) {
-    atomicOr(&a.nf_bits[slot >> 5], 1u << (slot & 31));
-    atomicOr(a.nf_any, 1u);
-  }
-  if (a.out) {
-    const float W = wsum + wcor;
-    if (a.out_w) a.out_w[u] = W;
-    if (!bad) {
-#pragma unroll
-      for (int k = 0; k < CN; ++k)
-        if (k < a.C) a.out[(size_t)u * a.C + k] = (W > 0.f) ? num[k] / W : __int_as_float(0x7fc00000);
+  };
+
+  if (total <= kSpDirect) {
+    // ---- lanes over targets: no list, and no sum over lanes ----
+    stage(0);
+    __syncthreads();
+    const int64_t slot = tile * kTile + tid;
+    const float4 at = S.tv[tid];
+    Axes2 A{};
+    if (FORM != kWGauss1 && FORM != kWGauss1Ds && a.kd.type == CG_GAUSS2D) {
+      const float4 u = a.tgt_f1[slot], v = a.tgt_f2[slot];
+      A.ax = f2(u.x); A.ay = f2(u.y); A.az = f2(u.z);
+      A.bx = f2(v.x); A.by = f2(v.y); A.bz = f2(v.z);
     }
-    if (!a.keep) return;
-  }
-  const bool splits = a.n_split > 1;
-  if (!bad) {
-    float* dst = splits ? a.part_num + ((size_t)split * a.n_slots + slot) * a.C
-                        : a.acc_num + (size_t)slot * a.C;
-    const bool add = a.accumulate && !splits;
+    const WeightConst& kc = na.kc;
+    // four chains of additions: candidates 4 k, 4 k + 1, ... apart (short chains
+    // keep the digits that sums over lanes keep in the other forms)
+    float2 ws[2], wc[2], acc[2][CN];
 #pragma unroll
-    for (int k = 0; k < CN; ++k)
-      if (k < a.C) dst[k] = add ? dst[k] + num[k] : num[k];
-  }
-  if (splits) {
-    a.part_w[(size_t)split * a.n_slots + slot] = make_float2(wsum, wcor);
+    for (int h = 0; h < 2; ++h) {
+      ws[h] = wc[h] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < CN; ++c) acc[h][c] = make_float2(0.f, 0.f);
+    }
+    unsigned npair = 0;
+#pragma unroll 1
+    for (int k0 = 0; k0 < total; k0 += 4) {   // (padding follows the last one)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = k0 + 2 * h;
+        const float4 p = S.rec[k], q = S.rec[k + 1];
+        const float2 dx = __fadd2_rn(f2(at.x), make_float2(-p.x, -q.x));
+        const float2 dy = __fadd2_rn(f2(at.y), make_float2(-p.y, -q.y));
+        const float2 dz = __fadd2_rn(f2(at.z), make_float2(-p.z, -q.z));
+        const float2 c2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+        const float2 v = __fmul2_rn(weight2<FORM>(kc, a.kd, c2, dx, dy, dz, A), make_float2(p.w, q.w));
+        bool i0 = c2.x <= kc.c2_out, i1 = c2.y <= kc.c2_out;
+        if (band_near(kc, c2, INFINITY) <= kc.hw) {
+          // guard band: the cut is decided from the coordinates
+          const double2 tll = a.tgt_ll[slot];
+          if (i0 && c2.x >= a.kd.c2_in)
+            i0 = pair_inside(tll, a.sll[S.idx[k]], a.kd.c2r_hi, a.kd.c2r_lo, a.kd.c2r_tol, a.kd.r_rad);
+          if (i1 && c2.y >= a.kd.c2_in)
+            i1 = pair_inside(tll, a.sll[S.idx[k + 1]], a.kd.c2r_hi, a.kd.c2r_lo, a.kd.c2r_tol, a.kd.r_rad);
+        }
+        npair += (i0 ? 1u : 0u) + (i1 ? 1u : 0u);
+        const float2 w = make_float2(i0 ? v.x : -0.f, i1 ? v.y : -0.f);
+        kahan2(ws[h], wc[h], w);
+#pragma unroll
+        for (int c = 0; c < CN; ++c)
+          acc[h][c] = __ffma2_rn(w, make_float2(S.dat[k * CN + c], S.dat[(k + 1) * CN + c]), acc[h][c]);
+      }
+    }
+    float num[CN];
+#pragma unroll
+    for (int c = 0; c < CN; ++c) num[c] = (acc[0][c].x + acc[0][c].y) + (acc[1][c].x + acc[1][c].y);
+    comp_add(ws[0].x, wc[0].x, ws[0].y, wc[0].y);
+    comp_add(ws[1].x, wc[1].x, ws[1].y, wc[1].y);
+    comp_add(ws[0].x, wc[0].x, ws[1].x, wc[1].x);
+    npair = __reduce_add_sync(0xffffffffu, npair);
+    if (lane == 0 && npair && a.pairs) atomicAdd(a.pairs, (unsigned long long)npair);
+    write_target<CN>(a, slot, ws[0].x, wc[0].x, num, 0);
     return;
   }
-  float2 old = a.accumulate ? a.acc_w[slot] : make_float2(0.f, 0.f);
-  comp_add(old.x, old.y, wsum, wcor);
-  a.acc_w[slot] = old;
+
+  const int n_steps = (total + kSpStep - 1) / kSpStep;
+#pragma unroll 1
+  for (int q = 0; q < 4; ++q) {
+    const int group = 4 * warp + q;
+    const int64_t slot0 = tile * kTile + group * kNG;
+    const float4 near = group_reach(S.tv[group * kNG + (lane & 7)], a.kd.c2_out);
+    const uint32_t pair_s = (uint32_t)__cvta_generic_to_shared(&S.pair[group][0][0]);
+    LaneSums<CN> L;
+    L.clear();
+    for (int step = 0; step < n_steps; ++step) {
+      if (q == 0 || n_steps > 1) {
+        __syncthreads();   // everyone is done with what was staged before
+        stage(step * kSpStep);
+        __syncthreads();
+      }
+      const int cnt = list_near(S.rec, min(kSpStep, total - step * kSpStep), near, S.list[warp]);
+      add_listed<CN, FORM>(na, L, S.list[warp], cnt, S.rec, S.dat, S.idx, pair_s, S.tv + group * kNG, slot0);
+      __syncwarp();        // the warp's list is rewritten
+    }
+    write_group(na, L, slot0, 0);
+  }
 }
 
 // Channel rows in sorted order, padded to CN channels (BF16 values as FP32).
@@ -429,11 +677,15 @@ cudaError_t launch_narrow(const NarrowArgs& na, int64_t n_tiles, int64_t n, int 
     k_rows_sorted<float, CN><<<ceil_div(n, 256), 256, 0, s>>>(
         static_cast<const float*>(na.g.data), na.g.perm, n, na.g.C, rows);
   const dim3 grid((unsigned)n_tiles, 1, (unsigned)na.g.n_split);
+  auto go = [&](auto dense, auto sparse) {
+    if (na.sparse) sparse<<<(unsigned)n_tiles, kSpTh, 0, s>>>(na);
+    else dense<<<grid, kNTh, 0, s>>>(na);
+  };
   switch (weight_form(na.g.kd)) {
-    case kWGauss1: k_grid_narrow<CN, kWGauss1><<<grid, kNTh, 0, s>>>(na); break;
-    case kWGauss2: k_grid_narrow<CN, kWGauss2><<<grid, kNTh, 0, s>>>(na); break;
-    case kWGauss1Ds: k_grid_narrow<CN, kWGauss1Ds><<<grid, kNTh, 0, s>>>(na); break;
-    default: k_grid_narrow<CN, kWAny><<<grid, kNTh, 0, s>>>(na); break;
+    case kWGauss1: go(k_grid_narrow<CN, kWGauss1>, k_grid_sparse<CN, kWGauss1>); break;
+    case kWGauss2: go(k_grid_narrow<CN, kWGauss2>, k_grid_sparse<CN, kWGauss2>); break;
+    case kWGauss1Ds: go(k_grid_narrow<CN, kWGauss1Ds>, k_grid_sparse<CN, kWGauss1Ds>); break;
+    default: go(k_grid_narrow<CN, kWAny>, k_grid_sparse<CN, kWAny>); break;
   }
   return cudaGetLastError();
 }
@@ -451,12 +703,26 @@ int narrow_splits(int64_t n_tiles, int64_t n, int n_sms) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(64, std::min(want, most)));
 }
 
-cudaError_t grid_narrow(const GridArgs& a, const Tiling& t, int64_t n, int dtype, float* rows,
+// Where k_grid_sparse is the faster form: few samples per tile (a tile sees two to
+// four times those), and the more tiles the more, because the dense form's CTAs
+// are few per SM.  Measured on GB300, sparse / dense, one channel: 32,768 tiles 12
+// samples each 0.58, 25 0.84, 32 0.99, 40 1.08; 2048 tiles 8 0.84, 18 0.95, 25
+// 1.05; seven channels: 32,768 tiles 28 0.80, 36 0.91, 48 0.98; 3633 tiles 20 0.86,
+// 28 0.97, 36 1.04.  Around one tile per SM a tile's own latency counts, which is
+// shorter with eight warps (156 tiles, 13 samples each: 1.12).
+bool sparse_tiles(int64_t n_tiles, int64_t n, int C, int n_sms) {
+  if (2 * n_tiles < 3 * n_sms) return false;
+  const int most = n_tiles < 20 * n_sms ? 16 : (n_tiles < 60 * n_sms ? 26 : (C <= 2 ? 30 : 44));
+  return n < most * n_tiles;
+}
+
+cudaError_t grid_narrow(const GridArgs& a, const Tiling& t, int64_t n, int dtype, float* rows, int n_sms,
                         cudaStream_t s) {
   NarrowArgs na;
   na.g = a;
   na.range_c = t.range_c;
   na.rows = rows;
+  na.sparse = a.n_split == 1 && sparse_tiles(t.n_tiles, n, a.C, n_sms);
   na.kc = weight_const(a.kd);
   switch (narrow_width(a.C)) {
     case 1: return launch_narrow<1>(na, t.n_tiles, n, dtype, rows, s);
