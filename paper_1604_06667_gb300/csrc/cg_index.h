@@ -22,10 +22,12 @@ CG_HD int wide_shares(int total, int n_split) {
 }
 
 // Chunks of kc candidates between two folds of the wide form's sums: a tile's
-// `total` candidates in n_fold parts, of at least two chunks.
+// `total` candidates in up to n_fold parts, of at least two chunks each (one part:
+// never).
 CG_HD int wide_fold_chunks(int total, int n_fold, int kc) {
-  const int64_t part = (int64_t)n_fold * kc, k = (total + part - 1) / part;
-  return k < 2 ? 2 : (int)k;
+  const int chunks = total / kc + (total % kc ? 1 : 0);
+  const int parts = chunks / 2 < n_fold ? chunks / 2 : n_fold;
+  return parts < 2 ? 1 << 30 : (chunks + parts - 1) / parts;
 }
 
 // Partial sums of a slot: the shares of its tile, 0 for an empty slot.  Slots

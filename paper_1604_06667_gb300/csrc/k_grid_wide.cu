@@ -315,22 +315,54 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
   const int pitch = wa.rows_mode == kRowsTma ? wa.box_cols : CPAD;
 
   float2 acc[T][CL / 2];
-  // FOLD: the sums of the parts before; above 8 in local memory, because in
+  // FOLD: the sums of the parts before; above 8 of them in local memory, because in
   // registers they push out what the sums in hand need (scans of 37 channels 1.27
-  // against 1.21 ms)
+  // against 1.21 ms), and so does an address kept for them (95,000 x 256: 270 against
+  // 256 us)
   constexpr bool IN_REGS = T * CL <= 8;
-  float2 part[FOLD ? T * CL / 2 : 1];
-  float2* tot = part;
-  if constexpr (FOLD && !IN_REGS) asm volatile("" : "+l"(tot) : : "memory");
+  float2 tot[T][CL / 2];
+  float4 part[T * CL / 4];
   float ws = 0.f, wc = 0.f;
 #pragma unroll
   for (int i = 0; i < T; ++i)
 #pragma unroll
     for (int j = 0; j < CL / 2; ++j) {
       acc[i][j] = make_float2(0.f, 0.f);
-      if (FOLD && IN_REGS) part[i * (CL / 2) + j] = make_float2(0.f, 0.f);
+      if constexpr (FOLD && IN_REGS) tot[i][j] = make_float2(0.f, 0.f);
     }
-  int fold_at = FOLD ? wide_fold_chunks(total, a.n_fold, KC) : 0, folds = 0;
+  int fold_at = FOLD ? wide_fold_chunks(total, a.n_fold, KC) : 0;
+  // acc += the parts before (add: there are any); keep: to be the parts before, with
+  // acc cleared
+  auto fold = [&](bool add, bool keep) {
+    if constexpr (IN_REGS) {
+#pragma unroll
+      for (int i = 0; i < T; ++i)
+#pragma unroll
+        for (int j = 0; j < CL / 2; ++j) {
+          const float2 t = __fadd2_rn(tot[i][j], acc[i][j]);
+          if (keep) tot[i][j] = t;
+          acc[i][j] = keep ? make_float2(0.f, 0.f) : t;
+        }
+    } else {
+      float4* mem = part;
+      asm volatile("" : "+l"(mem) : : "memory");   // (stays in memory)
+#pragma unroll
+      for (int i = 0; i < T; ++i)
+#pragma unroll
+        for (int j = 0; j < CL / 2; j += 2) {
+          float4& m = mem[(i * CL + 2 * j) / 4];
+          float2 t0 = acc[i][j], t1 = acc[i][j + 1];
+          if (add) {
+            const float4 v = m;
+            t0 = __fadd2_rn(make_float2(v.x, v.y), t0);
+            t1 = __fadd2_rn(make_float2(v.z, v.w), t1);
+          }
+          if (keep) m = make_float4(t0.x, t0.y, t1.x, t1.y);
+          acc[i][j] = keep ? make_float2(0.f, 0.f) : t0;
+          acc[i][j + 1] = keep ? make_float2(0.f, 0.f) : t1;
+        }
+    }
+  };
   unsigned npair = 0;
 
   bool ok = true;
@@ -458,26 +490,14 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
     if (lane == 0) mbar_arrive(&S.empty[st]);
     if constexpr (FOLD) {
       if (q + 1 == fold_at) {
-        fold_at += wide_fold_chunks(total, a.n_fold, KC);
-#pragma unroll
-        for (int i = 0; i < T; ++i)
-#pragma unroll
-          for (int j = 0; j < CL / 2; ++j) {
-            float2& t = tot[i * (CL / 2) + j];
-            t = IN_REGS || folds ? __fadd2_rn(t, acc[i][j]) : acc[i][j];
-            acc[i][j] = make_float2(0.f, 0.f);
-          }
-        ++folds;
+        const int every = wide_fold_chunks(total, a.n_fold, KC);
+        fold(fold_at > every, true);
+        fold_at += every;
       }
     }
   }
   if constexpr (FOLD) {
-    if (IN_REGS || folds) {
-#pragma unroll
-      for (int i = 0; i < T; ++i)
-#pragma unroll
-        for (int j = 0; j < CL / 2; ++j) acc[i][j] = __fadd2_rn(tot[i * (CL / 2) + j], acc[i][j]);
-    }
+    if (IN_REGS || fold_at != wide_fold_chunks(total, a.n_fold, KC)) fold(true, false);
   }
 
   // ---- W: lane l holds a part of target l % G's sum ----

@@ -87,16 +87,16 @@ int main() {
 
 
 def test_folds_keep_chains_short(tmp_path):
-    """Parts of a tile's candidates that are summed apart: no longer than a share
-    of n_fold equal ones rounded up to chunks (or two chunks), for any total."""
+    """Parts of a tile's candidates that are summed apart: at least two chunks, and
+    no longer than n_fold equal ones, or than three chunks, whatever the total."""
     _run(tmp_path, r"""
 int main() {
-  for (int total : {0, 1, 63, 64, 65, 200, 1000, 4097, 1 << 20, 2147483647})
-    for (int n : {2, 3, 29, 64}) {
-      const int64_t k = cg::wide_fold_chunks(total, n, 32);
+  for (int total : {0, 1, 63, 64, 65, 96, 97, 128, 200, 1000, 4097, 1 << 20, 2147483647})
+    for (int n : {1, 2, 3, 29, 64}) {
+      const int64_t k = cg::wide_fold_chunks(total, n, 32), chunks = ((int64_t)total + 31) / 32;
       CHECK(k >= 2);
-      CHECK(k * 32 * n >= total);
-      CHECK(k == 2 || (k - 1) * 32 * n < total);
+      if (n == 1 || chunks < 4) CHECK(k >= chunks);
+      else CHECK(k <= 3 || (k - 1) * n < chunks);
     }
 }
 """)
