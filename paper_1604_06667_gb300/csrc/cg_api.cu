@@ -219,12 +219,13 @@ cg_status do_add(cg_grid* g, const double* lon, const double* lat, const void* d
   CG_CUDA(cudaSetDevice(g->device), where);
   Tiling& t = tc ? g->t128 : g->t64;
   cudaEvent_t t0 = tmark(g);
+  bool rec_values = false;
   if (!reuse) {
     g->index_valid = false;
     // a single channel's values travel with the records when they are there
     // already (host-buffer calls still copy them) and the FP32 form reads them
-    g->rec_values = g->C == 1 && !tc && g->f32_cfg < 0 && !g->data_ready;
-    CG_CUDA(samples_keys(g, lon, lat, weights, n, g->rec_values ? data : nullptr, dtype), where);
+    rec_values = g->C == 1 && !tc && g->f32_cfg < 0 && !g->data_ready;
+    CG_CUDA(samples_keys(g, lon, lat, weights, n, rec_values ? data : nullptr, dtype), where);
   }
   cudaEvent_t t1 = tmark(g);
   if (!reuse) CG_CUDA(samples_sort(g, n), where);
@@ -251,6 +252,7 @@ cg_status do_add(cg_grid* g, const double* lon, const double* lat, const void* d
     // one-shot calls: the gridder writes R = N / W itself where it can
     const bool want = out != nullptr && g->acc_empty;
     bool direct = false;
+    g->rec_values = rec_values;
     const cudaError_t eg = grid_tiles_f32(g, data, dtype, want ? out : nullptr,
                                           want ? out_w : nullptr, &direct, &kept);
     g->rec_values = false;   // later passes bring values of their own
