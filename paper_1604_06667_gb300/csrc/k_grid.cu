@@ -862,7 +862,8 @@ cudaError_t run_wide(cg_grid* g, GridArgs& a, int dtype, bool* direct, bool* kep
   // x 128 of flags onto 178 x 178 1.5e-7 (1.0e-7, 1.1e-7); the folds cost 0 to 7 %
   // of a call.
   const int blocked = blocked_splits(nt, a.C, sm_count());
-  a.n_fold = blocked >= a.n_split ? blocked : 1;
+  const bool few = 2 * g->last_n < 384 * (int64_t)blocked * nt;   // (shares of 256: wide_shares)
+  a.n_fold = blocked > a.n_split || (blocked == a.n_split && few) ? blocked : 1;
   cudaError_t e = begin_pass(g, a, n_slabs, direct, kept);
   if (e == cudaSuccess) e = grid_wide(a, g->t64, g->last_n, dtype, g->stream);
   if (e != cudaSuccess) return e;

@@ -177,18 +177,18 @@ struct LaneSums {
   }
 };
 
-// The warp's list of the first n candidates (32 at a time) in reach of its group;
-// their number.
-__device__ __forceinline__ int list_near(const float4* rec, int n, float4 g, uint16_t* list) {
+// The warp's list of the first 32 B candidates in reach of its group; their number.
+template <int B>
+__device__ __forceinline__ int list_near(const float4* rec, float4 g, uint16_t* list) {
   const int lane = threadIdx.x & 31;
   int cnt = 0;
-#pragma unroll 8
-  for (int b = 0; b < n; b += 32) {
-    const float4 p = rec[b + lane];
+#pragma unroll
+  for (int b = 0; b < B; ++b) {
+    const float4 p = rec[32 * b + lane];
     const float ex = p.x - g.x, ey = p.y - g.y, ez = p.z - g.z;
     const bool in = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= g.w;
     const uint32_t m = __ballot_sync(0xffffffffu, in);
-    if (in) list[cnt + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(b + lane);
+    if (in) list[cnt + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(32 * b + lane);
     cnt += __popc(m);
   }
   __syncwarp();
@@ -465,7 +465,9 @@ __global__ void __launch_bounds__(kNTh, CN <= 2 ? 3 : 2)
         put(pre, st ^ 1);
         if (q + 2 < n_steps) pre = fetch(v_lo + (q + 2) * kNTh);
       }
-      const int cnt = list_near(S.rec[st], min(kNTh, v_hi - v_lo - q * kNTh), near, S.list[warp]);
+      // (a step's loads and ballots at once; a nearly empty last one apart)
+      const int cnt = v_hi - v_lo - q * kNTh > kNTh / 4 ? list_near<kNTh / 32>(S.rec[st], near, S.list[warp])
+                                                        : list_near<kNTh / 128>(S.rec[st], near, S.list[warp]);
       add_listed<CN, FORM>(na, L, S.list[warp], cnt, S.rec[st], S.dat[st], S.idx[st], pair_s, S.tv + warp * kNG, slot0);
       __syncthreads();   // the stage may be rewritten; the next one is visible
     }
@@ -635,7 +637,7 @@ __global__ void __launch_bounds__(kSpTh, CN <= 2 ? 12 : 8) k_grid_sparse(const _
         stage(step * kSpStep);
         __syncthreads();
       }
-      const int cnt = list_near(S.rec, min(kSpStep, total - step * kSpStep), near, S.list[warp]);
+      const int cnt = list_near<kSpStep / 32>(S.rec, near, S.list[warp]);
       add_listed<CN, FORM>(na, L, S.list[warp], cnt, S.rec, S.dat, S.idx, pair_s, S.tv + group * kNG, slot0);
       __syncwarp();        // the warp's list is rewritten
     }
