@@ -99,9 +99,6 @@ cg_status build_plan(cg_batch* b) {
   b->plan = p;
   cudaStream_t s = b->own;
   const int nj = (int)b->jobs.size();
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   // ---- the shared sample index ----
   std::vector<int64_t> samp_off(1, 0), key_blk(1, 0), gth_blk(1, 0), tile_off(1, 0);
   uint64_t key_base = 0;

@@ -17,11 +17,12 @@
 //            warp's shared memory, rows straight from L2.
 //
 // The map's rows come in the index's order, times 1 / W (k_adjoint_rows).
-// Bound by instruction issue (56 % of the slots) and by the latency of the
-// searches.  Measured on GB300 against one warp per 32 samples with the targets
-// one after another (k_degrid.cu, which stays for the elliptical kernel and for
-// maps with non-finite values): 1e6 samples, one channel 3.6 -> 0.7 ms; 2e5
-// samples, 64 channels 3.8 -> 0.42 ms; 16 channels 1.9 -> 0.36 ms.  A form with
+// Bound by instruction issue (57 % of the slots with one channel, 47 % with 64)
+// and by the latency of the searches.  Measured on GB300 against one warp per 32
+// samples with the targets one after another (k_degrid.cu, which stays for the
+// elliptical kernel and for maps with non-finite or out-of-range values): 1e6
+// samples, one channel 3.6 -> 0.7 ms; 2e5 samples, 64 channels 3.8 -> 0.41 ms; 16
+// channels 1.9 -> 0.36 ms.  A form with
 // tiles of 64 samples, targets staged for 8 warps and listed by each, took
 // 0.75 ms for the first and 1.9 ms for the second: a third of the staged
 // targets was in reach of a warp.

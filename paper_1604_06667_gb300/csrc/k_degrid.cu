@@ -402,7 +402,7 @@ cudaError_t grid_degrid(cg_grid* g, const float* y, const float* wmap, float* ou
   a.dirty = nullptr;
   if (a.n == 0) return cudaGetLastError();
   if (g->kernel_type != CG_GAUSS2D) {
-    // circular kernels: the tiled gather; the general kernel below then only
+    // circular kernels: k_adjoint.cu; the general kernel below then only
     // runs where the map holds non-finite or out-of-range values
     AdjointArgs t;
     t.ns = g->nside;

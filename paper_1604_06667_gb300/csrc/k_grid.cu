@@ -920,7 +920,7 @@ cudaError_t grid_tiles_f32_to(cg_grid* g, const void* data, int dtype, float* ac
   a.n_fold = 1;
   int cfg = g->f32_cfg;
   if (cfg < 0 || cfg >= kF32Configs || C != g->C) {
-    // the register-blocked shapes stay for shapes asked for and fused batches
+    // the register-blocked shapes stay for shapes asked for (by a caller or the autotuner)
     return C <= kNarrowMaxC ? run_narrow(g, a, dtype, direct, kept)
                             : run_wide(g, a, dtype, direct, kept);
   }

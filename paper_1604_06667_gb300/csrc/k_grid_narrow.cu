@@ -19,14 +19,17 @@
 //   weights  8 targets as 4 packed f32x2 pairs per lane: chord, kernel value,
 //            cut (guard band decided from the coordinates), weight sums
 //            (Kahan) and channel sums;
-//   end      the lanes' sums are added up by shuffles (compensated for W).
+//   end      the lanes' sums meet by shuffles that halve the targets a lane holds
+//            at every step (compensated for W).
+// Maps of few samples per tile run k_grid_sparse, below.
 //
-// Bound by issue slots and by the barrier per step (58 % of the issue slots
-// used, ALU pipe 46 %).  Measured on GB300 against the register-blocked form
-// it replaced (one target per thread, weights through shared memory, every
-// candidate of the tile evaluated): 1e8 samples onto 8,100 targets 36.6 ->
-// 8.3 ms, 1e6 samples onto 512 x 512 targets 0.95 -> 0.33 ms, 1.2e7 samples on
-// the sphere onto 786,432 targets 4.48 -> 1.37 ms; the sums of 32 lanes are
+// Bound by the barrier per step and by issue slots (1e7 samples onto 8,100
+// targets: 48 % of the issue slots used, the barrier the largest stall, ALU pipe
+// 32 %).  Measured on GB300 against the register-blocked form it replaced (one
+// target per thread, weights through shared memory, every candidate of the tile
+// evaluated): 1e8 samples onto 8,100 targets 36.6 -> 8.0 ms, 1e6 samples onto
+// 512 x 512 targets 0.95 -> 0.32 ms, 1.2e7 samples on the sphere onto 786,432
+// targets 4.48 -> 1.29 ms; the sums of 32 lanes are
 // also ten times more accurate than one long one.  The bounds of 3 CTAs per
 // SM (2 above two channels, where the sums take the registers) measured best:
 // 17.91 ms per call of 1e8 samples against 18.44 (2) and 18.02 (4).  One

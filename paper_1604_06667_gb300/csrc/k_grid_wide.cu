@@ -22,11 +22,12 @@
 // per 8 to 16 targets keeps 50-65 % of the executed FMAs inside the support.
 //
 // Measured on GB300 against the register-blocked form (k_grid.cu), per call:
-// 1e6 samples x 256 channels onto 512 x 512 targets 6.55 -> 3.78 ms, 1e7 x 32
-// on the sphere, elliptical, onto 4096 x 2048 20.0 -> 10.9 ms, 2.5e5 x 256 onto
-// 256 x 256 2.12 -> 1.26 ms, eight scans of 25,000 x 37 2.70 -> 1.20 ms.  Of
-// the cube's 4.0 ms of gridder 2.5 are channel sums (FMA pipe ~90 % while they
-// run), 1.4 staging, lists and weights.  What it took: no spilled sums (with
+// 1e6 samples x 256 channels onto 512 x 512 targets 6.55 -> 3.73 ms, 1e7 x 32
+// on the sphere, elliptical, onto 4096 x 2048 20.0 -> 10.95 ms, 2.5e5 x 256 onto
+// 256 x 256 2.12 -> 1.24 ms, eight scans of 25,000 x 37 2.70 -> 1.20 ms.  On the
+// cube the FMA pipe is busy 61 % of the time and 54 % of the issue slots are used
+// (32 channels: 54 % and 69 %); with the sums taken out a third of the time was
+// left, for staging, lists and weights.  What it took: no spilled sums (with
 // two CTAs per SM the stages leave no L1 for them: a ninth, producing warp and
 // 96 registers cost 0.9 ms), candidates of every chunk from all over the
 // tile's reach (0.2 ms), records staged two chunks before their rows, targets
