@@ -316,11 +316,10 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
   const int pitch = wa.rows_mode == kRowsTma ? wa.box_cols : CPAD;
 
   float2 acc[T][CL / 2];
-  // FOLD: the sums of the parts before; above 8 of them in local memory, because in
-  // registers they push out what the sums in hand need (scans of 37 channels 1.27
-  // against 1.21 ms), and so does an address kept for them (95,000 x 256: 270 against
-  // 256 us)
-  constexpr bool IN_REGS = T * CL <= 8;
+  // FOLD: the sums of the parts before, in registers or (128 channels and more, no
+  // room) in local memory; an address kept for them would take registers too
+  // (95,000 x 256 270 against 256 us)
+  constexpr bool IN_REGS = CPAD <= 64;
   float2 tot[T][CL / 2];
   float4 part[T * CL / 4];
   float ws = 0.f, wc = 0.f;
@@ -592,13 +591,17 @@ cudaError_t launch_wide(const WideArgs& wa, const CUtensorMap& tmap, int64_t n_t
     k<<<grid, SH::NTH, smem, s>>>(tmap, wa);
     return cudaGetLastError();
   };
+  // the folding variant keeps its second set of sums in registers where one CTA
+  // less per SM makes room for them (2e5 x 16 onto 256 x 256 266 -> 257 us, x 32
+  // 292 -> 282); from 128 channels on it would halve the warps
+  constexpr int FB = SH::CPAD <= 64 ? MINB - 1 : MINB;
   const bool fold = wa.g.n_fold > 1;
   switch (weight_form(wa.g.kd)) {
-    case kWGauss1: return fold ? go(k_grid_wide<SH, kWGauss1, MINB, true>) : go(k_grid_wide<SH, kWGauss1, MINB, false>);
-    case kWGauss2: return fold ? go(k_grid_wide<SH, kWGauss2, MINB, true>) : go(k_grid_wide<SH, kWGauss2, MINB, false>);
+    case kWGauss1: return fold ? go(k_grid_wide<SH, kWGauss1, FB, true>) : go(k_grid_wide<SH, kWGauss1, MINB, false>);
+    case kWGauss2: return fold ? go(k_grid_wide<SH, kWGauss2, FB, true>) : go(k_grid_wide<SH, kWGauss2, MINB, false>);
     case kWGauss1Ds:
-      return fold ? go(k_grid_wide<SH, kWGauss1Ds, MINB, true>) : go(k_grid_wide<SH, kWGauss1Ds, MINB, false>);
-    default: return fold ? go(k_grid_wide<SH, kWAny, MINB, true>) : go(k_grid_wide<SH, kWAny, MINB, false>);
+      return fold ? go(k_grid_wide<SH, kWGauss1Ds, FB, true>) : go(k_grid_wide<SH, kWGauss1Ds, MINB, false>);
+    default: return fold ? go(k_grid_wide<SH, kWAny, FB, true>) : go(k_grid_wide<SH, kWAny, MINB, false>);
   }
 }
 
