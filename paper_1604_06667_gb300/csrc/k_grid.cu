@@ -859,8 +859,8 @@ cudaError_t run_wide(cg_grid* g, GridArgs& a, int dtype, bool* direct, bool* kep
   // further (its tiles of few candidates too), the sums are folded as often:
   // chains of additions no longer than its own.  With one chain per tile 2e5 x 16
   // onto 256 x 256 had an error of 2.9e-7 (1.8e-7 now, 2.3e-7 in that form), 7,900
-  // x 128 of flags onto 178 x 178 1.5e-7 (1.0e-7, 1.1e-7); the folds cost 2 to 8 %
-  // of a call from 128 channels on.
+  // x 128 of flags onto 178 x 178 1.5e-7 (1.0e-7, 1.1e-7); the folds cost 0 to 4 %
+  // of a call up to 64 channels and 2 to 8 % above.
   const int blocked = blocked_splits(nt, a.C, sm_count());
   const bool few = 2 * g->last_n < 384 * (int64_t)blocked * nt;   // (shares of 256: wide_shares)
   a.n_fold = blocked > a.n_split || (blocked == a.n_split && few) ? blocked : 1;

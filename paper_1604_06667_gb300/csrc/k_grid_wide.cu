@@ -316,10 +316,10 @@ __global__ void __launch_bounds__(SH::NTH, MINB)
   const int pitch = wa.rows_mode == kRowsTma ? wa.box_cols : CPAD;
 
   float2 acc[T][CL / 2];
-  // FOLD: the sums of the parts before, in registers or (128 channels and more, no
+  // FOLD: the sums of the parts before, in registers or (64 channels and more, no
   // room) in local memory; an address kept for them would take registers too
   // (95,000 x 256 270 against 256 us)
-  constexpr bool IN_REGS = CPAD <= 64;
+  constexpr bool IN_REGS = CPAD <= 32;
   float2 tot[T][CL / 2];
   float4 part[T * CL / 4];
   float ws = 0.f, wc = 0.f;
@@ -593,8 +593,9 @@ cudaError_t launch_wide(const WideArgs& wa, const CUtensorMap& tmap, int64_t n_t
   };
   // the folding variant keeps its second set of sums in registers where one CTA
   // less per SM makes room for them (2e5 x 16 onto 256 x 256 266 -> 257 us, x 32
-  // 292 -> 282); from 128 channels on it would halve the warps
-  constexpr int FB = SH::CPAD <= 64 ? MINB - 1 : MINB;
+  // 292 -> 282) and still holds the four that wide_splits fills; 64 channels would
+  // be left with three (73,000 x 48 onto 128 x 128 239 us), more with half the warps
+  constexpr int FB = SH::CPAD <= 32 ? MINB - 1 : MINB;
   const bool fold = wa.g.n_fold > 1;
   switch (weight_form(wa.g.kd)) {
     case kWGauss1: return fold ? go(k_grid_wide<SH, kWGauss1, FB, true>) : go(k_grid_wide<SH, kWGauss1, MINB, false>);
